@@ -85,3 +85,21 @@ def test_noise_full_size_sampled(api):
     assert np.abs(sample - c * ref).max() < 3e-7
     del out
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("Nx,Ny,Nz,kw", [
+    (11, 11, 4, {}),                        # two points per sum, smallest grid
+    (12, 12, 5, {}),                        # four points per sum, smallest grid
+    (14, 9 + 8, 5, {"kperp2_max": 10.0}),   # Nx even, not a multiple of four; a short last row group
+    (128, 13, 9, {}),
+    (516, 12, 3, {}),                       # more points than threads
+    (204, 203, 3, {"kperp2_min": 9999.0, "kperp2_max": 10001.0, "m_min": 1, "m_max": 1}),   # fewer rows per block
+])
+def test_noise_folded_rows_match_oracle(api, Nx, Ny, Nz, kw):
+    """The folded row sums in both arithmetics, one value at a time."""
+    out64, draws = _run(api, Nx, Ny, Nz, torch.float64, 17, **kw)
+    out32, _ = _run(api, Nx, Ny, Nz, torch.float32, 17, **kw)
+    ref = _oracle(Nx, Ny, Nz, draws, **kw)
+    assert np.abs(out64 - ref).max() < 1e-13
+    # one float32 rounding of values <= 1; the pairs' own error is below 1e-12
+    assert np.abs(out32 - ref).max() <= 2.0 ** -24 + 1e-12
