@@ -96,6 +96,28 @@ fc_status injected(const char* entry) {
   return out;
 }
 
+// Which float32 calls take the dense operators instead of the transforms.  A
+// tile of 128 lines passes through one SM in 6 us (N' = 75) to 45 us (538), so
+// a call needs a wave of tiles (152 x 128 lines) or more, and the gain depends
+// on how far the transform length lies above N'.  Measured, dense against
+// transform (us):
+//   padded, N' >= 180   257 x 16k lines 35 / 39, 513 x 16k 51 / 64, 513 x 41k
+//                       131 / 152, 400 x 82k 180 / 351, 513 x 400k 886 / 1520;
+//                       8k lines: 33 / 22 and 46 / 31, so from 16384 lines on
+//   padded, N' >= 75    50 x 164k 96 / 106, 65 x 164k 100 / 121, 129 x 164k
+//                       141 / 170; 65 x 82k 59 / 57: from 131072 lines on
+//   direct, N' >= 200   (the transform has length N') 487 x 82k 206 / 236, 231 x
+//                       164k 207 / 225; 487 x 41k 125 / 127: from 98304 lines on
+//   direct, shorter     103 x 400k 275 / 299, 39 x 400k 220 / 121: transforms
+static long long dense_min_lines(const PlanData& p) {
+  const long long never = 1LL << 62;
+  if (p.dense_direct) return p.Np >= 200 ? 98304 : never;
+  return p.Np >= 180 ? 16384 : (p.Np >= 75 ? 131072 : never);
+}
+bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines) {
+  return dtype == FC_F32 && p.dense.NQ && lines >= dense_min_lines(p);
+}
+
 }  // namespace fcns
 
 using namespace fcns;
@@ -187,6 +209,15 @@ fc_status fc_setup_ex(int d, int C, int Nz, int M, int n_os, fc_plan_t* out) {
     const float hi = (float)p->data.Mr[i];
     p->deriv.Mr2[i] = make_float2(hi, (float)(p->data.Mr[i] - (double)hi));
   }
+  p->data.dense_direct = L == p->data.Np;
+  if (L > 0 && dense_min_lines(p->data) < (1LL << 31) && dense_geom(Nz, p->data.Np, &p->data.dense)) {
+    std::vector<double> c1, c2;
+    deriv_kernels_closed(p->data.Np, &c1, &c2);
+    p->data.dense_exp[0] = dense_blocks(p->data.dense, c1, &p->data.dense_blocks);
+    p->data.dense_exp[1] = dense_blocks(p->data.dense, c2, &p->data.dense_blocks);
+  } else {
+    p->data.dense = DenseGeom();
+  }
   *out = p;
   return FC_OK;
 }
@@ -221,6 +252,8 @@ fc_status fc_destroy(fc_plan_t plan) {
       cudaDeviceSynchronize();
       cudaFree(t.Mr); cudaFree(t.Mr2); cudaFree(t.tw32); cudaFree(t.tw64);
       cudaFree(t.H1_32); cudaFree(t.H1_64); cudaFree(t.H2_32); cudaFree(t.H2_64);
+      cudaFree(t.dense);
+      if (t.dense_err) cudaFreeHost(t.dense_err);
       for (auto& slot : t.stage)
         for (void* b : slot) cudaFree(b);
       for (int k = 0; k < 3; ++k) {
@@ -282,9 +315,16 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
   if (!s) s = up(plan->deriv.H2_64.data(), 16 * L, &t.H2_64);
   if (!s) s = upload<float2>(plan->deriv.tw, &t.tw32);
   if (!s) s = upload<double2>(plan->deriv.tw, &t.tw64);
+  if (!s && plan->data.dense.NQ) {
+    s = up(plan->data.dense_blocks.data(), 2 * plan->data.dense_blocks.size(), &t.dense);
+    if (!s) s = cuda_status(cudaHostAlloc((void**)&t.dense_err, sizeof(unsigned), cudaHostAllocDefault), "cudaHostAlloc");
+    if (!s) *t.dense_err = 0;
+  }
   if (s) {
     cudaFree(t.Mr); cudaFree(t.Mr2); cudaFree(t.tw32); cudaFree(t.tw64);
       cudaFree(t.H1_32); cudaFree(t.H1_64); cudaFree(t.H2_32); cudaFree(t.H2_64);
+      cudaFree(t.dense);
+      if (t.dense_err) cudaFreeHost(t.dense_err);
     return s;
   }
   plan->data.dev.push_back(t);
@@ -327,6 +367,8 @@ extern "C" fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int N
     s = deriv_tables_locked(plan, &t);
   }
   if (s) return s;
+  if (deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch))
+    return launch_deriv_dense(*t, plan->data, batch, (long long)Nx * Ny, Lz, f, df, d2f, (cudaStream_t)stream);
   return launch_deriv_z(*t, plan->data, dtype, batch, (long long)Nx * Ny, Lz, f, df, d2f, (cudaStream_t)stream);
 }
 
@@ -393,6 +435,8 @@ extern "C" fc_status fc_deriv_z_host_ex(fc_plan_t plan, fc_dtype dtype, int batc
   const char* fh = static_cast<const char*>(f);
   char* oh[2] = {static_cast<char*>(df), static_cast<char*>(d2f)};
   const size_t hp = (size_t)Ny * Nx * es;     // host pitch between z rows
+  // the whole call picks the kernel, so that the slabs give what one call on device arrays gives
+  const bool dense = deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch);
   long long i = 0;
   for (size_t si = 0; si < slabs.size() && !s; ++si, ++i) {
     {  // slab si in staging slot i % 3
@@ -405,8 +449,9 @@ extern "C" fc_status fc_deriv_z_host_ex(fc_plan_t plan, fc_dtype dtype, int batc
                               "cudaMemcpy2DAsync(H2D)");
       if (!s) s = cuda_status(cudaEventRecord(t->ev_in[k], t->st_in), "cudaEventRecord");
       if (!s) s = cuda_status(cudaStreamWaitEvent(t->st_run, t->ev_in[k], 0), "cudaStreamWaitEvent");
-      if (!s) s = launch_deriv_z(*t, plan->data, dtype, 1, (long long)Nx * yc, Lz, t->stage[k][0],
-                                 df ? t->stage[k][1] : nullptr, d2f ? t->stage[k][2] : nullptr, t->st_run);
+      void *o1 = df ? t->stage[k][1] : nullptr, *o2 = d2f ? t->stage[k][2] : nullptr;
+      if (!s) s = dense ? launch_deriv_dense(*t, plan->data, 1, (long long)Nx * yc, Lz, t->stage[k][0], o1, o2, t->st_run)
+                        : launch_deriv_z(*t, plan->data, dtype, 1, (long long)Nx * yc, Lz, t->stage[k][0], o1, o2, t->st_run);
       if (!s) s = cuda_status(cudaEventRecord(t->ev_run[k], t->st_run), "cudaEventRecord");
       if (!s) s = cuda_status(cudaStreamWaitEvent(t->st_out, t->ev_run[k], 0), "cudaStreamWaitEvent");
       for (int o = 0; o < 2 && !s; ++o)

@@ -10,6 +10,9 @@
 // matrix is M_r = A_r Q_r^T (App. B, eq. Af).
 #include "host_tables.hpp"
 
+#include <cuda_fp16.h>
+
+
 #include <cmath>
 #include <map>
 #include <mutex>
@@ -572,6 +575,84 @@ void engine_twiddles(int L1, int L2, std::vector<std::complex<double>>* tw) {
       (*tw)[n2 * L1 + k1] = w;          // read by the k1-threads (B side)
       (*tw)[L + k1 * L2 + n2] = w;      // read by the n2-threads (A side)
     }
+}
+
+void deriv_kernels_closed(int Np, std::vector<double>* d1, std::vector<double>* d2) {
+  // sums over the modes of i k e^{ikj} / N' and -k^2 e^{ikj} / N', k = 2 pi l / N'
+  const double h = 2 * M_PI / Np;
+  d1->assign(Np, 0.0);
+  d2->assign(Np, 0.0);
+  const bool even = Np % 2 == 0;
+  (*d2)[0] = -h * h * ((double)Np * Np + (even ? 2.0 : -1.0)) / 12.0;
+  for (int j = 1; 2 * j <= Np; ++j) {
+    double c, s;   // of pi j / N'
+    sincos2pi(j, 2LL * Np, &c, &s);
+    const double sg = j % 2 ? -1.0 : 1.0;
+    const double v1 = 2 * j == Np ? 0.0 : 0.5 * h * sg * (even ? c : 1.0) / s;
+    const double v2 = -h * h * sg * (even ? 1.0 : c) / (2 * s * s);
+    (*d1)[j] = v1;
+    if (2 * j != Np) (*d1)[Np - j] = -v1;
+    (*d2)[j] = (*d2)[Np - j] = v2;
+  }
+}
+
+int dense_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out) {
+  // B(jo, ji) of part (s, m): sum over the distinct rows n of orbit ji of
+  // sign(n) c(n0(jo) - n) / NQ, sign = 1, m, s, s m for the four members
+  std::vector<double> B((size_t)g.NQ * g.No * g.No);
+  double most = 0.0;
+  for (int ji = 0; ji < g.No; ++ji) {
+    int rows[4], n = 0, member[4];
+    for (int i = 0; i < g.NQ; ++i) {
+      const int r = dense_row(g, ji, i);
+      bool seen = false;
+      for (int k = 0; k < n; ++k) seen = seen || rows[k] == r;
+      if (seen) continue;
+      rows[n] = r;
+      member[n++] = i;
+    }
+    for (int jo = 0; jo < g.No; ++jo) {
+      const int n0 = dense_row(g, jo, 0);
+      for (int q = 0; q < g.NQ; ++q) {   // q & 1: m = -1, q & 2: s = -1
+        double v = 0.0;
+        for (int k = 0; k < n; ++k) {
+          const int neg = ((q & member[k] & 1) + ((q & member[k] & 2) >> 1)) & 1;
+          const double x = c[((n0 - rows[k]) % g.Np + g.Np) % g.Np];
+          v += neg ? -x : x;
+        }
+        v /= g.NQ;
+        B[((size_t)q * g.No + jo) * g.No + ji] = v;
+        most = std::max(most, std::fabs(v));
+      }
+    }
+  }
+  const int e = 12 - (most > 0.0 ? std::ilogb(most) : 0);
+  const double sc = std::ldexp(1.0, e);
+  auto half_bits = [](double v, double* back) {
+    const __half h = __double2half(v);
+    *back = (double)__half2float(h);
+    unsigned short b;
+    std::memcpy(&b, &h, 2);
+    return b;
+  };
+  out->reserve(out->size() + (size_t)dense_order_halves(g));
+  std::vector<unsigned short> low;
+  for (int ch = 0; ch < g.chunks; ++ch)
+    for (int q = 0; q < g.NQ; ++q)
+      for (int s = 0; s < g.slabs; ++s) {
+        low.clear();
+        for (int kc = 2 * s * g.per; kc < 2 * (s * g.per + dense_slab(g, s)); ++kc)
+          for (int r = 0; r < g.NC; ++r)
+            for (int k = 0; k < 8; ++k) {
+              const int jo = ch * g.NC + r, ji = kc * 8 + k;
+              const double v = jo < g.No && ji < g.No ? sc * B[((size_t)q * g.No + jo) * g.No + ji] : 0.0;
+              double hv, lv;
+              out->push_back(half_bits(v, &hv));
+              low.push_back(half_bits(v - hv, &lv));
+            }
+        out->insert(out->end(), low.begin(), low.end());
+      }
+  return e;
 }
 
 }  // namespace fcns

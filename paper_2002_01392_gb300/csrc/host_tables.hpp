@@ -3,6 +3,8 @@
 #include <complex>
 #include <vector>
 
+#include "dense_geom.hpp"
+
 namespace fcns {
 
 struct FcTables {
@@ -53,6 +55,20 @@ void bluestein_tables(int Np, int L, std::vector<std::complex<double>>* chirp,
 void engine_twiddles(int L1, int L2, std::vector<std::complex<double>>* tw);
 // e^{-2 pi i k / N}, k = 0 .. N/2 (computed in binary128, rounded to double)
 void split_twiddles(int N, std::vector<std::complex<double>>* tw);
+
+// Derivative kernels of the N'-periodic unit grid, c[j] for j = 0..N'-1
+// (d1 odd and d2 even exactly; the Nyquist mode zeroed in d1, kept in d2), from
+// their closed forms.
+void deriv_kernels_closed(int Np, std::vector<double>* d1, std::vector<double>* d2);
+
+// Blocks of the dense z operator with kernel c (c[j], j modulo N'; odd or
+// even) on the geometry g, scaled by 2^(12 - e), e the exponent of the largest
+// entry, and split into float16 high and low parts: per output chunk, part and
+// contraction slab the high values and then the low values, each as groups of
+// eight contraction indexes x NC outputs (the shared-memory image the kernel
+// copies).  `out` gets dense_order_halves(g) values appended; returns the
+// scale exponent 12 - e.
+int dense_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out);
 
 // cos / sin of 2 pi num / den, correctly rounded to double from binary128.
 void sincos2pi(long long num, long long den, double* c, double* s);

@@ -214,6 +214,33 @@ int fchc_ns_autotune(void* h, int* tiles) {
   for (int k = 0; k < NsCore<EmuBK>::TK_N; ++k) tiles[k] = c->tile[k];
   return s;
 }
+// geometry of the dense z operators for (Nz, N'): out = NQ, No, KQ, NC, chunks, slabs; 1 where there is none
+int fchc_dense_geom(int Nz, int Np, int* out) {
+  DenseGeom g;
+  if (!dense_geom(Nz, Np, &g)) return 1;
+  const int v[6] = {g.NQ, g.No, g.KQ, g.NC, g.chunks, g.slabs};
+  for (int i = 0; i < 6; ++i) out[i] = v[i];
+  return 0;
+}
+int fchc_dense_row(int Nz, int Np, int j, int i) {
+  DenseGeom g;
+  return dense_geom(Nz, Np, &g) ? dense_row(g, j, i) : -1;
+}
+int fchc_dense_slab(int Nz, int Np, int s) {
+  DenseGeom g;
+  return dense_geom(Nz, Np, &g) ? dense_slab(g, s) : -1;
+}
+// blocks of derivative order 1 or 2 (float16 bits, as the kernel copies them) and their scale exponent
+int fchc_dense_blocks(int Nz, int Np, int order, unsigned short* halves, int* exponent) {
+  DenseGeom g;
+  if (!dense_geom(Nz, Np, &g)) return 1;
+  std::vector<double> c1, c2;
+  deriv_kernels_closed(Np, &c1, &c2);
+  std::vector<unsigned short> out;
+  *exponent = dense_blocks(g, order == 1 ? c1 : c2, &out);
+  std::memcpy(halves, out.data(), 2 * out.size());
+  return (long long)out.size() == dense_order_halves(g) ? 0 : 2;
+}
 // thread order inside a phase (0 ascending, 1 descending) and shared-memory
 // poisoning of the emulation (see phased_emulate)
 void fchc_set_emulation(int order, int poison) {

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/fcns.h"
+#include "dense_geom.hpp"
 
 namespace fcns {
 
@@ -34,6 +35,8 @@ struct DerivDevTables {
   void* H1_64 = nullptr;
   void* H2_32 = nullptr;
   void* H2_64 = nullptr;
+  void* dense = nullptr;          // blocks of the dense operators (float16 pairs), both orders; null: not used
+  unsigned* dense_err = nullptr;  // host word (pinned) that a kernel sets when a wait runs out
   // staging of fc_deriv_z_host: three rotating slots of (input, d1, d2) slab
   // buffers of stage_bytes each, and the copy-in / compute / copy-out streams
   size_t stage_bytes = 0;
@@ -46,6 +49,10 @@ struct PlanData {
   int d, C, Nz, Np, M, n_os;
   double ls_residual;
   std::vector<double> Mr;
+  DenseGeom dense;                        // dense operators (NQ = 0: none)
+  int dense_exp[2] = {0, 0};
+  bool dense_direct = false;              // the transform kernel would run at length N' itself
+  std::vector<unsigned short> dense_blocks;
   std::mutex mtx;
   std::mutex host_mtx;   // serialises fc_deriv_z_host calls on the plan (shared staging)
   std::vector<DerivDevTables> dev;
@@ -77,5 +84,10 @@ namespace fcns {
 fc_status launch_deriv_z(const DerivDevTables& t, const PlanData& p, fc_dtype dtype, int batch,
                          long long lines, double Lz, const void* f, void* df, void* d2f,
                          cudaStream_t stream);
+// the same by the dense operators (float32; plans with a dense geometry)
+fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int batch, long long lines, double Lz,
+                             const void* f, void* df, void* d2f, cudaStream_t stream);
+// whether a whole call (all its lines) takes the dense operators
+bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines);
 
 }  // namespace fcns

@@ -1,0 +1,74 @@
+// Launch of the dense z operators (dense_z.cuh).
+#include <atomic>
+#include <cmath>
+
+#include "dense_z.cuh"
+#include "internal.hpp"
+
+namespace fcns {
+
+static fc_status launch_dense(DenseArgs a, cudaStream_t stream) {
+  // as many slabs as fit beside the tile; a block set that fits whole is loaded once per CTA
+  const int slab = dense_slab_bytes(a.g), room = 227 * 1024 - dense_smem(a.g, a.d, a.Cc, 0).total;
+  const int nord = (a.orders & 1) + (a.orders >> 1);
+  const int all = nord * a.g.chunks * a.g.NQ * a.g.slabs;
+  a.stages = room / slab < 8 ? room / slab : 8;
+  if (a.stages < 2) return FC_ERR_UNSUPPORTED;
+  a.resident = all <= a.stages ? 1 : 0;
+  const DenseSmem so = dense_smem(a.g, a.d, a.Cc, a.stages);
+  // d = 5 (the default continuation) is compiled on its own
+  const int form = (a.g.NQ == 4 ? 1 : 0) + (a.d == 5 ? 2 : 0);
+  auto kern = form == 0 ? dense_z_kernel<2, 0> : form == 1 ? dense_z_kernel<4, 0> : form == 2 ? dense_z_kernel<2, 5> : dense_z_kernel<4, 5>;
+  static std::atomic<unsigned long long> attr_set[4];
+  std::atomic<unsigned long long>& attr = attr_set[form];
+  static std::atomic<int> sm_count[64];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 64 || !(attr.load() >> dev & 1ull)) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(dense z)");
+    if (dev < 64) attr.fetch_or(1ull << dev);
+  }
+  int sms = dev < 64 ? sm_count[dev].load() : 0;
+  if (!sms) {
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return cuda_status(e, "cudaDeviceGetAttribute");
+    if (dev < 64) sm_count[dev].store(sms);
+  }
+  a.tiles = (a.lines + kDenseLines - 1) / kDenseLines;
+  const unsigned grid = (unsigned)(a.tiles < sms ? a.tiles : sms);
+  kern<<<grid, kDenseThreads, so.total, stream>>>(a, so);
+  return cuda_status(cudaGetLastError(), "dense z launch");
+}
+
+fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int batch, long long lines, double Lz,
+                             const void* f, void* df, void* d2f, cudaStream_t stream) {
+  const unsigned gave_up = t.dense_err ? *static_cast<volatile unsigned*>(t.dense_err) : 0;
+  if (gave_up) {
+    *static_cast<volatile unsigned*>(t.dense_err) = 0;
+    set_error("fc_deriv_z: an earlier call's kernel gave up wait " + std::to_string(gave_up));
+    return FC_ERR_TIMEOUT;
+  }
+  DenseArgs a = {};
+  a.g = p.dense;
+  a.d = p.d;
+  a.Cc = p.C;
+  a.orders = (df ? 1 : 0) | (d2f ? 2 : 0);
+  a.Zin = p.Nz;
+  a.per = lines;
+  a.in_outer = a.out_outer = lines * p.Nz;
+  a.lines = lines * batch;
+  a.in = static_cast<const float*>(f);
+  a.out1 = static_cast<float*>(df);
+  a.out2 = static_cast<float*>(d2f);
+  a.B = static_cast<const __half*>(t.dense);
+  a.order_halves = dense_order_halves(a.g);
+  a.Mr2 = t.Mr2;
+  const double dz = Lz / (p.Nz - 1);
+  a.f1 = (float)std::ldexp(1.0 / dz, -p.dense_exp[0]);
+  a.f2 = (float)std::ldexp(1.0 / (dz * dz), -p.dense_exp[1]);
+  a.err = t.dense_err;
+  return launch_dense(a, stream);
+}
+
+}  // namespace fcns

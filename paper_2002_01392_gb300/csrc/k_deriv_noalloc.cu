@@ -11,8 +11,8 @@
 // until the process exits).  A call whose plan and precision differ from the
 // tables the array holds on this device copies the plan's tables into it on
 // the caller's stream first; a call with the same plan and precision as the
-// previous call on the device launches the kernel at once.
-#include <mutex>
+// previous call on the device launches the kernel at once.  Calls that
+// fc_deriv_z runs with the dense operators have a second array of their own.
 #include <mutex>
 
 #include "internal.hpp"
@@ -25,9 +25,15 @@ constexpr int kMaxDevices = 64;
 
 // Shared by every call on a device; holds the tables of the last call.
 static __device__ __align__(256) unsigned char g_deriv_scratch[kNoAllocBytes];
+// The same for calls that fc_deriv_z runs with the dense operators: their
+// blocks (at most 1.33 MB, N' = 575) and the continuation matrix.
+constexpr size_t kNoAllocDense = 1376 * 1024;
+static __device__ __align__(256) unsigned char g_dense_scratch[kNoAllocDense];
 
 std::mutex g_mtx;
 void* g_scratch_addr[kMaxDevices] = {};
+void* g_dense_addr[kMaxDevices] = {};
+unsigned long long g_dense_serial[kMaxDevices] = {};
 // which tables the array holds per device: the plan's serial number and the
 // precision of the last upload (0: none, or an upload that failed part-way)
 unsigned long long g_loaded_serial[kMaxDevices] = {};
@@ -46,6 +52,37 @@ fc_status scratch_address(int dev, unsigned char** out) {
   }
   *out = static_cast<unsigned char*>(g_scratch_addr[dev]);
   return FC_OK;
+}
+
+// the dense-operator call: blocks and matrix copied when the plan differs from the previous such call's
+fc_status noalloc_dense(fc_plan* plan, int dev, int batch, long long lines, double Lz, const void* f, void* df, void* d2f,
+                        cudaStream_t st) {
+  const size_t nB = 2 * plan->data.dense_blocks.size(), nM = sizeof(float2) * plan->deriv.Mr2.size();
+  if (nB + nM > kNoAllocDense) {
+    set_error("fc_deriv_z_noalloc: dense blocks of this plan exceed the static scratch");
+    return FC_ERR_UNSUPPORTED;
+  }
+  unsigned char* base = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_mtx);
+    fc_status s = FC_OK;
+    if (!g_dense_addr[dev])
+      s = cuda_status(cudaGetSymbolAddress(&g_dense_addr[dev], g_dense_scratch), "cudaGetSymbolAddress(g_dense_scratch)");
+    if (s) return s;
+    base = static_cast<unsigned char*>(g_dense_addr[dev]);
+    if (g_dense_serial[dev] != plan->deriv.serial) {
+      g_dense_serial[dev] = 0;
+      s = cuda_status(cudaMemcpyAsync(base, plan->data.dense_blocks.data(), nB, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(dense)");
+      if (!s) s = cuda_status(cudaMemcpyAsync(base + nB, plan->deriv.Mr2.data(), nM, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(Mr2)");
+      if (s) return s;
+      g_dense_serial[dev] = plan->deriv.serial;
+    }
+  }
+  DerivDevTables t;
+  t.device = dev;
+  t.dense = base;
+  t.Mr2 = reinterpret_cast<float2*>(base + nB);
+  return launch_deriv_dense(t, plan->data, batch, lines, Lz, f, df, d2f, st);
 }
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }
@@ -77,6 +114,8 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
   s = scratch_address(dev, &base);
   if (s) return s;
   cudaStream_t st = (cudaStream_t)stream;
+  if (deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch))
+    return noalloc_dense(plan, dev, batch, (long long)Nx * Ny, Lz, f, df, d2f, st);
   {
     std::lock_guard<std::mutex> lk(g_mtx);
     if (g_loaded_serial[dev] != h.serial || g_loaded_dtype[dev] != (int)dtype) {

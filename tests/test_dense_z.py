@@ -1,0 +1,170 @@
+"""The dense z operators (tensor-core form of the z derivatives): tables and
+geometry on the CPU, the kernel against the oracle and the transform kernel on
+the GPU."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from oracle import fc
+
+
+def _lib():
+    from paper_2002_01392_gb300 import build
+    build.build()
+    return ctypes.CDLL(build.HOSTCHECK)
+
+
+@pytest.mark.parametrize("Nz,C", [(10, 25), (33, 25), (32, 25), (39, 25), (103, 25), (104, 25), (129, 25), (231, 33),
+                                  (487, 25), (488, 25), (512, 25), (513, 25), (513, 33), (549, 25), (550, 25)])
+def test_dense_tables_are_the_derivative_operators(Nz, C):
+    """Orbits cover every row once per member; the blocks, put together by the
+    kernel's own rules (parts of a line, high + low values per slab, members of
+    an output orbit), are the circular derivative operators of the continued grid."""
+    lib, Np = _lib(), Nz + C
+    o = (ctypes.c_int * 6)()
+    assert lib.fchc_dense_geom(Nz, Np, o) == 0
+    NQ, No, KQ, NC, chunks, slabs = list(o)
+    assert NQ * KQ <= 576 and NC % 16 == 0 and NQ * NC <= 192 and chunks * NC >= No
+    rows = np.array([[lib.fchc_dense_row(Nz, Np, j, i) for i in range(NQ)] for j in range(No)])
+    assert sorted(set(rows.ravel())) == list(range(Np))
+    assert len({tuple(sorted(set(r))) for r in rows}) == No
+    x = np.random.default_rng(Nz).standard_normal((Np, 4))
+    # members (mirror, shift) and parts (m, s): sign (-1)^(bits of part & member)
+    sign = np.array([[(-1.0) ** bin(q & i).count("1") for i in range(NQ)] for q in range(NQ)])
+    parts = [sum(sign[q, i] * x[rows[:, i]] for i in range(NQ)) for q in range(NQ)]
+    cuts = np.cumsum([0] + [lib.fchc_dense_slab(Nz, Np, s) for s in range(slabs)])
+    assert cuts[-1] * 16 == KQ and (np.diff(cuts) > 0).all()
+    k = fc.kz_wavenumbers(Nz, C, Nz - 1.0)          # unit spacing
+    for order in (1, 2):
+        halves = np.zeros(2 * KQ * NC * chunks * NQ, dtype=np.uint16)
+        e = ctypes.c_int()
+        assert lib.fchc_dense_blocks(Nz, Np, order, halves.ctypes.data_as(ctypes.c_void_p), ctypes.byref(e)) == 0
+        v = halves.view(np.float16).astype(np.float64)
+        assert np.isfinite(v).all() and 2.0 ** 12 <= np.abs(v).max() <= 2.0 ** 13
+        Y = np.zeros((NQ, chunks * NC, 4))
+        p = 0
+        for ch in range(chunks):
+            for q in range(NQ):
+                for a, b in zip(cuts, cuts[1:]):
+                    n = (b - a) * 16 * NC
+                    B = (v[p:p + n] + v[p + n:p + 2 * n]).reshape(2 * (b - a), NC, 8).transpose(1, 0, 2).reshape(NC, -1)
+                    p += 2 * n
+                    src = np.zeros((KQ, 4))
+                    src[:No] = parts[q]
+                    Y[q, ch * NC:(ch + 1) * NC] += B @ src[16 * a:16 * b]
+        assert p == v.size and not Y[:, No:].any()
+        par = -1.0 if order == 1 else 1.0
+        y = np.full((Np, 4), np.nan)
+        for i in range(NQ):
+            y[rows[:, i]] = (par if i & 1 else 1.0) * sum(sign[q, i] * Y[q, :No] for q in range(NQ))
+        ref = np.fft.ifft(np.fft.fft(x, axis=0) * fc.deriv_factor(k, order)[:, None], axis=0).real
+        # the blocks carry 22 bits and a sign: each entry within 2^-23 of itself or 2^-25 of 1 (scaled to 2^12..2^13)
+        y *= 2.0 ** -e.value
+        assert np.abs(y - ref).max() < 2.0 ** -22 * np.pi ** order * np.abs(x).max() * np.sqrt(Np)
+
+
+# ---------------------------------------------------------------------------
+# the kernel (GPU)
+# ---------------------------------------------------------------------------
+@pytest.fixture(scope="module")
+def api():
+    torch = pytest.importorskip("torch")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2002_01392_gb300 import api as a
+    assert torch.cuda.is_available()
+    return a
+
+
+def _oracle(f, Mr, order, Lz=1.0):
+    """Derivative of f [Nz][lines] as the dense operator, in float64."""
+    return fc.dense_deriv_operator(f.shape[0], Mr.shape[0], Lz, Mr, order) @ f.astype(np.float64)
+
+
+def _bound(f, Mr, order, Lz=1.0):
+    """Rounding of the split operands and of the float32 sums, per line: the operator's entries and the line carry
+    2^-23 of their largest magnitudes each, products and sums of a block of at most 36 16-steps 2^-24 per addition,
+    all amplified by at most k_max^order over the continued line's 2-norm."""
+    xe = fc.extend(f.astype(np.float64), Mr)
+    kmax = np.pi * (f.shape[0] - 1) / Lz
+    return 16 * 2.0 ** -23 * kmax ** order * np.linalg.norm(xe, axis=0)
+
+
+# every branch: parts 4 (N' even) and 2 (odd), one and several chunks and slabs, resident blocks, direct lengths, a last
+# tile of few lines, a tile across two fields, odd line counts, one output, Lz
+@pytest.mark.gpu
+@pytest.mark.parametrize("Nz,Ny,Nx,B,Lz", [(50, 257, 511, 1, 1.0), (65, 256, 513, 1, 2.0), (104, 363, 121, 3, 1.0),
+                                            (155, 128, 128, 1, 1.0), (231, 193, 255, 2, 1.0), (257, 129, 128, 1, 1.0),
+                                            (350, 64, 257, 1, 0.5), (487, 317, 311, 1, 1.0), (512, 131, 127, 1, 1.0),
+                                            (513, 64, 129, 2, 1.0), (549, 128, 129, 1, 1.0)])
+def test_dense_kernel_matches_oracle(api, Mr_5_25, Nz, Ny, Nx, B, Lz):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(Nz)
+    z = torch.arange(Nz, device="cuda") / (Nz - 1)
+    amp = torch.rand((3, B, 1, Ny, Nx), generator=g, device="cuda") * 2 - 1
+    zz = z[None, :, None, None]
+    f = amp[0] * torch.sin(9 * zz) + amp[1] * torch.cos(31 * zz * amp[2]) * 10
+    f[:, ::7] += 1e-3 * torch.rand((B, (Nz + 6) // 7, Ny, Nx), generator=g, device="cuda")
+    f = f.contiguous()
+    plan = api.Plan(5, 25, Nz)
+    d1, d2 = torch.full_like(f, float("nan")), torch.full_like(f, float("nan"))
+    api.fc_deriv_z(plan, f, d1, d2, Lz=Lz)
+    only = torch.full_like(f, float("nan"))
+    api.fc_deriv_z(plan, f, None, only, Lz=Lz)
+    torch.cuda.synchronize()
+    assert torch.equal(only, d2) and torch.isfinite(d1).all() and torch.isfinite(d2).all()
+    lines = lambda t: t.permute(0, 2, 3, 1).reshape(-1, Nz)  # noqa: E731
+    n = Ny * Nx * B
+    pick = np.unique(np.r_[0:130, n // 2 - 65:n // 2 + 65, n - 140:n])
+    fp, o1, o2 = (lines(t)[pick].cpu().numpy().T for t in (f, d1, d2))
+    for order, out in ((1, o1), (2, o2)):
+        err = np.linalg.norm(out - _oracle(fp, Mr_5_25, order, Lz), axis=0)
+        assert (err <= _bound(fp, Mr_5_25, order, Lz)).all(), (order, (err / _bound(fp, Mr_5_25, order, Lz)).max())
+
+
+@pytest.mark.gpu
+def test_dense_kernel_magnitudes_and_nonfinite(api, Mr_5_25):
+    """Lines whose sample gives the wrong scale (a peak between sampled rows, zero but for one row), of magnitudes from
+    1e-37 to 1e33, of zeros: each to its own bound; a NaN or Inf spoils its own line only.  Entry points that route the
+    same call agree bitwise."""
+    import ctypes
+    import torch
+    Nz, Ny, Nx = 513, 8, 2050
+    r = np.random.default_rng(5)
+    z = np.arange(Nz) / (Nz - 1)
+    base = (np.sin(np.outer(z, r.uniform(3, 40, Ny * Nx)) + 1)).astype(np.float32)
+    f = base.copy()
+    f[:, 0:9] = 0
+    f[Nz // 2 + 1, 0:9] = 1e5
+    f[:, 9:18] *= 1e-3
+    f[Nz // 3 + 1, 9:18] = 1e4
+    for i, s in enumerate((1e33, 1e-30, 1e-37)):
+        f[:, 18 + 9 * i:27 + 9 * i] *= np.float32(s)
+    f[:, 45:54] = 0
+    f[5, 300], f[7, 500] = np.nan, np.inf
+    ft = torch.from_numpy(f).cuda().view(Nz, Ny, Nx)
+    plan = api.Plan(5, 25, Nz)
+    d = [torch.empty_like(ft) for _ in range(2)]
+    api.fc_deriv_z(plan, ft, *d)
+    out = [t.view(Nz, -1).cpu().numpy() for t in d]
+    good = np.ones(Ny * Nx, bool)
+    good[[300, 500]] = False
+    for o in out:
+        assert np.isfinite(o[:, good]).all() and not np.isfinite(o[:, ~good]).any()
+        assert not o[:, 45:54].any()
+    pick = np.r_[0:45, 54:200, 640:700]
+    for order in (1, 2):
+        err = np.linalg.norm(out[order - 1][:, pick] - _oracle(f[:, pick], Mr_5_25, order), axis=0)
+        assert (err <= _bound(f[:, pick], Mr_5_25, order)).all()
+    # host arrays in slabs, and the variant without allocations
+    h = [torch.empty((Nz, Ny, Nx)) for _ in range(2)]
+    api.fc_deriv_z_host(plan, ft.cpu(), *h, slab_bytes=2 * Nz * Nx * 4)
+    n = [torch.empty_like(ft) for _ in range(2)]
+    assert api._lib.fc_deriv_z_noalloc(plan.handle, api.FC_F32, 1, Nx, Ny, ctypes.c_double(1.0), ft.data_ptr(),
+                                       n[0].data_ptr(), n[1].data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+    torch.cuda.synchronize()
+    for a, b, c in zip(d, h, n):
+        av = a.cpu().view(torch.int32)
+        fin = torch.isfinite(a.cpu())
+        assert torch.equal(av[fin], b.view(torch.int32)[fin]) and torch.equal(av[fin], c.cpu().view(torch.int32)[fin])
