@@ -13,15 +13,7 @@
 // FFT of length L = L1 * L2 in two register passes with one shared-memory
 // exchange each way (engine.cuh).
 #pragma once
-#include "phases.cuh"
-
-#if defined(__CUDACC__)
-#define DERIV_NOINLINE __host__ __device__ __noinline__
-#else
-#define DERIV_NOINLINE
-#endif
-
-#include "engine.cuh"
+#include "continuation.cuh"
 
 namespace fcns {
 
@@ -62,10 +54,8 @@ struct DerivPair {
   using C = cx<T>;
   static constexpr int L1 = L1_, L2 = L2_, LINES = LINES_, JN = JN_;
   static_assert(JI <= JN_, "interior rows lie among the loaded rows");
-  static constexpr int THREADS = E::THREADS, NPHASE = 4;
+  static constexpr int THREADS = E::THREADS, NPHASE = 5;
   static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
-  static constexpr int MR_MAX = 640;
-  static constexpr int DMAX = 10;
 
   struct Args {
     const T* f;
@@ -94,34 +84,6 @@ struct DerivPair {
   static constexpr size_t off_E = off_b1 + sizeof(C) * E::BUF;
   static constexpr size_t smem_bytes = off_E + sizeof(C) * LINES * 2 * DMAX;
 
-  // continuation value jj of a complex line: M_r f_last + M_l f_first, with
-  // compensated sums in both precisions (float-float / double-double)
-  static DERIV_NOINLINE C cont_cplx(int jj, const C* first, const C* last, int d, int Cc, const double* Ms,
-                                    const float2* Ms2) {
-    if constexpr (sizeof(T) == 4) {
-      ff re{0.f, 0.f}, im{0.f, 0.f};
-      for (int i = 0; i < d; ++i) {
-        const float2 m1 = Ms2[jj * d + i];
-        const float2 m2 = Ms2[(Cc - 1 - jj) * d + (d - 1 - i)];
-        ff_fma(re, m1.x, m1.y, last[i].x);
-        ff_fma(im, m1.x, m1.y, last[i].y);
-        ff_fma(re, m2.x, m2.y, first[i].x);
-        ff_fma(im, m2.x, m2.y, first[i].y);
-      }
-      return mk<T>(ff_round(re), ff_round(im));
-    } else {
-      dd re{0.0, 0.0}, im{0.0, 0.0};
-      for (int i = 0; i < d; ++i) {
-        const double m1 = Ms[jj * d + i], m2 = Ms[(Cc - 1 - jj) * d + (d - 1 - i)];
-        dd_fma(re, m1, last[i].x);
-        dd_fma(im, m1, last[i].y);
-        dd_fma(re, m2, first[i].x);
-        dd_fma(im, m2, first[i].y);
-      }
-      return mk<T>((T)dd_round(re), (T)dd_round(im));
-    }
-  }
-
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
     C* b0 = reinterpret_cast<C*>(sm);
@@ -130,8 +92,8 @@ struct DerivPair {
     const float2* Ms2 = a.Mr2;
     const int r = tid / LINES, li = tid % LINES;
     C* Ev = reinterpret_cast<C*>(sm + off_E) + li * 2 * DMAX;
-    const long long field = bid / a.tiles;
-    const long long pair = (bid % a.tiles) * LINES + li;
+    const long long field = (unsigned)bid / (unsigned)a.tiles;
+    const long long pair = (long long)((unsigned)bid % (unsigned)a.tiles) * LINES + li;
     const long long la = 2 * pair;                 // first line of the pair
     const bool va = FULL || la < a.lines, vb = FULL || la + 1 < a.lines;
     const long long base = field * a.bstride + la;
@@ -169,19 +131,23 @@ struct DerivPair {
       // bring its input rows into L2 while this block computes
       if (a.pf_dist > 0 && bid + a.pf_dist < a.nblocks) {
         const long long b2 = bid + a.pf_dist;
-        const long long f2 = b2 / a.tiles, p2 = (b2 % a.tiles) * LINES;
+        const long long f2 = (unsigned)b2 / (unsigned)a.tiles, p2 = (long long)((unsigned)b2 % (unsigned)a.tiles) * LINES;
         const T* src = a.f + f2 * a.bstride + 2 * p2;
         for (int n = tid; n < a.Nz; n += THREADS) prefetch_l2(src + (long long)n * a.zstride);
       }
+      // continuation values into the second exchange buffer, idle until the inverse transforms (C <= 64 <= L)
+      continue_lines<T, LINES, THREADS>(tid, reinterpret_cast<const C*>(sm + off_E), 2 * DMAX, a.d, a.Cc, Ms, Ms2,
+                                        [&](int jj, int l, C v) { b1[jj * LINES + l] = v; });
+    } else if constexpr (P == 2) {
       if (r < L2) {
 #pragma unroll
         for (int j = JI; j < JN; ++j) {
           const int n = r + L2 * j;
-          if (n >= a.Nz && n < a.Np) R.v[j] = cont_cplx(n - a.Nz, Ev, Ev + DMAX, a.d, a.Cc, Ms, Ms2);
+          if (n >= a.Nz && n < a.Np) R.v[j] = b1[(n - a.Nz) * LINES + li];
         }
         E::template A<-1>(R.v, b0, a.tw, r, li);
       }
-    } else if constexpr (P == 2) {
+    } else if constexpr (P == 3) {
       if (r < L1) {
         E::template B<-1>(R.u, b0, r, li);
 #pragma unroll
@@ -204,7 +170,7 @@ struct DerivPair {
           E::template Bi<1>(R.u, bo, a.tw, r, li);
         }
       }
-    } else if constexpr (P == 3) {
+    } else if constexpr (P == 4) {
       if (r < L2 && va) {
 #pragma unroll 1
         for (int o = 0; o < 2; ++o) {

@@ -344,6 +344,25 @@ __host__ __device__ __forceinline__ void ff_fma(ff& s, float mhi, float mlo, flo
 
 __host__ __device__ __forceinline__ float ff_round(const ff& s) { return s.hi + s.lo; }
 
+// the same sum for the two parts of a complex value (h + l) += (mhi + mlo) x,
+// on the device as packed 2 x fp32 operations: half the instructions
+__host__ __device__ __forceinline__ void ff_fma2(float2& h, float2& l, float mhi, float mlo, float2 x) {
+#if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 1000)
+  const float2 m = make_float2(mhi, mhi), n1 = make_float2(-1.f, -1.f), p = __fmul2_rn(m, x);
+  const float2 e = __ffma2_rn(m, x, make_float2(-p.x, -p.y));
+  const float2 t = __fadd2_rn(h, p), z = __ffma2_rn(h, n1, t);   // t - h
+  const float2 r = __fadd2_rn(__ffma2_rn(__ffma2_rn(z, n1, t), n1, h), __ffma2_rn(z, n1, p));
+  h = t;
+  l = __fadd2_rn(l, __fadd2_rn(__fadd2_rn(r, e), __fmul2_rn(make_float2(mlo, mlo), x)));
+#else
+  ff a{h.x, l.x}, b{h.y, l.y};
+  ff_fma(a, mhi, mlo, x.x);
+  ff_fma(b, mhi, mlo, x.y);
+  h.x = a.hi; l.x = a.lo;
+  h.y = b.hi; l.y = b.lo;
+#endif
+}
+
 // The same compensated sum in double (a "double-double" accumulator): the
 // float64 path's continuation product, whose weights reach 4e3 and cancel, so
 // that plain double sums would put ~1e-12 |f| of rounding into the continued

@@ -18,7 +18,7 @@
 #pragma once
 #include <cmath>
 
-#include "engine.cuh"
+#include "continuation.cuh"
 
 namespace fcns {
 
@@ -66,6 +66,19 @@ FC_HD int lay(long long f, long long z, long long line, long long Z, long long n
   return ((((int)f * (int)ntiles + (l >> 4)) * (int)Z + (int)z) << 4) + (l & (TL - 1));
 }
 
+// quotient and remainder of non-negative values below 2^31 (block, line and row numbers), in 32 bits: a 64-bit division
+// is about 100 instructions, and a kernel makes several per thread
+FC_HD int qdiv(long long a, long long b) { return (int)((unsigned)a / (unsigned)b); }
+FC_HD int qmod(long long a, long long b) { return (int)((unsigned)a % (unsigned)b); }
+// the x kernels: element 0 of row (z, y) = row of field 0, and what element k of a row lies further (Kxp is a multiple of
+// TL, so a row starts a tile)
+template <class A>
+FC_HD int xbase(const A& a, long long row) {
+  return lay(0, qdiv(row, a.Ny), (long long)qmod(row, a.Ny) * a.Kxp, a.Nz, a.ntiles);
+}
+template <class A>
+FC_HD int xoff(const A& a, int k) { return (k / TL) * (a.Nz * TL) + k % TL; }
+
 // lines of a tile row that share one 32-byte L2 sector
 template <class C>
 constexpr int sector_lines() { return sizeof(C) >= 32 ? 1 : 32 / (int)sizeof(C); }
@@ -84,47 +97,8 @@ FC_HD void prefetch_line(const C* base, long long f, long long line, int Z, int 
   }
 }
 
-#if defined(__CUDACC__)
-#define FC_NOINLINE __host__ __device__ __noinline__
-#else
-#define FC_NOINLINE
-#endif
 
-constexpr int DMAX = 10;
 constexpr int MRMAX = 640;
-
-
-// C continuation value jj (point Nz + jj) of a complex line from its first /
-// last d values (Sec. 3 continuation formula; right matrix M_r, left matrix
-// its row/column reversal), with compensated sums: float-float products in
-// float32, double-double in float64 (the weights reach 4e3 and cancel).
-template <class T>
-FC_NOINLINE cx<T> continuation_value(int jj, const cx<T>* first, const cx<T>* last, int d, int Cc,
-                                     const double* Ms, const float2* Ms2) {
-  if constexpr (sizeof(T) == 4) {
-    ff re{0.f, 0.f}, im{0.f, 0.f};
-    for (int i = 0; i < d; ++i) {
-      const float2 m1 = Ms2[jj * d + i];
-      const float2 m2 = Ms2[(Cc - 1 - jj) * d + (d - 1 - i)];
-      ff_fma(re, m1.x, m1.y, last[i].x);
-      ff_fma(im, m1.x, m1.y, last[i].y);
-      ff_fma(re, m2.x, m2.y, first[i].x);
-      ff_fma(im, m2.x, m2.y, first[i].y);
-    }
-    return mk<T>(ff_round(re), ff_round(im));
-  } else {
-    dd re{0.0, 0.0}, im{0.0, 0.0};
-    for (int i = 0; i < d; ++i) {
-      const double m1 = Ms[jj * d + i];
-      const double m2 = Ms[(Cc - 1 - jj) * d + (d - 1 - i)];
-      dd_fma(re, m1, last[i].x);
-      dd_fma(im, m1, last[i].y);
-      dd_fma(re, m2, first[i].x);
-      dd_fma(im, m2, first[i].y);
-    }
-    return mk<T>((T)dd_round(re), (T)dd_round(im));
-  }
-}
 
 template <class T>
 FC_HD void load_mr(unsigned char* sm, const ZTab<T>& t, int n, int tid, int threads) {
@@ -171,9 +145,9 @@ struct KZDeriv {
     C* b0 = reinterpret_cast<C*>(sm);
     C* b1 = reinterpret_cast<C*>(sm + off_b1);
     const int r = tid / LINES, li = tid % LINES;
-    const long long f = bid / a.tiles;
-    const long long line = (bid % a.tiles) * LINES + li;
-    const bool valid = line < a.g.lines && (line % a.g.Kxp) < a.g.Kx;
+    const long long f = qdiv(bid, a.tiles);
+    const long long line = (qmod(bid, a.tiles)) * LINES + li;
+    const bool valid = line < a.g.lines && (qmod(line, a.g.Kxp)) < a.g.Kx;
     if constexpr (P == 0) {
       if (r < L2) {
         const C* x = a.X + lay(f, 0, line, a.g.Np, a.g.ntiles);
@@ -183,9 +157,9 @@ struct KZDeriv {
           R.v[j] = (j < JN && valid && n < a.g.Np) ? x[n * TL] : mk<T>(0, 0);
         }
         if (a.pf > 0 && bid + a.pf < a.nblocks) {
-          const long long b2 = bid + a.pf, line2 = (b2 % a.tiles) * LINES + li;
-          if (line2 < a.g.lines && (line2 % a.g.Kxp) < a.g.Kx)
-            prefetch_line<C, JN>(a.X, b2 / a.tiles, line2, a.g.Np, a.g.Np, a.g.ntiles, r, L2, li);
+          const long long b2 = bid + a.pf, line2 = (qmod(b2, a.tiles)) * LINES + li;
+          if (line2 < a.g.lines && (qmod(line2, a.g.Kxp)) < a.g.Kx)
+            prefetch_line<C, JN>(a.X, qdiv(b2, a.tiles), line2, a.g.Np, a.g.Np, a.g.ntiles, r, L2, li);
         }
         E::template A<-1>(R.v, b0, a.t.tw, r, li);
       }
@@ -241,7 +215,7 @@ template <class T, int L1, int L2, int LINES, int JN = L1>
 struct KZCombine {
   using E = Eng<T, L1, L2, LINES>;
   using C = cx<T>;
-  static constexpr int THREADS = E::THREADS, NPHASE = 5;
+  static constexpr int THREADS = E::THREADS, NPHASE = 6;
   static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
   struct Args {
     ZGeom g;
@@ -261,18 +235,21 @@ struct KZCombine {
   struct Regs { C v[L1]; C u[L2]; };
   static constexpr size_t off_M = sizeof(C) * E::BUF;
   static constexpr size_t off_E = off_M + sizeof(double) * MRMAX;
-  static constexpr size_t smem_bytes = off_E + sizeof(C) * LINES * 2 * DMAX;
+  static constexpr size_t off_C = off_E + sizeof(C) * LINES * 2 * DMAX;   // continuation values [C][LINES]
+  static constexpr size_t smem_bytes = off_C + sizeof(C) * LINES * CMAX;
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
     C* b0 = reinterpret_cast<C*>(sm);
     const double* Ms = reinterpret_cast<const double*>(sm + off_M);
     const float2* Ms2 = reinterpret_cast<const float2*>(sm + off_M);
-    C* Ev = reinterpret_cast<C*>(sm + off_E) + li_of(tid) * 2 * DMAX;
+    C* E0 = reinterpret_cast<C*>(sm + off_E);
+    C* Ev = E0 + li_of(tid) * 2 * DMAX;
+    C* Cv = reinterpret_cast<C*>(sm + off_C);
     const int r = tid / LINES, li = tid % LINES;
-    const int f = (int)(bid / a.tiles);
-    const long long line = (bid % a.tiles) * LINES + li;
-    const bool valid = line < a.g.lines && (line % a.g.Kxp) < a.g.Kx;
+    const int f = (int)(qdiv(bid, a.tiles));
+    const long long line = (qmod(bid, a.tiles)) * LINES + li;
+    const bool valid = line < a.g.lines && (qmod(line, a.g.Kxp)) < a.g.Kx;
     const int Nz = a.g.Nz, Np = a.g.Np, d = a.g.d;
     const long long Ls = a.g.lines;
     if constexpr (P == 0) {
@@ -301,30 +278,33 @@ struct KZCombine {
           if (a.Xt) prefetch_line<C, JN>(a.Xt, f, line, Np, Nz, a.g.ntiles, r, L2, li);
         }
         if (a.pf > 0 && bid + a.pf < a.nblocks) {
-          const long long b2 = bid + a.pf, line2 = (b2 % a.tiles) * LINES + li;
-          if (line2 < a.g.lines && (line2 % a.g.Kxp) < a.g.Kx)
-            prefetch_line<C, JN>(a.NL, b2 / a.tiles, line2, Nz, Nz, a.g.ntiles, r, L2, li);
+          const long long b2 = bid + a.pf, line2 = (qmod(b2, a.tiles)) * LINES + li;
+          if (line2 < a.g.lines && (qmod(line2, a.g.Kxp)) < a.g.Kx)
+            prefetch_line<C, JN>(a.NL, qdiv(b2, a.tiles), line2, Nz, Nz, a.g.ntiles, r, L2, li);
         }
       }
     } else if constexpr (P == 1) {
+      continue_lines<T, LINES, THREADS>(tid, E0, 2 * DMAX, d, a.g.Cc, Ms, Ms2,
+                                        [&](int jj, int l, C v) { Cv[jj * LINES + l] = v; });
+    } else if constexpr (P == 2) {
       if (r < L2) {
 #pragma unroll
         for (int j = 0; j < JN; ++j) {
           const int n = r + L2 * j;
-          if (n >= Nz && n < Np) R.v[j] = continuation_value<T>(n - Nz, Ev, Ev + DMAX, d, a.g.Cc, Ms, Ms2);
+          if (n >= Nz && n < Np) R.v[j] = Cv[(n - Nz) * LINES + li];
         }
         E::template A<-1>(R.v, b0, a.t.tw, r, li);
       }
-    } else if constexpr (P == 2) {
+    } else if constexpr (P == 3) {
       if (r < L1) {
         E::template B<-1>(R.u, b0, r, li);
         E::mulH_real(R.u, a.t.Hf, r);   // even filter kernel: real spectrum
         E::template Bi<1>(R.u, b0, a.t.tw, r, li);
       }
-    } else if constexpr (P == 3) {
+    } else if constexpr (P == 4) {
       if (r < L2) {
         E::template Ai<1>(R.v, b0, r, li);
-        const int kx = (int)(line % a.g.Kxp), ky = (int)(line / a.g.Kxp);
+        const int kx = (int)(qmod(line, a.g.Kxp)), ky = (int)(qdiv(line, a.g.Kxp));
         const T fxy = valid ? a.t.fx[kx] * a.t.fy[ky] : T(0);
         const T ckp2 = valid ? a.t.kx[kx] * a.t.kx[kx] + a.t.ky[ky] * a.t.ky[ky] : T(0);
         const T cdt = (T)a.dtj, cnu = (T)(a.dif[f]);
@@ -361,16 +341,12 @@ struct KZCombine {
           }
         }
       }
-    } else if constexpr (P == 4) {
-      if (r < L2 && valid) {
-        C* xo = a.Xout + lay(f, 0, line, Np, a.g.ntiles);
-#pragma unroll
-        for (int j = 0; j < JN; ++j) {
-          const int n = r + L2 * j;
-          if (n >= Nz && n < Np)
-            xo[n * TL] = continuation_value<T>(n - Nz, Ev, Ev + DMAX, d, a.g.Cc, Ms, Ms2);
-        }
-      }
+    } else if constexpr (P == 5) {
+      const long long line0 = (qmod(bid, a.tiles)) * LINES;
+      continue_lines<T, LINES, THREADS>(tid, E0, 2 * DMAX, d, a.g.Cc, Ms, Ms2, [&](int jj, int l, C v) {
+        const long long ln = line0 + l;
+        if (ln < a.g.lines && (qmod(ln, a.g.Kxp)) < a.g.Kx) a.Xout[lay(f, Nz + jj, ln, Np, a.g.ntiles)] = v;
+      });
     }
   }
   static FC_HD int li_of(int tid) { return tid % LINES; }
@@ -405,9 +381,9 @@ struct KZContinue {
     const float2* Ms2 = reinterpret_cast<const float2*>(sm);
     const int r = tid / LINES, li = tid % LINES;
     C* Ev = reinterpret_cast<C*>(sm + off_E) + li * 2 * DMAX;
-    const int f = (int)(bid / a.tiles);
-    const long long line = (bid % a.tiles) * LINES + li;
-    const bool valid = line < a.g.lines && (line % a.g.Kxp) < a.g.Kx;
+    const int f = (int)(qdiv(bid, a.tiles));
+    const long long line = (qmod(bid, a.tiles)) * LINES + li;
+    const bool valid = line < a.g.lines && (qmod(line, a.g.Kxp)) < a.g.Kx;
     const int Nz = a.g.Nz, Np = a.g.Np, d = a.g.d;
     const long long Ls = a.g.lines;
     const C* m = a.M + lay(f, 0, line, Nz, a.g.ntiles);
@@ -415,6 +391,7 @@ struct KZContinue {
     if constexpr (P == 0) {
       load_mr<T>(sm, a.t, a.g.Cc * d, tid, THREADS);
       if (valid) {
+#pragma unroll 4
         for (int n = r; n < Nz; n += G) {
           C val = m[n * TL];
           if (a.gradp && (n == 0 || n == Nz - 1)) {
@@ -431,10 +408,10 @@ struct KZContinue {
           if (n >= Nz - d) Ev[DMAX + n - (Nz - d)] = val;
         }
       }
-    } else {
+    } else {   // (32 threads per line: one value each, out of line, which keeps the copying phase's registers few)
       if (valid)
         for (int n = Nz + r; n < Np; n += G)
-          x[n * TL] = continuation_value<T>(n - Nz, Ev, Ev + DMAX, d, a.g.Cc, Ms, Ms2);
+          x[n * TL] = continuation_any<T>(n - Nz, Ev, Ev + DMAX, d, a.g.Cc, Ms, Ms2);
     }
   }
 };
@@ -557,10 +534,10 @@ struct KZProject {
     double* W = reinterpret_cast<double*>(sm + off_W) + li * 16;
     C* Ev = reinterpret_cast<C*>(sm + off_E) + li * 4 * DMAX;   // Phi first, Phi last, Phi' first, Phi' last
     const long long line = bid * LINES + li;
-    const bool valid = line < a.g.lines && (line % a.g.Kxp) < a.g.Kx;
+    const bool valid = line < a.g.lines && (qmod(line, a.g.Kxp)) < a.g.Kx;
     const int Nz = a.g.Nz, Np = a.g.Np, d = a.g.d;
     const long long Ls = a.g.lines;
-    const int kxi = valid ? (int)(line % a.g.Kxp) : 0, kyi = valid ? (int)(line / a.g.Kxp) : 0;
+    const int kxi = valid ? (int)(qmod(line, a.g.Kxp)) : 0, kyi = valid ? (int)(qdiv(line, a.g.Kxp)) : 0;
     const T kxo = a.t.kxo[kxi], kyo = a.t.kyo[kyi];
     C* xu = a.X + lay(0, 0, line, Np, a.g.ntiles);
     C* xv = a.X + lay(1, 0, line, Np, a.g.ntiles);
@@ -674,38 +651,51 @@ struct KZProject {
         Ev[2 * DMAX + (q < d ? q : DMAX + (q - d))] = dph;
       }
     } else if constexpr (P == 6) {  // X -= grad phi^I + FC(grad phi^H); wall planes
+      // row n of line ln (wave numbers kx, ky): subtract the gradient of sigma and Phi, Phi' = ph, dph
+      auto update = [&](int n, long long ln, int l, T kx, T ky, C ph, C dph) {
+        C* q0 = SG ? reinterpret_cast<C*>(sm + off_G) + l : a.G0 + lay(0, 0, ln, Np, a.g.ntiles);
+        C* q1 = SG ? reinterpret_cast<C*>(sm + off_G) + LINES * NPC + l : a.G1 + lay(0, 0, ln, Np, a.g.ntiles);
+        const C sg = q1[n * GS], sz = q0[n * GS];
+        // i k Phi = (-k Phi.y, k Phi.x)
+        const C gx = cadd(cscale(sg, kx), mk<T>(-kx * ph.y, kx * ph.x));
+        const C gy = cadd(cscale(sg, ky), mk<T>(-ky * ph.y, ky * ph.x));
+        const C gz = cadd(sz, dph);
+        C* u = a.X + lay(0, n, ln, Np, a.g.ntiles);
+        C* v = a.X + lay(1, n, ln, Np, a.g.ntiles);
+        C* w = a.X + lay(2, n, ln, Np, a.g.ntiles);
+        *u = csub(*u, gx);
+        *v = csub(*v, gy);
+        *w = csub(*w, gz);
+        if (n == 0 || n == Nz - 1) {
+          const int wall = (n == 0) ? 0 : 1;
+          const double s = 1.0 / a.dtj;
+          a.gradp[((long long)wall * 2 + 0) * Ls + ln] = make_double2((double)gx.x * s, (double)gx.y * s);
+          a.gradp[((long long)wall * 2 + 1) * Ls + ln] = make_double2((double)gy.x * s, (double)gy.y * s);
+        }
+      };
       if (r < L2 && valid) {
         const T cf[5] = {(T)W[8], (T)W[9], (T)W[10], (T)W[11], (T)W[12]};
         const T tdz = (T)a.g.dz, tLz = (T)a.g.Lz;
 #pragma unroll
         for (int j = 0; j < JN; ++j) {
           const int n = r + L2 * j;
-          if (n < Np) {
+          if (n < Nz) {
             C ph, dph;
-            if (n < Nz) {
-              phi_at(cf, kxo, kyo, tdz, tLz, n, &ph, &dph);
-            } else {
-              ph = continuation_value<T>(n - Nz, Ev, Ev + DMAX, d, a.g.Cc, Ms, Ms2);
-              dph = continuation_value<T>(n - Nz, Ev + 2 * DMAX, Ev + 3 * DMAX, d, a.g.Cc, Ms, Ms2);
-            }
-            const int o = n * TL;
-            const C sg = g1[n * GS];
-            const C sz = g0[n * GS];
-            // i k Phi = (-k Phi.y, k Phi.x)
-            const C gx = cadd(cscale(sg, kxo), mk<T>(-kxo * ph.y, kxo * ph.x));
-            const C gy = cadd(cscale(sg, kyo), mk<T>(-kyo * ph.y, kyo * ph.x));
-            const C gz = cadd(sz, dph);
-            xu[o] = csub(xu[o], gx);
-            xv[o] = csub(xv[o], gy);
-            xw[o] = csub(xw[o], gz);
-            if (n == 0 || n == Nz - 1) {
-              const int wall = (n == 0) ? 0 : 1;
-              const double s = 1.0 / a.dtj;
-              a.gradp[((long long)wall * 2 + 0) * Ls + line] = make_double2((double)gx.x * s, (double)gx.y * s);
-              a.gradp[((long long)wall * 2 + 1) * Ls + line] = make_double2((double)gy.x * s, (double)gy.y * s);
-            }
+            phi_at(cf, kxo, kyo, tdz, tLz, n, &ph, &dph);
+            update(n, line, li, kxo, kyo, ph, dph);
           }
         }
+      }
+      // the continuation rows, spread over all threads
+      const C* E0 = reinterpret_cast<const C*>(sm + off_E);
+      for (int i = tid; i < a.g.Cc * LINES; i += THREADS) {
+        const int jj = i / LINES, l = i % LINES;
+        const long long ln = bid * LINES + l;
+        if (ln >= a.g.lines || (qmod(ln, a.g.Kxp)) >= a.g.Kx) continue;
+        const C* e = E0 + l * 4 * DMAX;
+        const C ph = continuation_value<T>(jj, e, e + DMAX, d, a.g.Cc, Ms, Ms2);
+        const C dph = continuation_value<T>(jj, e + 2 * DMAX, e + 3 * DMAX, d, a.g.Cc, Ms, Ms2);
+        update(Nz + jj, ln, l, a.t.kxo[qmod(ln, a.g.Kxp)], a.t.kyo[qdiv(ln, a.g.Kxp)], ph, dph);
       }
     }
   }
@@ -771,9 +761,9 @@ struct KYInv3 {
     C* b0 = reinterpret_cast<C*>(sm);
     C* b1 = b0 + E::BUF;
     const int r = tid / LINES, li = tid % LINES;
-    const long long tile = bid % a.tiles;
-    const long long pz = bid / a.tiles;          // f * Nz + z
-    const long long f = pz / a.g.Nz, z = pz % a.g.Nz;
+    const long long tile = qmod(bid, a.tiles);
+    const long long pz = qdiv(bid, a.tiles);          // f * Nz + z
+    const long long f = qdiv(pz, a.g.Nz), z = qmod(pz, a.g.Nz);
     const int kx = (int)(tile * LINES + li);
     const bool valid = kx < a.g.Kx;
     // line = ky * Kxp + kx with Kxp a multiple of TL: element offset base + ky * Kxp * Z
@@ -848,9 +838,9 @@ struct KYInv3S {
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
     C* b0 = reinterpret_cast<C*>(sm);
     const int r = tid / LINES, li = tid % LINES;
-    const long long tile = bid % a.tiles;
-    const long long pz = bid / a.tiles;          // f * Nz + z
-    const long long f = pz / a.g.Nz, z = pz % a.g.Nz;
+    const long long tile = qmod(bid, a.tiles);
+    const long long pz = qdiv(bid, a.tiles);          // f * Nz + z
+    const long long f = qdiv(pz, a.g.Nz), z = qmod(pz, a.g.Nz);
     const int kx = (int)(tile * LINES + li);
     const bool valid = kx < a.g.Kx;
     const int sb = lay(f, z, kx, a.a_fstride, a.g.ntiles), ss = a.g.Kxp * (int)a.a_fstride;
@@ -911,9 +901,9 @@ struct KY1 {
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
     C* b0 = reinterpret_cast<C*>(sm);
     const int r = tid / LINES, li = tid % LINES;
-    const long long tile = bid % a.tiles;
-    const long long pz = bid / a.tiles;
-    const long long f = pz / a.g.Nz, z = pz % a.g.Nz;
+    const long long tile = qmod(bid, a.tiles);
+    const long long pz = qdiv(bid, a.tiles);
+    const long long f = qdiv(pz, a.g.Nz), z = qmod(pz, a.g.Nz);
     const int kx = (int)(tile * LINES + li);
     const bool valid = kx < a.g.Kx;
     if constexpr (P == 0) {
@@ -1028,13 +1018,14 @@ struct KXPass {
       if (g < L2) {
         const int f = q / 2, type = q % 2;
         const C* A = (type == 0 ? a.V : a.DY);
-        const long long z = row / a.Ny, yb = (row % a.Ny) * a.Kxp;
+        const int fs = (int)a.ntiles * a.Nz * TL;
+        const int xb = xbase(a, row);
 #pragma unroll
         for (int j = 0; j < L1; ++j) {
           const int k = g + L2 * j;
           const bool up = k > Nx / 2;
           const int kk = up ? Nx - k : k;
-          const long long o = lay(f, z, yb + kk, a.Nz, a.ntiles);
+          const int o = xb + f * fs + xoff(a, kk);
           C av = A[o], bv;
           if (type == 0) {
             const T kx = a.kxo[kk];
@@ -1097,14 +1088,15 @@ struct KXPass {
         // O = FFT(N_f[2m+1]) (length Nx/2, read off Z_f by its Hermitian
         // parts), X_k = E_k + e^{-2 pi i k/Nx} O_k, k = 0..Nx/2
         constexpr int H = Nx / 2;
-        const long long z = row / a.Ny, yb = (row % a.Ny) * a.Kxp;
+        const int fs = (int)a.ntiles * a.Nz * TL;
+        const int xb = xbase(a, row);
         for (int i = tid; i < NF * (H + 1); i += THREADS) {
           const int f = i / (H + 1), k = i % (H + 1);
           const C* Zn = Zb + (NF + f) * RE::BUF;
           const C zk = Zn[k % H], zm = Zn[(H - k) % H];
           const C Ev = mk<T>((zk.x + zm.x) * T(0.5), (zk.y - zm.y) * T(0.5));
           const C Ov = mk<T>((zk.y + zm.y) * T(0.5), (zm.x - zk.x) * T(0.5));
-          a.NL[lay(f, z, yb + k, a.Nz, a.ntiles)] = cadd(Ev, cmul(a.twh[Nx + k], Ov));
+          a.NL[xb + f * fs + xoff(a, k)] = cadd(Ev, cmul(a.twh[Nx + k], Ov));
         }
       }
     } else {
@@ -1128,7 +1120,7 @@ struct KXPass {
           for (int k2 = 0; k2 < L2; ++k2) Zn[g + L1 * k2] = R.u[k2];
         }
       } else if constexpr (P == 7) {
-        const long long z = row / a.Ny, yb = (row % a.Ny) * a.Kxp;
+        const int fs = (int)a.ntiles * a.Nz * TL, xb = xbase(a, row);
         for (int i = tid; i < NFWD * (Nx / 2 + 1); i += THREADS) {
           const int qq = i / (Nx / 2 + 1), k = i % (Nx / 2 + 1);
           const C* Zn = Zb + (NFWD + qq) * RE::BUF;
@@ -1136,8 +1128,8 @@ struct KXPass {
           // A = (Z_k + conj Z_{N-k}) / 2,  B = (Z_k - conj Z_{N-k}) / (2i)
           const C Av = mk<T>((zk.x + zm.x) * T(0.5), (zk.y - zm.y) * T(0.5));
           const C Bv = mk<T>((zk.y + zm.y) * T(0.5), (zm.x - zk.x) * T(0.5));
-          a.NL[lay(2 * qq, z, yb + k, a.Nz, a.ntiles)] = Av;
-          if (2 * qq + 1 < NF) a.NL[lay(2 * qq + 1, z, yb + k, a.Nz, a.ntiles)] = Bv;
+          a.NL[xb + 2 * qq * fs + xoff(a, k)] = Av;
+          if (2 * qq + 1 < NF) a.NL[xb + (2 * qq + 1) * fs + xoff(a, k)] = Bv;
         }
       }
     }
@@ -1163,10 +1155,10 @@ struct KXRow {
   struct Regs { C v[L1]; C u[L2]; };
   static constexpr size_t smem_bytes = sizeof(C) * RE::BUF * JOBS * 2;
 
-  // element k of row R (rows ordered [f][z][y]) in the tiled layout
-  static FC_HD long long sidx(const Args& a, long long R, long long k) {
-    const long long y = R % a.Ny, fz = R / a.Ny;
-    return lay(fz / a.Nz, fz % a.Nz, y * a.Kxp + k, a.Nz, a.ntiles);
+  // element 0 of row R (rows ordered [f][z][y]) in the tiled layout; element k is xoff(a, k) further
+  static FC_HD int sbase(const Args& a, long long R) {
+    const int y = qmod(R, a.Ny), fz = qdiv(R, a.Ny);
+    return lay(qdiv(fz, a.Nz), qmod(fz, a.Nz), (long long)y * a.Kxp, a.Nz, a.ntiles);
   }
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& Rg) {
@@ -1194,23 +1186,28 @@ struct KXRow {
           for (int k2 = 0; k2 < L2; ++k2) Zn[g + L1 * k2] = Rg.u[k2];
         }
       } else {
-        if (valid)
+        if (valid) {
+          C* s0 = a.S + sbase(a, 2 * pair);
+          C* s1 = a.S + sbase(a, 2 * pair + 1);
           for (int k = g; k <= Nx / 2; k += G) {
             const C zk = Zn[k], zm = Zn[(Nx - k) % Nx];
-            a.S[sidx(a, 2 * pair, k)] = mk<T>((zk.x + zm.x) * T(0.5), (zk.y - zm.y) * T(0.5));
-            a.S[sidx(a, 2 * pair + 1, k)] = mk<T>((zk.y + zm.y) * T(0.5), (zm.x - zk.x) * T(0.5));
+            s0[xoff(a, k)] = mk<T>((zk.x + zm.x) * T(0.5), (zk.y - zm.y) * T(0.5));
+            s1[xoff(a, k)] = mk<T>((zk.y + zm.y) * T(0.5), (zm.x - zk.x) * T(0.5));
           }
+        }
       }
     } else {
       if constexpr (P == 0) {
         if (g < L2) {
+          const C* s0 = a.S + (valid ? sbase(a, 2 * pair) : 0);
+          const C* s1 = a.S + (valid ? sbase(a, 2 * pair + 1) : 0);
 #pragma unroll
           for (int j = 0; j < L1; ++j) {
             const int k = g + L2 * j;
             const bool up = k > Nx / 2;
             const int kk = up ? Nx - k : k;
-            C av = valid ? a.S[sidx(a, 2 * pair, kk)] : mk<T>(0, 0);
-            C bv = valid ? a.S[sidx(a, 2 * pair + 1, kk)] : mk<T>(0, 0);
+            C av = valid ? s0[xoff(a, kk)] : mk<T>(0, 0);
+            C bv = valid ? s1[xoff(a, kk)] : mk<T>(0, 0);
             if (kk == 0 || kk == Nx / 2) { av.y = T(0); bv.y = T(0); }
             if (up) { av.y = -av.y; bv.y = -bv.y; }
             Rg.v[j] = mk<T>(av.x - bv.y, av.y + bv.x);
@@ -1273,7 +1270,7 @@ struct KDiag {
       const int li = tid % TL, zr = tid / TL;           // 16 lines x 16 z rows per pass
       const long long line = bid * TL + li;
       const int Nz = a.g.Nz, Np = a.g.Np;
-      const int kx = (int)(line % a.g.Kxp), ky = (int)(line / a.g.Kxp);
+      const int kx = (int)(qmod(line, a.g.Kxp)), ky = (int)(qdiv(line, a.g.Kxp));
       if (line < a.g.lines && kx < a.g.Kx) {
         const double wgt = (kx == 0 || 2 * kx == a.Nx) ? 1.0 : 2.0;
         const double kxo = (double)a.t.kxo[kx], kyo = (double)a.t.kyo[ky];
@@ -1465,12 +1462,12 @@ struct KInterp {
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char*, int tid, long long bid, Regs&) {
     const int li = tid & 15, sl = tid >> 4;
-    const long long tile = (bid / a.sblocks) % a.ntiles2;
-    const int f = (int)(bid / a.sblocks / a.ntiles2);
-    const int s = (int)(bid % a.sblocks) * 16 + sl;
+    const long long tile = qmod(qdiv(bid, a.sblocks), a.ntiles2);
+    const int f = (int)(qdiv(qdiv(bid, a.sblocks), a.ntiles2));
+    const int s = (int)(qmod(bid, a.sblocks)) * 16 + sl;
     if (s >= a.Nz2) return;
     const long long line2 = tile * TL + li;
-    const int kx2 = (int)(line2 % a.Kxp2), ky2 = (int)(line2 / a.Kxp2);
+    const int kx2 = (int)(qmod(line2, a.Kxp2)), ky2 = (int)(qdiv(line2, a.Kxp2));
     C acc = mk<T>(0, 0);
     // source line and weight of this destination mode (none: zero)
     int kx1 = -1, ky1 = -1;
@@ -1529,14 +1526,14 @@ struct KProf {
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
     double* red = reinterpret_cast<double*>(sm);
     double* bins = red + THREADS;
-    const int f = (int)(bid / a.g.Nz), s = (int)(bid % a.g.Nz);
+    const int f = (int)(qdiv(bid, a.g.Nz)), s = (int)(qmod(bid, a.g.Nz));
     double* o = a.out + ((long long)f * a.g.Nz + s) * (2 + a.nshell);
     if constexpr (P == 0) {
       for (int j = tid; j < a.nshell; j += THREADS) bins[j] = 0.0;
     } else if constexpr (P == 1) {
       R.s = 0.0;
       for (long long l = tid; l < a.g.lines; l += THREADS) {
-        const int kx = (int)(l % a.g.Kxp), ky = (int)(l / a.g.Kxp);
+        const int kx = qmod(l, a.g.Kxp), ky = qdiv(l, a.g.Kxp);
         if (kx >= a.g.Kx) continue;
         const C v = a.X[lay(f, s, l, a.g.Np, a.g.ntiles)];
         if (kx == 0 && ky == 0) {
@@ -1631,7 +1628,7 @@ struct KFinite {
       R.n = 0;
       const int li = tid % TL, zr = tid / TL;
       const long long line = bid * TL + li;
-      if (line < a.g.lines && (int)(line % a.g.Kxp) < a.g.Kx)
+      if (line < a.g.lines && (int)(qmod(line, a.g.Kxp)) < a.g.Kx)
         for (int f = 0; f < a.g.nf; ++f) {
           const C* x = a.X + lay(f, 0, line, a.g.Np, a.g.ntiles);
           for (int z = zr; z < a.g.Np; z += THREADS / TL) {
