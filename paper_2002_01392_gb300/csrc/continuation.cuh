@@ -62,6 +62,8 @@ FC_HD cx<T> continuation_value(int jj, const cx<T>* first, const cx<T>* last, in
 // per thread and turn, whatever thread holds those rows otherwise (where each
 // thread continued the rows it holds, a few lanes of every warp did all the
 // sums, twice: the stage combine of 256^2 x 257 x 4 went 734 -> 675 us).
+// A thread's items are all of line li = tid % LINES (THREADS is a multiple of
+// LINES), so a thread of an absent or unused line may leave the call out.
 // Ev: [LINES][stride] with the first d values, then (at DMAX) the last d.
 template <class T, int LINES, int THREADS, class F>
 FC_HD void continue_lines(int tid, const cx<T>* Ev, int stride, int d, int Cc, const double* Ms, const float2* Ms2, F&& f) {

@@ -454,23 +454,26 @@ struct NsCore {
   }
 
   template <class T, int SIGN, int A1, int B1, int LN>
-  fc_status y_one_run(const cx<T>* IN, long long in_fs, cx<T>* OUT, long long out_fs, int nf, double scale, void* st) {
+  fc_status y_one_run(const cx<T>* IN, long long in_fs, cx<T>* OUT, long long out_fs, int nf, double scale, void* st,
+                      int cols) {
     using K = KY1<T, A1, B1, LN, SIGN>;
     typename K::Args a;
     a.g = ygeom(); a.tw = at<cx<T>>(l.twy);
     a.IN = IN; a.in_fstride = in_fs; a.OUT = OUT; a.out_fstride = out_fs;
-    a.tiles = (l.Kx + LN - 1) / LN;
+    a.tiles = (cols + LN - 1) / LN;
     a.scale = (T)scale;
     return bk.template run<K>(a, a.tiles * nf * p.Nz, st);
   }
   template <class T, int SIGN>
-  fc_status y_one(const cx<T>* IN, long long in_fs, cx<T>* OUT, long long out_fs, int nf, double scale, void* st) {
+  fc_status y_one(const cx<T>* IN, long long in_fs, cx<T>* OUT, long long out_fs, int nf, double scale, void* st,
+                  int cols = 0) {
     fc_status s = FC_ERR_UNSUPPORTED;
+    if (!cols) cols = l.Kx;   // columns kx to transform
 #define FC_Y1(NN, A1, B1)                                                                              \
   if (p.Ny == NN) {                                                                                   \
     constexpr int LN = y_lines<T, NN>();                                                              \
-    s = tile[TK_Y1] ? y_one_run<T, SIGN, A1, B1, y_lines_alt<T, NN>()>(IN, in_fs, OUT, out_fs, nf, scale, st) \
-                    : y_one_run<T, SIGN, A1, B1, LN>(IN, in_fs, OUT, out_fs, nf, scale, st);          \
+    s = tile[TK_Y1] ? y_one_run<T, SIGN, A1, B1, y_lines_alt<T, NN>()>(IN, in_fs, OUT, out_fs, nf, scale, st, cols) \
+                    : y_one_run<T, SIGN, A1, B1, LN>(IN, in_fs, OUT, out_fs, nf, scale, st, cols);    \
   }
     FC_XYSHAPES(FC_Y1)
 #undef FC_Y1
@@ -499,7 +502,7 @@ struct NsCore {
   fc_status x_pass_run(long long rows, void* st) {
     if (K::smem_bytes > 227 * 1024) return FC_ERR_UNSUPPORTED;
     typename K::Args a;
-    a.Kx = l.Kx; a.Kxp = l.Kxp; a.Ny = p.Ny; a.Nz = p.Nz; a.rows = rows; a.ntiles = l.ntiles;
+    a.Kx = l.Kx; a.Kxp = l.Kxp; a.Ny = p.Ny; a.Nz = p.Nz; a.Kw = kx_written(); a.rows = rows; a.ntiles = l.ntiles;
     a.tw = at<cx<T>>(l.twx); a.twh = at<cx<T>>(l.twxh); a.kxo = at<T>(l.tkxo);
     a.V = at<cx<T>>(l.V); a.DY = at<cx<T>>(l.DY); a.DZ = at<cx<T>>(l.DZ); a.NL = at<cx<T>>(l.NL);
     a.forcing = (T)p.forcing_x; a.gamma = (T)p.gamma; a.scale = (T)(1.0 / p.Nx);
@@ -546,13 +549,18 @@ struct NsCore {
     return s;
   }
 
+  // columns kx of the nonlinear term that the stage combine reads (all but those of the 2/3 mask), and the same rounded
+  // up to whole tiles, which is what the x pass writes and the y forward transform covers at most
+  int kx_active() const { return p.filter == 1 ? std::min(l.Kx, p.Nx / 3 + 1) : l.Kx; }
+  int kx_written() const { return std::min(l.Kx, (kx_active() + TL - 1) / TL * TL); }
+
   // nonlinear term of the state Xj into NL (mixed, filtered later); DZZ filled
   template <class T>
   fc_status nonlinear(const cx<T>* Xj, void* st) {
     fc_status s = z_deriv<T>(Xj, l.nf, st);
     if (!s) s = y_inv3<T>(Xj, l.Np, l.nf, st);
     if (!s) s = x_pass<T>(st);
-    if (!s) s = y_one<T, -1>(buf<T>(l.NL), p.Nz, buf<T>(l.NL), p.Nz, l.nf, 1.0, st);
+    if (!s) s = y_one<T, -1>(buf<T>(l.NL), p.Nz, buf<T>(l.NL), p.Nz, l.nf, 1.0, st, kx_active());
     return s;
   }
 
@@ -717,7 +725,7 @@ struct NsCore {
         case TK_ZC: return z_combine<T>(buf<T>(l.NL), Xb<T>(cur), Xb<T>(cur), Xo, 0.0, 0, l.nf, st);
         case TK_ZP: return z_project<T>(Xs, 1.0, st);
         case TK_YI: return y_inv3<T>(Xb<T>(cur), l.Np, l.nf, st);
-        default: return y_one<T, -1>(buf<T>(l.NL), p.Nz, buf<T>(l.NL), p.Nz, l.nf, 1.0, st);
+        default: return y_one<T, -1>(buf<T>(l.NL), p.Nz, buf<T>(l.NL), p.Nz, l.nf, 1.0, st, kx_active());
       }
     };
     std::array<int, TK_N> pick{};

@@ -252,6 +252,11 @@ struct KZCombine {
     const bool valid = line < a.g.lines && (qmod(line, a.g.Kxp)) < a.g.Kx;
     const int Nz = a.g.Nz, Np = a.g.Np, d = a.g.d;
     const long long Ls = a.g.lines;
+    // x, y factor of the nonlinear term.  Where it is 0 (with the 2/3 mask, 5/9 of the lines) the term is not read, not
+    // filtered and not added
+    const int kx = valid ? qmod(line, a.g.Kxp) : 0, ky = valid ? qdiv(line, a.g.Kxp) : 0;
+    const T fxy = valid ? a.t.fx[kx] * a.t.fy[ky] : T(0);
+    const bool act = fxy != T(0);
     if constexpr (P == 0) {
       load_mr<T>(sm + off_M, a.t, a.g.Cc * d, tid, THREADS);
       if (r < L2) {
@@ -264,7 +269,7 @@ struct KZCombine {
             R.v[j] = val;
             continue;
           }
-          if (valid && n < Nz) val = x[n * TL];
+          if (act && n < Nz) val = x[n * TL];
           R.v[j] = val;
           if (n < d) Ev[n] = val;
           if (n >= Nz - d && n < Nz) Ev[DMAX + n - (Nz - d)] = val;
@@ -279,15 +284,17 @@ struct KZCombine {
         }
         if (a.pf > 0 && bid + a.pf < a.nblocks) {
           const long long b2 = bid + a.pf, line2 = (qmod(b2, a.tiles)) * LINES + li;
-          if (line2 < a.g.lines && (qmod(line2, a.g.Kxp)) < a.g.Kx)
+          if (line2 < a.g.lines && (qmod(line2, a.g.Kxp)) < a.g.Kx &&
+              a.t.fx[qmod(line2, a.g.Kxp)] * a.t.fy[qdiv(line2, a.g.Kxp)] != T(0))
             prefetch_line<C, JN>(a.NL, qdiv(b2, a.tiles), line2, Nz, Nz, a.g.ntiles, r, L2, li);
         }
       }
     } else if constexpr (P == 1) {
-      continue_lines<T, LINES, THREADS>(tid, E0, 2 * DMAX, d, a.g.Cc, Ms, Ms2,
-                                        [&](int jj, int l, C v) { Cv[jj * LINES + l] = v; });
+      if (act)
+        continue_lines<T, LINES, THREADS>(tid, E0, 2 * DMAX, d, a.g.Cc, Ms, Ms2,
+                                          [&](int jj, int l, C v) { Cv[jj * LINES + l] = v; });
     } else if constexpr (P == 2) {
-      if (r < L2) {
+      if (r < L2 && act) {
 #pragma unroll
         for (int j = 0; j < JN; ++j) {
           const int n = r + L2 * j;
@@ -296,16 +303,14 @@ struct KZCombine {
         E::template A<-1>(R.v, b0, a.t.tw, r, li);
       }
     } else if constexpr (P == 3) {
-      if (r < L1) {
+      if (r < L1 && act) {
         E::template B<-1>(R.u, b0, r, li);
         E::mulH_real(R.u, a.t.Hf, r);   // even filter kernel: real spectrum
         E::template Bi<1>(R.u, b0, a.t.tw, r, li);
       }
     } else if constexpr (P == 4) {
       if (r < L2) {
-        E::template Ai<1>(R.v, b0, r, li);
-        const int kx = (int)(qmod(line, a.g.Kxp)), ky = (int)(qdiv(line, a.g.Kxp));
-        const T fxy = valid ? a.t.fx[kx] * a.t.fy[ky] : T(0);
+        if (act) E::template Ai<1>(R.v, b0, r, li);
         const T ckp2 = valid ? a.t.kx[kx] * a.t.kx[kx] + a.t.ky[ky] * a.t.ky[ky] : T(0);
         const T cdt = (T)a.dtj, cnu = (T)(a.dif[f]);
         const long long fo = lay(f, 0, line, Np, a.g.ntiles);
@@ -321,7 +326,7 @@ struct KZCombine {
             if (valid) {
               const C vj = xj[n * TL];
               const C zz = dzz[n * TL];
-              const C nlf = cscale(R.v[j], fxy);
+              const C nlf = act ? cscale(R.v[j], fxy) : mk<T>(0, 0);
               const C visc = csub(zz, cscale(vj, ckp2));
               const C base = a.Xt ? xt[n * TL] : mk<T>(0, 0);
               vs = cadd(base, cscale(cadd(nlf, cscale(visc, cnu)), cdt));
@@ -342,11 +347,10 @@ struct KZCombine {
         }
       }
     } else if constexpr (P == 5) {
-      const long long line0 = (qmod(bid, a.tiles)) * LINES;
-      continue_lines<T, LINES, THREADS>(tid, E0, 2 * DMAX, d, a.g.Cc, Ms, Ms2, [&](int jj, int l, C v) {
-        const long long ln = line0 + l;
-        if (ln < a.g.lines && (qmod(ln, a.g.Kxp)) < a.g.Kx) a.Xout[lay(f, Nz + jj, ln, Np, a.g.ntiles)] = v;
-      });
+      C* xo = a.Xout + lay(f, Nz, line, Np, a.g.ntiles);
+      if (valid)
+        continue_lines<T, LINES, THREADS>(tid, E0, 2 * DMAX, d, a.g.Cc, Ms, Ms2,
+                                          [&](int jj, int, C v) { xo[jj * TL] = v; });
     }
   }
   static FC_HD int li_of(int tid) { return tid % LINES; }
@@ -651,26 +655,22 @@ struct KZProject {
         Ev[2 * DMAX + (q < d ? q : DMAX + (q - d))] = dph;
       }
     } else if constexpr (P == 6) {  // X -= grad phi^I + FC(grad phi^H); wall planes
-      // row n of line ln (wave numbers kx, ky): subtract the gradient of sigma and Phi, Phi' = ph, dph
-      auto update = [&](int n, long long ln, int l, T kx, T ky, C ph, C dph) {
-        C* q0 = SG ? reinterpret_cast<C*>(sm + off_G) + l : a.G0 + lay(0, 0, ln, Np, a.g.ntiles);
-        C* q1 = SG ? reinterpret_cast<C*>(sm + off_G) + LINES * NPC + l : a.G1 + lay(0, 0, ln, Np, a.g.ntiles);
-        const C sg = q1[n * GS], sz = q0[n * GS];
+      // row n of the thread's line: subtract the gradient of sigma and Phi, Phi' = ph, dph
+      auto update = [&](int n, C ph, C dph) {
+        const int o = n * TL;
+        const C sg = g1[n * GS], sz = g0[n * GS];
         // i k Phi = (-k Phi.y, k Phi.x)
-        const C gx = cadd(cscale(sg, kx), mk<T>(-kx * ph.y, kx * ph.x));
-        const C gy = cadd(cscale(sg, ky), mk<T>(-ky * ph.y, ky * ph.x));
+        const C gx = cadd(cscale(sg, kxo), mk<T>(-kxo * ph.y, kxo * ph.x));
+        const C gy = cadd(cscale(sg, kyo), mk<T>(-kyo * ph.y, kyo * ph.x));
         const C gz = cadd(sz, dph);
-        C* u = a.X + lay(0, n, ln, Np, a.g.ntiles);
-        C* v = a.X + lay(1, n, ln, Np, a.g.ntiles);
-        C* w = a.X + lay(2, n, ln, Np, a.g.ntiles);
-        *u = csub(*u, gx);
-        *v = csub(*v, gy);
-        *w = csub(*w, gz);
+        xu[o] = csub(xu[o], gx);
+        xv[o] = csub(xv[o], gy);
+        xw[o] = csub(xw[o], gz);
         if (n == 0 || n == Nz - 1) {
           const int wall = (n == 0) ? 0 : 1;
           const double s = 1.0 / a.dtj;
-          a.gradp[((long long)wall * 2 + 0) * Ls + ln] = make_double2((double)gx.x * s, (double)gx.y * s);
-          a.gradp[((long long)wall * 2 + 1) * Ls + ln] = make_double2((double)gy.x * s, (double)gy.y * s);
+          a.gradp[((long long)wall * 2 + 0) * Ls + line] = make_double2((double)gx.x * s, (double)gx.y * s);
+          a.gradp[((long long)wall * 2 + 1) * Ls + line] = make_double2((double)gy.x * s, (double)gy.y * s);
         }
       };
       if (r < L2 && valid) {
@@ -682,21 +682,15 @@ struct KZProject {
           if (n < Nz) {
             C ph, dph;
             phi_at(cf, kxo, kyo, tdz, tLz, n, &ph, &dph);
-            update(n, line, li, kxo, kyo, ph, dph);
+            update(n, ph, dph);
           }
         }
       }
-      // the continuation rows, spread over all threads
-      const C* E0 = reinterpret_cast<const C*>(sm + off_E);
-      for (int i = tid; i < a.g.Cc * LINES; i += THREADS) {
-        const int jj = i / LINES, l = i % LINES;
-        const long long ln = bid * LINES + l;
-        if (ln >= a.g.lines || (qmod(ln, a.g.Kxp)) >= a.g.Kx) continue;
-        const C* e = E0 + l * 4 * DMAX;
-        const C ph = continuation_value<T>(jj, e, e + DMAX, d, a.g.Cc, Ms, Ms2);
-        const C dph = continuation_value<T>(jj, e + 2 * DMAX, e + 3 * DMAX, d, a.g.Cc, Ms, Ms2);
-        update(Nz + jj, ln, l, a.t.kxo[qmod(ln, a.g.Kxp)], a.t.kyo[qdiv(ln, a.g.Kxp)], ph, dph);
-      }
+      // the continuation rows, spread over all threads (a thread's items are of its own line)
+      if (valid)
+        for (int jj = r; jj < a.g.Cc; jj += E::G)
+          update(Nz + jj, continuation_value<T>(jj, Ev, Ev + DMAX, d, a.g.Cc, Ms, Ms2),
+                 continuation_value<T>(jj, Ev + 2 * DMAX, Ev + 3 * DMAX, d, a.g.Cc, Ms, Ms2));
     }
   }
 
@@ -993,6 +987,7 @@ struct KXPass {
   static constexpr int THREADS = NJOB * G, NPHASE = 8, MINB = 2;
   struct Args {
     int Kx, Kxp, Ny, Nz;
+    int Kw;                  // columns of NL that are used later (the rest is not written)
     long long rows;          // Nz * Ny
     long long ntiles;
     const C* tw;             // Nx engine twiddles
@@ -1096,7 +1091,7 @@ struct KXPass {
           const C zk = Zn[k % H], zm = Zn[(H - k) % H];
           const C Ev = mk<T>((zk.x + zm.x) * T(0.5), (zk.y - zm.y) * T(0.5));
           const C Ov = mk<T>((zk.y + zm.y) * T(0.5), (zm.x - zk.x) * T(0.5));
-          a.NL[xb + f * fs + xoff(a, k)] = cadd(Ev, cmul(a.twh[Nx + k], Ov));
+          if (k < a.Kw) a.NL[xb + f * fs + xoff(a, k)] = cadd(Ev, cmul(a.twh[Nx + k], Ov));
         }
       }
     } else {
@@ -1123,6 +1118,7 @@ struct KXPass {
         const int fs = (int)a.ntiles * a.Nz * TL, xb = xbase(a, row);
         for (int i = tid; i < NFWD * (Nx / 2 + 1); i += THREADS) {
           const int qq = i / (Nx / 2 + 1), k = i % (Nx / 2 + 1);
+          if (k >= a.Kw) continue;
           const C* Zn = Zb + (NFWD + qq) * RE::BUF;
           const C zk = Zn[k], zm = Zn[(Nx - k) % Nx];
           // A = (Z_k + conj Z_{N-k}) / 2,  B = (Z_k - conj Z_{N-k}) / (2i)
