@@ -15,6 +15,7 @@ FC_ZSHAPES_PADDED(FC_INST_Z)
 #undef FC_INST_Z
 template struct DevRun<KZContinue<double, 8>>;
 template struct DevRun<KDiag<double>>;
+template struct DevRun<KHom<double>>;
 template struct DevRun<KMeanLine<double>>;
 template struct DevRun<KMeanInit<double>>;
 template struct DevRun<KInterp<double>>;

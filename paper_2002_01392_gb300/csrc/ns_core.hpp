@@ -34,6 +34,7 @@ struct NsLayout {
   int nmean;
   size_t kxo, kyo, kzo, kx, ky, fx, fy, Mr, Mr2, twz, twz2, H1, H2, Hf, chirp, Hbf, Hbi, twx, twy, twxh;
   int L1alt;      // first-pass factor of the alternative z schedule (0: none)
+  size_t hom;     // line constants of the homogeneous pressure
   size_t tkxo, tkyo, tkzo, tkx, tky, tfx, tfy;   // copies in the simulation's precision
   size_t total;
 #if FC_LAYOUT_GUARD
@@ -83,8 +84,8 @@ inline fc_status ns_layout(const ns_params& p, NsLayout* o) {
   l.plines = l.ntiles * TL;
   l.es = p.prec == FC_F32 ? 4 : 8;
   if (!z_shape_for(l.Np, p.Nz, &l.L, &l.L1, &l.L2, &l.zdirect)) return FC_ERR_UNSUPPORTED;
-  // the float64 mean-line kernel keeps two continued lines in shared memory
-  if (l.Np > KMean<float>::NPMAX) return FC_ERR_UNSUPPORTED;
+  // the float64 mean-line kernel keeps a continued line in shared memory
+  if (l.Np > KMeanLine<float>::NPMAX) return FC_ERR_UNSUPPORTED;
   l.L1alt = 0;
 #define FC_ZALT(LL, A, B) \
   if (!l.zdirect && LL == l.L && p.prec == FC_F32) l.L1alt = A;
@@ -127,6 +128,7 @@ inline fc_status ns_layout(const ns_params& p, NsLayout* o) {
   l.chirp = take(cs * l.Np); l.Hbf = take(cs * l.L); l.Hbi = take(cs * l.L);
   l.twx = take(cs * 2 * p.Nx); l.twy = take(cs * 2 * p.Ny);
   l.twxh = take(cs * (p.Nx + p.Nx / 2 + 1));
+  l.hom = take(16 * (size_t)l.lines);
   l.total = off;
   // every array is indexed with 32-bit element offsets
   if ((double)l.nf * l.Np * l.plines >= 2147483647.0) return FC_ERR_UNSUPPORTED;
@@ -238,6 +240,12 @@ struct NsCore {
     if (!s) s = putc(l.twy, twy);
     if (!s) s = put(l.d2r, d2r.data(), 8 * d2r.size());
     if (!s) s = put(l.hfr, hfr.data(), 8 * hfr.size());
+    if (!s) {
+      using K = KHom<double>;
+      typename K::Args a;
+      a.g = zgeom(l.nf); a.kxo = at<double>(l.kxo); a.kyo = at<double>(l.kyo); a.hom = at<double2>(l.hom);
+      s = bk.template run<K>(a, (l.lines + K::THREADS - 1) / K::THREADS, nullptr);
+    }
     if (!s) s = bk.memset(ws + l.X64[0], 0, 3 * 16 * (size_t)l.nmean * l.Np, nullptr);
     if (!s) s = bk.memset(ws + l.gradp, 0, sizeof(double) * 8 * l.lines, nullptr);
     if (!s) s = bk.memset(ws + l.nfin, 0, sizeof(unsigned long long), nullptr);
@@ -274,7 +282,7 @@ struct NsCore {
     t.chirp = at<cx<T>>(l.chirp); t.Hbf = at<cx<T>>(l.Hbf); t.Hbi = at<cx<T>>(l.Hbi);
     t.kxo = at<T>(l.tkxo); t.kyo = at<T>(l.tkyo); t.kzo = at<T>(l.tkzo);
     t.kx = at<T>(l.tkx); t.ky = at<T>(l.tky); t.fx = at<T>(l.tfx); t.fy = at<T>(l.tfy);
-    t.kxo_d = at<double>(l.kxo); t.kyo_d = at<double>(l.kyo);
+    t.hom = at<double2>(l.hom);
     return t;
   }
   ZGeom zgeom(int nf) const {
@@ -588,7 +596,8 @@ struct NsCore {
     a.fxy00 = 1.0;   // x, y filter / mask factor of the (0, 0) mode in both filter modes
     mean_fmap<T>(a.fmap);
     a.nmean = l.nmean;
-    return bk.template run<K>(a, l.nmean, st);
+    a.nzb = (p.Nz + K::ZB - 1) / K::ZB + 1;
+    return bk.template run<K>(a, (long long)l.nmean * a.nzb, st);
   }
   fc_status mean_init_any(void* st) { return f32() ? mean_init<float>(cur, st) : FC_OK; }
 

@@ -43,8 +43,7 @@ struct ZTab {
   const T* ky;          // ky (Ny)
   const T* fx;          // x filter / mask factor (Kx)
   const T* fy;          // y filter / mask factor (Ny)
-  const double* kxo_d;  // float64 copies for the homogeneous-pressure coefficients
-  const double* kyo_d;
+  const double2* hom;   // per line: e^{-g Lz} and 1 / (g (1 - e^{-2 g Lz})), g = |k_perp| (second 0 where g = 0; see KHom)
 };
 
 struct ZGeom {
@@ -111,6 +110,23 @@ FC_HD void load_mr(unsigned char* sm, const ZTab<T>& t, int n, int tid, int thre
   }
 }
 
+// Blocks per SM that the registers of a z kernel are bounded for.  These kernels
+// wait for memory and barriers rather than for issue slots, so the float32 ones
+// whose register transforms are short (up to 24 values) get 100 registers a
+// thread and as many blocks as the shared memory then allows (256^2 x 257 x 4:
+// stage combine 588 -> 424 us, and with the changes at PhiLine and KHom the
+// projection 679 -> 489 us; before, 168 registers and 12 warps per SM; the z
+// derivatives, 357 us, gain nothing).  Longer transforms (30 to 48 values) spill
+// below 128 registers.
+template <class T>
+constexpr int z_min_blocks(int L1, int L2, int threads, size_t smem) {
+  const int base = threads <= 160 ? 3 : (threads <= 320 ? 2 : 1);
+  if (sizeof(T) != 4 || L1 > 24 || L2 > 24) return base;
+  const int regs = 65536 / (100 * threads), room = (int)(224 * 1024 / (smem + 1024));
+  const int most = regs < room ? regs : room;
+  return most > base ? most : base;
+}
+
 // ===========================================================================
 // K1  zderiv: dz and dzz of the state at the Nz physical points.
 // Circular convolution of the extended line with the derivative kernels of
@@ -125,7 +141,6 @@ struct KZDeriv {
   using E = Eng<T, L1, L2, LINES>;
   using C = cx<T>;
   static constexpr int THREADS = E::THREADS, NPHASE = 3;
-  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
   struct Args {
     ZGeom g;
     ZTab<T> t;
@@ -139,6 +154,7 @@ struct KZDeriv {
   struct Regs { C v[L1]; C u[L2]; };
   static constexpr size_t off_b1 = sizeof(C) * E::BUF;
   static constexpr size_t smem_bytes = 2 * sizeof(C) * E::BUF;
+  static constexpr int MINB = z_min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
@@ -216,7 +232,6 @@ struct KZCombine {
   using E = Eng<T, L1, L2, LINES>;
   using C = cx<T>;
   static constexpr int THREADS = E::THREADS, NPHASE = 6;
-  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
   struct Args {
     ZGeom g;
     ZTab<T> t;
@@ -237,6 +252,7 @@ struct KZCombine {
   static constexpr size_t off_E = off_M + sizeof(double) * MRMAX;
   static constexpr size_t off_C = off_E + sizeof(C) * LINES * 2 * DMAX;   // continuation values [C][LINES]
   static constexpr size_t smem_bytes = off_C + sizeof(C) * LINES * CMAX;
+  static constexpr int MINB = z_min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
@@ -449,7 +465,6 @@ struct KZProject {
   static constexpr int THREADS = E::THREADS, NPHASE = 7;
   // phases 1..3 run four times (Y^, W^, sigma, sigma_z) from one copy of code
   static constexpr int LB = 1, LE = 4, NIT = 4;
-  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
   struct Args {
     ZGeom g;
     ZTab<T> t;
@@ -472,6 +487,7 @@ struct KZProject {
   static constexpr bool SG = sizeof(T) == 4 && sg_bytes <= 24 * 1024;
   static constexpr int GS = SG ? LINES : TL;   // element stride of a scratch line
   static constexpr size_t smem_bytes = off_G + (SG ? sg_bytes : 0);
+  static constexpr int MINB = z_min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   // conj(chirp[n]) (1 outside the line)
   static FC_HD C cchirp(const ZTab<T>& t, int n, int Np) {
@@ -625,23 +641,20 @@ struct KZProject {
         }
       }
     } else if constexpr (P == 4) {  // homogeneous coefficients (float64) -> W[8..12]
-      if (r == 0) {
+      if (r == 0 && valid) {
         const double br = W[0], bi = W[1], tr = W[2], ti = W[3];
         double Ar = 0, Aim = 0, Br = 0, Bim = 0, D = 0;
         // gamma = |k_perp| of the Nyquist-zeroed wavenumbers (the same ones as
         // the gradient i kx Phi, i ky Phi), so grad phi^H is divergence-free;
         // where it vanishes, phi^H = D z with D = (b + t)/2.
-        const double kxd = a.t.kxo_d[kxi], kyd = a.t.kyo_d[kyi];
-        if (kxd == 0.0 && kyd == 0.0) {
+        const double2 h = a.t.hom[line];
+        if (h.y == 0.0) {
           D = 0.5 * (br + tr);
         } else {
-          const double gam = sqrt(kxd * kxd + kyd * kyd);
-          const double Ee = exp(-gam * a.g.Lz);
-          const double den = gam * (1.0 - Ee * Ee);
-          Ar = (tr - br * Ee) / den;
-          Aim = (ti - bi * Ee) / den;
-          Br = -(br - tr * Ee) / den;
-          Bim = -(bi - ti * Ee) / den;
+          Ar = (tr - br * h.x) * h.y;
+          Aim = (ti - bi * h.x) * h.y;
+          Br = -(br - tr * h.x) * h.y;
+          Bim = -(bi - ti * h.x) * h.y;
         }
         W[8] = Ar; W[9] = Aim; W[10] = Br; W[11] = Bim; W[12] = D;
       }
@@ -649,8 +662,8 @@ struct KZProject {
       for (int q = r; q < 2 * d; q += E::G) {
         const int s = q < d ? q : Nz - 2 * d + q;
         C ph, dph;
-        const T cf[5] = {(T)W[8], (T)W[9], (T)W[10], (T)W[11], (T)W[12]};
-        phi_at(cf, kxo, kyo, (T)a.g.dz, (T)a.g.Lz, s, &ph, &dph);
+        const PhiLine pl(W, kxo, kyo, (T)a.g.dz, (T)a.g.Lz);
+        pl.at(s, &ph, &dph);
         Ev[q < d ? q : DMAX + (q - d)] = ph;
         Ev[2 * DMAX + (q < d ? q : DMAX + (q - d))] = dph;
       }
@@ -674,14 +687,13 @@ struct KZProject {
         }
       };
       if (r < L2 && valid) {
-        const T cf[5] = {(T)W[8], (T)W[9], (T)W[10], (T)W[11], (T)W[12]};
-        const T tdz = (T)a.g.dz, tLz = (T)a.g.Lz;
+        const PhiLine pl(W, kxo, kyo, (T)a.g.dz, (T)a.g.Lz);
 #pragma unroll
         for (int j = 0; j < JN; ++j) {
           const int n = r + L2 * j;
           if (n < Nz) {
             C ph, dph;
-            phi_at(cf, kxo, kyo, tdz, tLz, n, &ph, &dph);
+            pl.at(n, &ph, &dph);
             update(n, ph, dph);
           }
         }
@@ -694,28 +706,64 @@ struct KZProject {
     }
   }
 
-  // Phi and Phi' at physical point s from the float64 coefficients W[8..12]
-  // (evaluated in the path's precision)
-  static FC_NOINLINE void phi_at(const T* cf, T kxo, T kyo, T dz, T Lz, int s, C* ph, C* dph) {
-    if (kxo == T(0) && kyo == T(0)) {
-      *ph = mk<T>(0, 0);
-      *dph = mk<T>(cf[4], 0);
-      return;
+  // Phi and Phi' at the physical points of a line from the float64
+  // coefficients W[8..12], evaluated in the path's precision.  In registers
+  // (out of line, with its values through local memory, and with the float64
+  // exponential and divisions of every line in one warp of the CTA, the
+  // projection of 256^2 x 257 took 679 us, see KHom)
+  struct PhiLine {
+    T Ar, Ai, Br, Bi, D, gam, dz, Lz;
+    FC_HD PhiLine(const double* W, T kxo, T kyo, T dz_, T Lz_)
+        : Ar((T)W[8]), Ai((T)W[9]), Br((T)W[10]), Bi((T)W[11]), D((T)W[12]), dz(dz_), Lz(Lz_) {
+      if constexpr (sizeof(T) == 4) gam = sqrtf(kxo * kxo + kyo * kyo);
+      else gam = sqrt(kxo * kxo + kyo * kyo);
+      if (kxo == T(0) && kyo == T(0)) gam = T(-1);
     }
-    const T z = (T)s * dz;
-    T gam, e1, e2;
-    if constexpr (sizeof(T) == 4) {
-      gam = sqrtf(kxo * kxo + kyo * kyo);
-      e1 = expf(gam * (z - Lz));
-      e2 = expf(-gam * z);
-    } else {
-      gam = sqrt(kxo * kxo + kyo * kyo);
-      e1 = exp(gam * (z - Lz));
-      e2 = exp(-gam * z);
+    FC_HD void at(int s, C* ph, C* dph) const {
+      if (gam < T(0)) {   // mean mode: Phi = D z
+        *ph = mk<T>(0, 0);
+        *dph = mk<T>(D, 0);
+        return;
+      }
+      const T z = (T)s * dz;
+      const T e1 = ex(gam * (z - Lz)), e2 = ex(-gam * z);
+      *ph = mk<T>(Ar * e1 + Br * e2, Ai * e1 + Bi * e2);
+      *dph = mk<T>(gam * (Ar * e1 - Br * e2), gam * (Ai * e1 - Bi * e2));
     }
-    const T Ar = cf[0], Aim = cf[1], Br = cf[2], Bim = cf[3];
-    *ph = mk<T>(Ar * e1 + Br * e2, Aim * e1 + Bim * e2);
-    *dph = mk<T>(gam * (Ar * e1 - Br * e2), gam * (Aim * e1 - Bim * e2));
+    static FC_HD float ex(float x) { return expf(x); }
+    static FC_NOINLINE double ex(double x) { return exp(x); }
+  };
+};
+
+// ===========================================================================
+// KHom  the line constants of the homogeneous pressure (Eqs. A, B), float64,
+// once per simulation: e^{-g Lz} and 1 / (g (1 - e^{-2 g Lz})).
+// ===========================================================================
+template <class T>
+struct KHom {
+  static constexpr int THREADS = 128, NPHASE = 1, MINB = 1;
+  struct Args {
+    ZGeom g;
+    const double* kxo;   // Nyquist-zeroed wavenumbers
+    const double* kyo;
+    double2* hom;
+  };
+  struct Regs { int dummy; };
+  static constexpr size_t smem_bytes = 16;
+  template <int P>
+  static FC_HD void phase(const Args& a, unsigned char*, int tid, long long bid, Regs&) {
+    const long long line = bid * THREADS + tid;
+    if (line >= a.g.lines) return;
+    const int kx = qmod(line, a.g.Kxp), ky = qdiv(line, a.g.Kxp);
+    double2 h = make_double2(1.0, 0.0);
+    if (kx < a.g.Kx) {
+      const double x = a.kxo[kx], y = a.kyo[ky], gam = sqrt(x * x + y * y);
+      if (gam > 0.0) {
+        const double E = exp(-gam * a.g.Lz);
+        h = make_double2(E, 1.0 / (gam * (1.0 - E * E)));
+      }
+    }
+    a.hom[line] = h;
   }
 };
 
@@ -1319,15 +1367,23 @@ namespace fcns {
 // unchanged on that line) is redone in float64 from a float64 shadow of the
 // line:  v* = v^t + dt_j [ (f_z * FC(N))(z) + nu dzz v^{j-1} ]  (direct sums
 // with the float64 real-space kernels), wall injection, continuation, and
-// both the shadow and the float32 state line are written.  One block per
-// field; runs after the stage combine.
-// ===========================================================================
+// both the shadow and the float32 state line are written.  Runs after the
+// stage combine.
+//
+// The work is N' multiply-adds per output, but float64 ones: a single block per
+// field took 33 us at Nz = 65 and 377 us at 513 (one SM's float64 pipe), longer
+// than the stage's other kernels on small grids.  A block computes ZB outputs, 16
+// threads each, so that the sums spread over many SMs (22 and 34 us with cold
+// caches, of which the float64 continuation sums are most); every block
+// continues N for itself, and one more block per field recomputes the 2 d end
+// values and continues them, so that no block waits for another.
 template <class T>
-struct KMean {
+struct KMeanLine {
   using C = cx<T>;
-  // NPMAX: the longest continued line held in shared memory (two lines); it
-  // covers every compiled z length (N' <= 1536), and ns_layout refuses longer
-  static constexpr int THREADS = 256, NPHASE = 4, MINB = 1, NPMAX = 1536;
+  // NPMAX: the longest continued line held in shared memory; it covers every
+  // compiled z length (N' <= 1536), and ns_layout refuses longer
+  static constexpr int ZB = 8, SPLIT = 16, THREADS = ZB * SPLIT, NPHASE = 5, MINB = 1, NPMAX = 1536;
+  static constexpr int OMAX = 2 * DMAX;   // outputs of a block at most
   struct Args {
     ZGeom g;
     const double* Mr;       // C x d
@@ -1344,48 +1400,76 @@ struct KMean {
     double fxy00;
     int fmap[3];            // field index of shadow entry 0, 1, 2
     int nmean;              // 2 (Navier-Stokes: u, v) or 3 (Boussinesq: u, v, theta)
+    int nzb;                // blocks per field: ceil(Nz / ZB), and one for the ends
   };
   struct Regs { int dummy; };
-  static constexpr size_t smem_bytes = 2 * sizeof(double2) * NPMAX;
+  static constexpr size_t off_P = sizeof(double2) * NPMAX;
+  static constexpr size_t off_V = off_P + sizeof(double) * 4 * OMAX * SPLIT;
+  static constexpr size_t smem_bytes = off_V + sizeof(double2) * OMAX;
+
+  // continuation value jj from the first and last d values
+  static FC_HD double2 cont(const Args& a, const double2* first, const double2* last, int jj) {
+    const int d = a.g.d, Cc = a.g.Cc;
+    dd re{0.0, 0.0}, im{0.0, 0.0};
+    for (int i = 0; i < d; ++i) {
+      const double m1 = a.Mr[jj * d + i], m2 = a.Mr[(Cc - 1 - jj) * d + (d - 1 - i)];
+      dd_fma(re, m1, last[i].x);
+      dd_fma(im, m1, last[i].y);
+      dd_fma(re, m2, first[i].x);
+      dd_fma(im, m2, first[i].y);
+    }
+    return make_double2(dd_round(re), dd_round(im));
+  }
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs&) {
     double2* nl = reinterpret_cast<double2*>(sm);
-    double2* vs = nl + NPMAX;
-    const int e = (int)bid, f = a.fmap[e];
-    const int Nz = a.g.Nz, Np = a.g.Np, d = a.g.d, Cc = a.g.Cc;
+    double* part = reinterpret_cast<double*>(sm + off_P);   // [4][OMAX][SPLIT]
+    double2* vs = reinterpret_cast<double2*>(sm + off_V);
+    const int e = qdiv(bid, a.nzb), zb = qmod(bid, a.nzb), f = a.fmap[e];
+    const int Nz = a.g.Nz, Np = a.g.Np, d = a.g.d;
     const int jlo = -(Np - 1);
-    auto cont = [&](const double2* x, int jj) {
-      dd re{0.0, 0.0}, im{0.0, 0.0};
-      for (int i = 0; i < d; ++i) {
-        const double m1 = a.Mr[jj * d + i], m2 = a.Mr[(Cc - 1 - jj) * d + (d - 1 - i)];
-        dd_fma(re, m1, x[Nz - d + i].x);
-        dd_fma(im, m1, x[Nz - d + i].y);
-        dd_fma(re, m2, x[i].x);
-        dd_fma(im, m2, x[i].y);
-      }
-      return make_double2(dd_round(re), dd_round(im));
-    };
+    const bool ends = zb == a.nzb - 1;
+    const int nout = ends ? 2 * d : (Nz - zb * ZB < ZB ? Nz - zb * ZB : ZB);
+    // level of output o
+    auto level = [&](int o) { return ends ? (o < d ? o : Nz - 2 * d + o) : zb * ZB + o; };
     if constexpr (P == 0) {
       const C* src = a.NL + lay(f, 0, 0, Nz, a.g.ntiles);
       for (int z = tid; z < Nz; z += THREADS) nl[z] = make_double2((double)src[z * TL].x, (double)src[z * TL].y);
     } else if constexpr (P == 1) {
-      for (int z = Nz + tid; z < Np; z += THREADS) nl[z] = cont(nl, z - Nz);
+      for (int jj = tid; jj < a.g.Cc; jj += THREADS) nl[Nz + jj] = cont(a, nl, nl + Nz - d, jj);
     } else if constexpr (P == 2) {
-      const double2* xt = a.Xt + (long long)e * Np;
       const double2* xj = a.Xj + (long long)e * Np;
-      const double s2 = 1.0 / (a.g.dz * a.g.dz);
-      for (int z = tid; z < Nz; z += THREADS) {
+      const int t = tid % SPLIT;
+      for (int o = tid / SPLIT; o < nout; o += ZB) {
+        const int z = level(o);
         double fr = 0, fi = 0, zr = 0, zi = 0;
-        for (int m = 0; m < Np; ++m) {
+        for (int m = t; m < Np; m += SPLIT) {
           const double hk = a.hf[z - m - jlo], dk = a.d2[z - m - jlo];
           fr += hk * nl[m].x;
           fi += hk * nl[m].y;
           zr += dk * xj[m].x;
           zi += dk * xj[m].y;
         }
-        double2 v = make_double2(xt[z].x + a.dtj * (a.fxy00 * fr + a.dif[e] * zr * s2),
-                                 xt[z].y + a.dtj * (a.fxy00 * fi + a.dif[e] * zi * s2));
+        double* q = part + o * SPLIT + t;
+        q[0] = fr;
+        q[OMAX * SPLIT] = fi;
+        q[2 * OMAX * SPLIT] = zr;
+        q[3 * OMAX * SPLIT] = zi;
+      }
+    } else if constexpr (P == 3) {
+      for (int o = tid; o < nout; o += THREADS) {
+        const int z = level(o);
+        double sum[4];
+        for (int k = 0; k < 4; ++k) {
+          const double* q = part + k * OMAX * SPLIT + o * SPLIT;
+          sum[k] = 0;
+          for (int t = 0; t < SPLIT; ++t) sum[k] += q[t];
+        }
+        const double s2 = 1.0 / (a.g.dz * a.g.dz);
+        const double2 xt = a.Xt[(long long)e * Np + z];
+        double2 v = make_double2(xt.x + a.dtj * (a.fxy00 * sum[0] + a.dif[e] * sum[2] * s2),
+                                 xt.y + a.dtj * (a.fxy00 * sum[1] + a.dif[e] * sum[3] * s2));
         if (z == 0 || z == Nz - 1) {
           const int wall = (z == 0) ? 0 : 1;
           if (f < 2) {
@@ -1395,36 +1479,18 @@ struct KMean {
             v = make_double2(0.0, 0.0);
           }
         }
-        vs[z] = v;
+        vs[o] = v;
+        if (!ends) write(a, e, f, z, v);
       }
-    } else if constexpr (P == 3) {
-      for (int z = Nz + tid; z < Np; z += THREADS) vs[z] = cont(vs, z - Nz);
+    } else if constexpr (P == 4) {
+      if (ends)
+        for (int jj = tid; jj < a.g.Cc; jj += THREADS) write(a, e, f, Nz + jj, cont(a, vs, vs + d, jj));
     }
   }
-  // final write (after a barrier): shadow and float32 line
-  static FC_HD void write(const Args& a, unsigned char* sm, int tid, long long bid) {
-    const double2* vs = reinterpret_cast<const double2*>(sm) + NPMAX;
-    const int e = (int)bid, f = a.fmap[e];
-    C* xo = a.Xo + lay(f, 0, 0, a.g.Np, a.g.ntiles);
-    for (int z = tid; z < a.g.Np; z += THREADS) {
-      a.Xn[(long long)e * a.g.Np + z] = vs[z];
-      xo[z * TL] = mk<T>((T)vs[z].x, (T)vs[z].y);
-    }
-  }
-};
-
-// wrapper with the final write as its own phase
-template <class T>
-struct KMeanLine {
-  using Base = KMean<T>;
-  using Args = typename Base::Args;
-  using Regs = typename Base::Regs;
-  static constexpr int THREADS = Base::THREADS, NPHASE = 5, MINB = 1;
-  static constexpr size_t smem_bytes = Base::smem_bytes;
-  template <int P>
-  static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& r) {
-    if constexpr (P < 4) Base::template phase<P>(a, sm, tid, bid, r);
-    else Base::write(a, sm, tid, bid);
+  // shadow and float32 line
+  static FC_HD void write(const Args& a, int e, int f, int z, double2 v) {
+    a.Xn[(long long)e * a.g.Np + z] = v;
+    a.Xo[lay(f, z, 0, a.g.Np, a.g.ntiles)] = mk<T>((T)v.x, (T)v.y);
   }
 };
 
