@@ -97,22 +97,22 @@ fc_status injected(const char* entry) {
 }
 
 // Which float32 calls take the dense operators instead of the transforms.  A
-// tile of 128 lines passes through one SM in 6 us (N' = 75) to 45 us (538), so
+// tile of 128 lines passes through one SM in 10 us (N' = 115) to 45 us (538), so
 // a call needs a wave of tiles (152 x 128 lines) or more, and the gain depends
 // on how far the transform length lies above N'.  Measured, dense against
 // transform (us):
-//   padded, N' >= 180   257 x 16k lines 35 / 39, 513 x 16k 51 / 64, 513 x 41k
-//                       131 / 152, 400 x 82k 180 / 351, 513 x 400k 886 / 1520;
+//   padded, N' >= 180   257 x 16k lines 34 / 37, 513 x 16k 51 / 65, 513 x 41k
+//                       131 / 156, 400 x 82k 180 / 333, 513 x 400k 881 / 1578;
 //                       8k lines: 33 / 22 and 46 / 31, so from 16384 lines on
-//   padded, N' >= 75    50 x 164k 96 / 106, 65 x 164k 100 / 121, 129 x 164k
-//                       141 / 170; 65 x 82k 59 / 57: from 131072 lines on
-//   direct, N' >= 200   (the transform has length N') 487 x 82k 206 / 236, 231 x
-//                       164k 207 / 225; 487 x 41k 125 / 127: from 98304 lines on
-//   direct, shorter     103 x 400k 275 / 299, 39 x 400k 220 / 121: transforms
+//   padded, N' >= 100   90 x 132k 88 / 94, 129 x 132k 113 / 131; 129 x 41k 51 /
+//                       42, 65 x 132k 80 / 74: from 131072 lines on
+//   direct, N' >= 400   (the transform has length N') 487 x 82k 206 / 228, 41k
+//                       124 / 121: from 98304 lines on
+//   direct, shorter     231 x 132k 167 / 139: transforms
 static long long dense_min_lines(const PlanData& p) {
   const long long never = 1LL << 62;
-  if (p.dense_direct) return p.Np >= 200 ? 98304 : never;
-  return p.Np >= 180 ? 16384 : (p.Np >= 75 ? 131072 : never);
+  if (p.dense_direct) return p.Np >= 400 ? 98304 : never;
+  return p.Np >= 180 ? 16384 : (p.Np >= 100 ? 131072 : never);
 }
 bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines) {
   return dtype == FC_F32 && p.dense.NQ && lines >= dense_min_lines(p);

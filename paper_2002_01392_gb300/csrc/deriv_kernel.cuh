@@ -55,7 +55,6 @@ struct DerivPair {
   static constexpr int L1 = L1_, L2 = L2_, LINES = LINES_, JN = JN_;
   static_assert(JI <= JN_, "interior rows lie among the loaded rows");
   static constexpr int THREADS = E::THREADS, NPHASE = 5;
-  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
 
   struct Args {
     const T* f;
@@ -83,6 +82,7 @@ struct DerivPair {
   static constexpr size_t off_b1 = sizeof(C) * E::BUF;
   static constexpr size_t off_E = off_b1 + sizeof(C) * E::BUF;
   static constexpr size_t smem_bytes = off_E + sizeof(C) * LINES * 2 * DMAX;
+  static constexpr int MINB = min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {

@@ -28,6 +28,25 @@ FC_HD void prefetch_l2(const void* p) {
 #endif
 }
 
+// Blocks per SM that the registers of a line kernel are bounded for.  These
+// kernels wait for memory and barriers rather than for issue slots, so the
+// float32 ones whose register transforms are short (up to 24 values) get 72 to
+// 100 registers a thread, which they fill without spilling, and as many blocks
+// as the shared memory then allows (256^2 x 257 x 4: stage combine 588 -> 424 us,
+// and with the changes at PhiLine and KHom the projection 679 -> 489 us; before,
+// 168 registers and 12 warps per SM; the z derivatives, 357 us, gain nothing;
+// x pass 404 -> 338 us; derivatives of 131580 lines x 103 104 -> 76 us, of 65536 x
+// 33 31 -> 25 us).
+// Longer transforms (30 to 48 values) spill below 128 registers.
+template <class T>
+constexpr int min_blocks(int L1, int L2, int threads, size_t smem) {
+  const int base = threads <= 160 ? 3 : (threads <= 320 ? 2 : 1), m = L1 > L2 ? L1 : L2;
+  if (sizeof(T) != 4 || m > 24) return base;
+  const int regs = 65536 / ((m <= 16 ? 72 : 100) * threads), room = (int)(224 * 1024 / (smem + 1024));
+  const int most = regs < room ? regs : room;
+  return most > base ? most : base;
+}
+
 template <class T, int L1_, int L2_, int LINES_>
 struct Eng {
   static constexpr int L1 = L1_, L2 = L2_, L = L1 * L2, LINES = LINES_;

@@ -110,23 +110,6 @@ FC_HD void load_mr(unsigned char* sm, const ZTab<T>& t, int n, int tid, int thre
   }
 }
 
-// Blocks per SM that the registers of a z kernel are bounded for.  These kernels
-// wait for memory and barriers rather than for issue slots, so the float32 ones
-// whose register transforms are short (up to 24 values) get 100 registers a
-// thread and as many blocks as the shared memory then allows (256^2 x 257 x 4:
-// stage combine 588 -> 424 us, and with the changes at PhiLine and KHom the
-// projection 679 -> 489 us; before, 168 registers and 12 warps per SM; the z
-// derivatives, 357 us, gain nothing).  Longer transforms (30 to 48 values) spill
-// below 128 registers.
-template <class T>
-constexpr int z_min_blocks(int L1, int L2, int threads, size_t smem) {
-  const int base = threads <= 160 ? 3 : (threads <= 320 ? 2 : 1);
-  if (sizeof(T) != 4 || L1 > 24 || L2 > 24) return base;
-  const int regs = 65536 / (100 * threads), room = (int)(224 * 1024 / (smem + 1024));
-  const int most = regs < room ? regs : room;
-  return most > base ? most : base;
-}
-
 // ===========================================================================
 // K1  zderiv: dz and dzz of the state at the Nz physical points.
 // Circular convolution of the extended line with the derivative kernels of
@@ -154,7 +137,7 @@ struct KZDeriv {
   struct Regs { C v[L1]; C u[L2]; };
   static constexpr size_t off_b1 = sizeof(C) * E::BUF;
   static constexpr size_t smem_bytes = 2 * sizeof(C) * E::BUF;
-  static constexpr int MINB = z_min_blocks<T>(L1, L2, THREADS, smem_bytes);
+  static constexpr int MINB = min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
@@ -252,7 +235,7 @@ struct KZCombine {
   static constexpr size_t off_E = off_M + sizeof(double) * MRMAX;
   static constexpr size_t off_C = off_E + sizeof(C) * LINES * 2 * DMAX;   // continuation values [C][LINES]
   static constexpr size_t smem_bytes = off_C + sizeof(C) * LINES * CMAX;
-  static constexpr int MINB = z_min_blocks<T>(L1, L2, THREADS, smem_bytes);
+  static constexpr int MINB = min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
@@ -487,7 +470,7 @@ struct KZProject {
   static constexpr bool SG = sizeof(T) == 4 && sg_bytes <= 24 * 1024;
   static constexpr int GS = SG ? LINES : TL;   // element stride of a scratch line
   static constexpr size_t smem_bytes = off_G + (SG ? sg_bytes : 0);
-  static constexpr int MINB = z_min_blocks<T>(L1, L2, THREADS, smem_bytes);
+  static constexpr int MINB = min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   // conj(chirp[n]) (1 outside the line)
   static FC_HD C cchirp(const ZTab<T>& t, int n, int Np) {
@@ -785,7 +768,6 @@ struct KYInv3 {
   using E = Eng<T, L1, L2, LINES>;
   using C = cx<T>;
   static constexpr int THREADS = E::THREADS, NPHASE = 4;
-  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
   struct Args {
     YGeom g;
     const C* tw;
@@ -797,6 +779,8 @@ struct KYInv3 {
   };
   struct Regs { C v[L1]; C u[L2]; };
   static constexpr size_t smem_bytes = 2 * sizeof(C) * E::BUF;
+  // (more blocks, by a tighter register bound, made the y inverse slower: 272 -> 366 us at 256^2 x 257 x 4)
+  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
@@ -871,10 +855,10 @@ struct KYInv3S {
   using E = Eng<T, L1, L2, LINES>;
   using C = cx<T>;
   static constexpr int THREADS = E::THREADS, NPHASE = 6;
-  static constexpr int MINB = 1;
   using Args = typename KYInv3<T, L1, L2, LINES>::Args;
   struct Regs { C v[L1]; C u[L2]; };
   static constexpr size_t smem_bytes = sizeof(C) * E::BUF;
+  static constexpr int MINB = 1;
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
@@ -927,7 +911,6 @@ struct KY1 {
   using E = Eng<T, L1, L2, LINES>;
   using C = cx<T>;
   static constexpr int THREADS = E::THREADS, NPHASE = 2;
-  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
   struct Args {
     YGeom g;
     const C* tw;
@@ -938,6 +921,7 @@ struct KY1 {
   };
   struct Regs { C v[L1]; C u[L2]; };
   static constexpr size_t smem_bytes = sizeof(C) * E::BUF;
+  static constexpr int MINB = THREADS <= 160 ? 3 : (THREADS <= 320 ? 2 : 1);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long bid, Regs& R) {
@@ -1032,7 +1016,7 @@ struct KXPass {
 #else
   static constexpr bool HALF = Nx >= 1024;
 #endif
-  static constexpr int THREADS = NJOB * G, NPHASE = 8, MINB = 2;
+  static constexpr int THREADS = NJOB * G, NPHASE = 8;
   struct Args {
     int Kx, Kxp, Ny, Nz;
     int Kw;                  // columns of NL that are used later (the rest is not written)
@@ -1050,6 +1034,7 @@ struct KXPass {
   static constexpr size_t zb_bytes = sizeof(C) * RE::BUF * NJOB;
   static constexpr size_t pr_bytes = sizeof(T) * 4 * NF * Nx;
   static constexpr size_t smem_bytes = zb_bytes > pr_bytes ? zb_bytes : pr_bytes;
+  static constexpr int MINB = L1 > 24 || L2 > 24 || sizeof(T) != 4 ? 2 : min_blocks<T>(L1, L2, THREADS, smem_bytes);
 
   template <int P>
   static FC_HD void phase(const Args& a, unsigned char* sm, int tid, long long row, Regs& R) {

@@ -94,8 +94,7 @@ def _bound(f, Mr, order, Lz=1.0):
 # every branch: parts 4 (N' even) and 2 (odd), one and several chunks and slabs, resident blocks, direct lengths, a last
 # tile of few lines, a tile across two fields, odd line counts, one output, Lz
 @pytest.mark.gpu
-@pytest.mark.parametrize("Nz,Ny,Nx,B,Lz", [(50, 257, 511, 1, 1.0), (65, 256, 513, 1, 2.0), (104, 363, 121, 3, 1.0),
-                                            (155, 128, 128, 1, 1.0), (231, 193, 255, 2, 1.0), (257, 129, 128, 1, 1.0),
+@pytest.mark.parametrize("Nz,Ny,Nx,B,Lz", [(104, 363, 121, 3, 1.0), (155, 128, 128, 1, 2.0), (257, 129, 128, 1, 1.0),
                                             (350, 64, 257, 1, 0.5), (487, 317, 311, 1, 1.0), (512, 131, 127, 1, 1.0),
                                             (513, 64, 129, 2, 1.0), (549, 128, 129, 1, 1.0)])
 def test_dense_kernel_matches_oracle(api, Mr_5_25, Nz, Ny, Nx, B, Lz):
