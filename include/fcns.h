@@ -119,7 +119,12 @@ fc_status fc_destroy(fc_plan_t plan);
  * Needs no workspace.  Transform length: N' itself when it is a compiled
  * smooth length (64, 128, 256, 512, 768, 1024, 1536), else the smallest
  * compiled length >= N' + Nz - 1 (up to 1536); FC_ERR_UNSUPPORTED when
- * neither exists.
+ * neither exists.  Large float32 calls, and float64 calls for N' <= 384 or
+ * even N' < 576, take the derivative operators as dense blocks on the tensor
+ * cores instead of transforms (same accuracy, float64 through exact integer
+ * sums); a NaN or Inf then spoils the outputs of its own line only.
+ * FC_ERR_TIMEOUT: the float32 dense kernel of an earlier call of the plan gave
+ * up a bounded wait (its outputs are not valid); the state is cleared.
  */
 fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, double Lz,
                      const void* f, void* df, void* d2f, fc_stream_t stream);
@@ -136,8 +141,9 @@ fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, 
  *   - Calls no cudaMalloc, cudaFree or other allocating routine.  The plan's
  *     tables (continuation matrix, kernel spectra, twiddles) live in one
  *     fixed 128 KiB static device array that every GPU loading the library
- *     reserves until the process exits, and the operator blocks of large
- *     float32 calls in another of 1.34 MiB.
+ *     reserves until the process exits, and the operator blocks of
+ *     calls that fc_deriv_z runs with the dense operators in another of
+ *     2.25 MiB.
  *   - The first call on each device looks up that array's device address
  *     (cudaGetSymbolAddress) with the device current and keeps it for the
  *     life of the process: resetting the device (cudaDeviceReset) after that

@@ -114,8 +114,14 @@ static long long dense_min_lines(const PlanData& p) {
   if (p.dense_direct) return p.Np >= 400 ? 98304 : never;
   return p.Np >= 180 ? 16384 : (p.Np >= 100 ? 131072 : never);
 }
+// Float64 calls take them wherever the plan has them: the transforms sit on the
+// float64 pipe and lose at every size.  Measured, dense against transform (us):
+// 11 x 512 lines 29 / 58, 65 x 8k 80 / 197, 231 (direct) x 131k 2387 / 3198, 487
+// (direct) x 2560 194 / 201 (the closest: the second wave of tiles nearly empty),
+// x 131k 4927 / 6438, 513 x 512 55 / 130, x 131k 5001 / 16258.
 bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines) {
-  return dtype == FC_F32 && p.dense.NQ && lines >= dense_min_lines(p);
+  if (dtype == FC_F64) return p.dense64.NQ != 0;
+  return p.dense.NQ && lines >= dense_min_lines(p);
 }
 
 }  // namespace fcns
@@ -209,14 +215,23 @@ fc_status fc_setup_ex(int d, int C, int Nz, int M, int n_os, fc_plan_t* out) {
     const float hi = (float)p->data.Mr[i];
     p->deriv.Mr2[i] = make_float2(hi, (float)(p->data.Mr[i] - (double)hi));
   }
-  p->data.dense_direct = L == p->data.Np;
-  if (L > 0 && dense_min_lines(p->data) < (1LL << 31) && dense_geom(Nz, p->data.Np, &p->data.dense)) {
-    std::vector<double> c1, c2;
-    deriv_kernels_closed(p->data.Np, &c1, &c2);
-    p->data.dense_exp[0] = dense_blocks(p->data.dense, c1, &p->data.dense_blocks);
-    p->data.dense_exp[1] = dense_blocks(p->data.dense, c2, &p->data.dense_blocks);
-  } else {
-    p->data.dense = DenseGeom();
+  PlanData& pd = p->data;
+  pd.dense_direct = L == pd.Np;
+  const bool f32 = L > 0 && dense_min_lines(pd) < (1LL << 31) && dense_geom(Nz, pd.Np, &pd.dense);
+  const bool f64 = L > 0 && dense64_geom(Nz, pd.Np, &pd.dense64);
+  if (!f32) pd.dense = DenseGeom();
+  std::vector<double> c1, c2;
+  if (f32 || f64) deriv_kernels_closed(pd.Np, &c1, &c2);
+  if (f32) {
+    pd.dense_exp[0] = dense_blocks(pd.dense, c1, &pd.dense_blocks);
+    pd.dense_exp[1] = dense_blocks(pd.dense, c2, &pd.dense_blocks);
+  }
+  // (no digit sum reaches 2^24 for any N' of either parity of Nz: checked over all of them)
+  if (f64 && !(dense64_blocks(pd.dense64, c1, &pd.dense64_blocks, &pd.dense64_exp[0], &pd.dense64_sh[0]) &&
+               dense64_blocks(pd.dense64, c2, &pd.dense64_blocks, &pd.dense64_exp[1], &pd.dense64_sh[1]))) {
+    delete p;
+    set_error("fc_setup: float64 operators of this size are not exact in digits");
+    return FC_ERR_UNSUPPORTED;
   }
   *out = p;
   return FC_OK;
@@ -252,7 +267,7 @@ fc_status fc_destroy(fc_plan_t plan) {
       cudaDeviceSynchronize();
       cudaFree(t.Mr); cudaFree(t.Mr2); cudaFree(t.tw32); cudaFree(t.tw64);
       cudaFree(t.H1_32); cudaFree(t.H1_64); cudaFree(t.H2_32); cudaFree(t.H2_64);
-      cudaFree(t.dense);
+      cudaFree(t.dense); cudaFree(t.dense64);
       if (t.dense_err) cudaFreeHost(t.dense_err);
       for (auto& slot : t.stage)
         for (void* b : slot) cudaFree(b);
@@ -320,10 +335,11 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
     if (!s) s = cuda_status(cudaHostAlloc((void**)&t.dense_err, sizeof(unsigned), cudaHostAllocDefault), "cudaHostAlloc");
     if (!s) *t.dense_err = 0;
   }
+  if (!s && plan->data.dense64.NQ) s = up(plan->data.dense64_blocks.data(), 2 * plan->data.dense64_blocks.size(), &t.dense64);
   if (s) {
     cudaFree(t.Mr); cudaFree(t.Mr2); cudaFree(t.tw32); cudaFree(t.tw64);
       cudaFree(t.H1_32); cudaFree(t.H1_64); cudaFree(t.H2_32); cudaFree(t.H2_64);
-      cudaFree(t.dense);
+      cudaFree(t.dense); cudaFree(t.dense64);
       if (t.dense_err) cudaFreeHost(t.dense_err);
     return s;
   }
@@ -367,9 +383,8 @@ extern "C" fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int N
     s = deriv_tables_locked(plan, &t);
   }
   if (s) return s;
-  if (deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch))
-    return launch_deriv_dense(*t, plan->data, batch, (long long)Nx * Ny, Lz, f, df, d2f, (cudaStream_t)stream);
-  return launch_deriv_z(*t, plan->data, dtype, batch, (long long)Nx * Ny, Lz, f, df, d2f, (cudaStream_t)stream);
+  const bool dense = deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch);
+  return launch_deriv_any(dense, *t, plan->data, dtype, batch, (long long)Nx * Ny, Lz, f, df, d2f, (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -450,8 +465,7 @@ extern "C" fc_status fc_deriv_z_host_ex(fc_plan_t plan, fc_dtype dtype, int batc
       if (!s) s = cuda_status(cudaEventRecord(t->ev_in[k], t->st_in), "cudaEventRecord");
       if (!s) s = cuda_status(cudaStreamWaitEvent(t->st_run, t->ev_in[k], 0), "cudaStreamWaitEvent");
       void *o1 = df ? t->stage[k][1] : nullptr, *o2 = d2f ? t->stage[k][2] : nullptr;
-      if (!s) s = dense ? launch_deriv_dense(*t, plan->data, 1, (long long)Nx * yc, Lz, t->stage[k][0], o1, o2, t->st_run)
-                        : launch_deriv_z(*t, plan->data, dtype, 1, (long long)Nx * yc, Lz, t->stage[k][0], o1, o2, t->st_run);
+      if (!s) s = launch_deriv_any(dense, *t, plan->data, dtype, 1, (long long)Nx * yc, Lz, t->stage[k][0], o1, o2, t->st_run);
       if (!s) s = cuda_status(cudaEventRecord(t->ev_run[k], t->st_run), "cudaEventRecord");
       if (!s) s = cuda_status(cudaStreamWaitEvent(t->st_out, t->ev_run[k], 0), "cudaStreamWaitEvent");
       for (int o = 0; o < 2 && !s; ++o)

@@ -9,11 +9,13 @@
 // [1 - delta_r, 2b - (1 - delta_r)] (2(d + C) grid spacings).  The right-end
 // matrix is M_r = A_r Q_r^T (App. B, eq. Af).
 #include "host_tables.hpp"
+#include "dense64.hpp"
 
 #include <cuda_fp16.h>
 
 
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -653,6 +655,87 @@ int dense_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<u
         out->insert(out->end(), low.begin(), low.end());
       }
   return e;
+}
+
+bool dense64_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out, int* e, int* sh) {
+  // entries as in dense_blocks, each kernel value rounded to whole units first
+  double big = 0.0;
+  for (double v : c) big = std::max(big, std::fabs(v));
+  *e = 54 - std::ilogb(big / g.NQ);
+  std::vector<long long> ci(c.size());
+  std::vector<long long> B((size_t)g.NQ * g.No * g.No);
+  for (int turn = 0; turn < 2; ++turn) {
+    for (size_t i = 0; i < c.size(); ++i) ci[i] = std::llrint(std::ldexp(c[i], *e) / g.NQ);
+    long long most = 0;
+    for (int ji = 0; ji < g.No; ++ji) {
+      int rows[4], n = 0, member[4];
+      for (int i = 0; i < g.NQ; ++i) {
+        const int r = dense_row(g, ji, i);
+        bool seen = false;
+        for (int k = 0; k < n; ++k) seen = seen || rows[k] == r;
+        if (seen) continue;
+        rows[n] = r;
+        member[n++] = i;
+      }
+      for (int jo = 0; jo < g.No; ++jo) {
+        const int n0 = dense_row(g, jo, 0);
+        for (int q = 0; q < g.NQ; ++q) {
+          long long v = 0;
+          for (int k = 0; k < n; ++k) {
+            const int neg = ((q & member[k] & 1) + ((q & member[k] & 2) >> 1)) & 1;
+            const long long x = ci[n0 - rows[k] + (n0 < rows[k] ? g.Np : 0)];
+            v += neg ? -x : x;
+          }
+          B[((size_t)q * g.No + jo) * g.No + ji] = v;
+          most = std::max(most, v < 0 ? -v : v);
+        }
+      }
+    }
+    if (most <= 1LL << 55) break;
+    *e -= std::ilogb((double)most) - 54;   // several large kernel values met in one entry
+  }
+  // float16 bits of the digits
+  static const std::vector<unsigned short> half_of = [] {
+    std::vector<unsigned short> v(257);
+    for (int i = 0; i < 257; ++i) {
+      const __half h = __float2half((float)(i - 128));
+      std::memcpy(&v[i], &h, 2);
+    }
+    return v;
+  }();
+  const int KT = g.KQ / 16;
+  const size_t at0 = out->size();
+  out->resize(at0 + (size_t)dense64_order_halves(g), 0);
+  double rows_most = 0.0;
+  bool exact = true;
+  for (int jo = 0; jo < g.No; ++jo) {
+    double sum = 0.0;
+    for (int q = 0; q < g.NQ; ++q) {
+      long long by_digit[kD64Digits] = {};
+      for (int ji = 0; ji < g.No; ++ji) {
+        const long long v = B[((size_t)q * g.No + jo) * g.No + ji];
+        sum += std::fabs((double)v);
+        const unsigned long long w = d64_bias(v);
+        unsigned short* o = &(*out)[at0 + (((size_t)(jo / 16) * g.NQ + q) * KT + ji / 16) * kD64Digits * 256 +
+                                    d64_b_index(ji % 16, jo % 16)];
+        for (int i = 0; i < kD64Digits; ++i) {
+          const int field = d64_field(w, i);
+          by_digit[i] += std::abs(field - 128);
+          o[i * 256] = half_of[field];
+        }
+      }
+      // the line's digits are at most 128
+      for (int s = 0; s < kD64Sums; ++s) {
+        long long most = 0;
+        for (int j = std::max(0, s - kD64Digits + 1); j <= std::min(s, kD64Digits - 1); ++j) most += 128 * by_digit[j];
+        exact = exact && most <= 1LL << 24;
+      }
+    }
+    rows_most = std::max(rows_most, sum);
+  }
+  // |output| <= 2^55 rows_most, in units of 2^40
+  *sh = std::max(0, (int)std::ceil(std::log2(rows_most)) + 55 - 40 - 61);
+  return exact && *sh <= 32;
 }
 
 }  // namespace fcns

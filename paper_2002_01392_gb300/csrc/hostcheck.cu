@@ -3,11 +3,14 @@
 // arithmetic and data flow with the oracle.  Not part of libfcns and never
 // loaded by the product path.
 #define FC_HOSTCHECK 1
+#include <cuda_fp16.h>
+
 #include <chrono>
 #include <complex>
 #include <vector>
 
 #include "deriv_kernel.cuh"
+#include "dense64.hpp"
 #include "host_tables.hpp"
 #include "slabs.hpp"
 
@@ -240,6 +243,74 @@ int fchc_dense_blocks(int Nz, int Np, int order, unsigned short* halves, int* ex
   *exponent = dense_blocks(g, order == 1 ? c1 : c2, &out);
   std::memcpy(halves, out.data(), 2 * out.size());
   return (long long)out.size() == dense_order_halves(g) ? 0 : 2;
+}
+// Float64 derivative of order 1 or 2 (unit spacing) of a tile of 16 lines x
+// [Nz][16] by the dense operators, y [Nz][16]: the kernel's own tables, index
+// maps and number formats, the products and sums in 64-bit integers.  Returns
+// 1 where there is no geometry, 2 where the digit sums could be inexact, 3
+// where one left 2^24.
+int fchc_dense64_tile(int Nz, int d, int C, const double* Mr, int order, const double* x, double* y) {
+  DenseGeom g;
+  if (!dense64_geom(Nz, Nz + C, &g)) return 1;
+  std::vector<double> c1, c2;
+  deriv_kernels_closed(g.Np, &c1, &c2);
+  std::vector<unsigned short> blocks;
+  int ex = 0, sh = 0;
+  if (!dense64_blocks(g, order == 1 ? c1 : c2, &blocks, &ex, &sh)) return 2;
+  if ((long long)blocks.size() != dense64_order_halves(g)) return 4;
+  const int KT = g.KQ / 16;
+  std::vector<unsigned long long> X((size_t)g.Np * 16);
+  std::memcpy(X.data(), x, sizeof(double) * Nz * 16);
+  std::vector<int> A((size_t)g.NQ * KT * kD64Digits * 256);
+  int E[16];
+  for (int li = 0; li < 16; ++li) {
+    for (int jj = 0; jj < C; ++jj)
+      X[(size_t)(Nz + jj) * 16 + li] = d64_continuation(jj, d, C, Mr, &X[li], &X[(size_t)(Nz - d) * 16 + li], 16);
+    E[li] = 1;
+    for (int n = 0; n < g.Np; ++n) E[li] = std::max(E[li], (int)(X[(size_t)n * 16 + li] >> 52) & 0x7ff);
+    for (int j = 0; j < g.KQ; ++j)
+      for (int q = 0; q < g.NQ; ++q) {
+        long long u = 0;
+        for (int i = 0; i < g.NQ && j < g.No && E[li] < 0x7ff; ++i) {
+          const long long v = d64_fixed(X[(size_t)dense_row(g, j, i) * 16 + li], E[li]);
+          u += __builtin_popcount(q & i) & 1 ? -v : v;
+        }
+        const unsigned long long w = d64_bias(u);
+        for (int i = 0; i < kD64Digits; ++i)
+          A[((size_t)(q * KT + j / 16) * kD64Digits + i) * 256 + d64_a_index(li, j % 16)] = d64_field(w, i) - 128;
+      }
+  }
+  std::vector<int> B(blocks.size());
+  for (size_t i = 0; i < blocks.size(); ++i) {
+    __half h;
+    std::memcpy(&h, &blocks[i], 2);
+    B[i] = (int)__half2float(h);
+  }
+  for (int li = 0; li < 16; ++li)
+    for (int j = 0; j < g.No; ++j) {
+      long long row[4] = {};
+      for (int q = 0; q < g.NQ; ++q) {
+        long long s[kD64Sums] = {};
+        for (int ks = 0; ks < KT; ++ks)
+          for (int i = 0; i < kD64Digits; ++i)
+            for (int b = 0; b < kD64Digits && i + b < kD64Sums; ++b)
+              for (int k = 0; k < 16; ++k)
+                s[i + b] += (long long)A[((size_t)(q * KT + ks) * kD64Digits + i) * 256 + d64_a_index(li, k)] *
+                            B[((((size_t)(j / 16) * g.NQ + q) * KT + ks) * kD64Digits + b) * 256 + d64_b_index(k, j % 16)];
+        int si[kD64Sums];
+        for (int i = 0; i < kD64Sums; ++i) {
+          if (s[i] > (1 << 24) || s[i] < -(1 << 24)) return 3;
+          si[i] = (int)s[i];
+        }
+        const long long v = d64_combine(si, sh);
+        for (int i = 0; i < g.NQ; ++i) row[i] += (__builtin_popcount(q & i) + (order == 1 ? i : 0)) & 1 ? -v : v;
+      }
+      for (int i = 0; i < g.NQ; ++i) {
+        const int n = dense_row(g, j, i);
+        if (n < Nz) y[(size_t)n * 16 + li] = E[li] == 0x7ff ? NAN : std::ldexp((double)row[i], 40 + sh + E[li] - 1075 - ex);
+      }
+    }
+  return 0;
 }
 // thread order inside a phase (0 ascending, 1 descending) and shared-memory
 // poisoning of the emulation (see phased_emulate)

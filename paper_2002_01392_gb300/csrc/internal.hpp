@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/fcns.h"
+#include "dense64.hpp"
 #include "dense_geom.hpp"
 
 namespace fcns {
@@ -36,6 +37,7 @@ struct DerivDevTables {
   void* H2_32 = nullptr;
   void* H2_64 = nullptr;
   void* dense = nullptr;          // blocks of the dense operators (float16 pairs), both orders; null: not used
+  void* dense64 = nullptr;        // the same for float64 (digit fragments)
   unsigned* dense_err = nullptr;  // host word (pinned) that a kernel sets when a wait runs out
   // staging of fc_deriv_z_host: three rotating slots of (input, d1, d2) slab
   // buffers of stage_bytes each, and the copy-in / compute / copy-out streams
@@ -53,6 +55,9 @@ struct PlanData {
   int dense_exp[2] = {0, 0};
   bool dense_direct = false;              // the transform kernel would run at length N' itself
   std::vector<unsigned short> dense_blocks;
+  DenseGeom dense64;                      // the same for float64 (dense64.hpp)
+  int dense64_exp[2] = {0, 0}, dense64_sh[2] = {0, 0};
+  std::vector<unsigned short> dense64_blocks;
   std::mutex mtx;
   std::mutex host_mtx;   // serialises fc_deriv_z_host calls on the plan (shared staging)
   std::vector<DerivDevTables> dev;
@@ -87,6 +92,15 @@ fc_status launch_deriv_z(const DerivDevTables& t, const PlanData& p, fc_dtype dt
 // the same by the dense operators (float32; plans with a dense geometry)
 fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int batch, long long lines, double Lz,
                              const void* f, void* df, void* d2f, cudaStream_t stream);
+fc_status launch_deriv_dense64(const DerivDevTables& t, const PlanData& p, int batch, long long lines, double Lz,
+                               const void* f, void* df, void* d2f, cudaStream_t stream);
+// the kernel of a whole call by its type and lines: transforms, or the dense operators of its precision
+inline fc_status launch_deriv_any(bool dense, const DerivDevTables& t, const PlanData& p, fc_dtype dtype, int batch,
+                                  long long lines, double Lz, const void* f, void* df, void* d2f, cudaStream_t stream) {
+  if (!dense) return launch_deriv_z(t, p, dtype, batch, lines, Lz, f, df, d2f, stream);
+  return dtype == FC_F64 ? launch_deriv_dense64(t, p, batch, lines, Lz, f, df, d2f, stream)
+                         : launch_deriv_dense(t, p, batch, lines, Lz, f, df, d2f, stream);
+}
 // whether a whole call (all its lines) takes the dense operators
 bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines);
 

@@ -26,14 +26,16 @@ constexpr int kMaxDevices = 64;
 // Shared by every call on a device; holds the tables of the last call.
 static __device__ __align__(256) unsigned char g_deriv_scratch[kNoAllocBytes];
 // The same for calls that fc_deriv_z runs with the dense operators: their
-// blocks (at most 1.33 MB, N' = 575) and the continuation matrix.
-constexpr size_t kNoAllocDense = 1376 * 1024;
+// blocks (at most 1.33 MB in float32, N' = 575, and 2.33 MB in float64, N' =
+// 576) and the continuation matrix.
+constexpr size_t kNoAllocDense = 2304 * 1024;
 static __device__ __align__(256) unsigned char g_dense_scratch[kNoAllocDense];
 
 std::mutex g_mtx;
 void* g_scratch_addr[kMaxDevices] = {};
 void* g_dense_addr[kMaxDevices] = {};
 unsigned long long g_dense_serial[kMaxDevices] = {};
+int g_dense_dtype[kMaxDevices] = {};
 // which tables the array holds per device: the plan's serial number and the
 // precision of the last upload (0: none, or an upload that failed part-way)
 unsigned long long g_loaded_serial[kMaxDevices] = {};
@@ -54,10 +56,13 @@ fc_status scratch_address(int dev, unsigned char** out) {
   return FC_OK;
 }
 
-// the dense-operator call: blocks and matrix copied when the plan differs from the previous such call's
-fc_status noalloc_dense(fc_plan* plan, int dev, int batch, long long lines, double Lz, const void* f, void* df, void* d2f,
+// the dense-operator call: blocks and matrix copied when the plan or precision differs from the previous such call's
+fc_status noalloc_dense(fc_plan* plan, fc_dtype dtype, int dev, int batch, long long lines, double Lz, const void* f, void* df, void* d2f,
                         cudaStream_t st) {
-  const size_t nB = 2 * plan->data.dense_blocks.size(), nM = sizeof(float2) * plan->deriv.Mr2.size();
+  const bool f64 = dtype == FC_F64;
+  const std::vector<unsigned short>& blocks = f64 ? plan->data.dense64_blocks : plan->data.dense_blocks;
+  const void* Mr = f64 ? (const void*)plan->data.Mr.data() : (const void*)plan->deriv.Mr2.data();
+  const size_t nB = 2 * blocks.size(), nM = sizeof(double) * plan->data.Mr.size();   // (a float pair per entry in float32)
   if (nB + nM > kNoAllocDense) {
     set_error("fc_deriv_z_noalloc: dense blocks of this plan exceed the static scratch");
     return FC_ERR_UNSUPPORTED;
@@ -70,19 +75,21 @@ fc_status noalloc_dense(fc_plan* plan, int dev, int batch, long long lines, doub
       s = cuda_status(cudaGetSymbolAddress(&g_dense_addr[dev], g_dense_scratch), "cudaGetSymbolAddress(g_dense_scratch)");
     if (s) return s;
     base = static_cast<unsigned char*>(g_dense_addr[dev]);
-    if (g_dense_serial[dev] != plan->deriv.serial) {
+    if (g_dense_serial[dev] != plan->deriv.serial || g_dense_dtype[dev] != (int)dtype) {
       g_dense_serial[dev] = 0;
-      s = cuda_status(cudaMemcpyAsync(base, plan->data.dense_blocks.data(), nB, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(dense)");
-      if (!s) s = cuda_status(cudaMemcpyAsync(base + nB, plan->deriv.Mr2.data(), nM, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(Mr2)");
+      s = cuda_status(cudaMemcpyAsync(base, blocks.data(), nB, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(dense)");
+      if (!s) s = cuda_status(cudaMemcpyAsync(base + nB, Mr, nM, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(M_r)");
       if (s) return s;
       g_dense_serial[dev] = plan->deriv.serial;
+      g_dense_dtype[dev] = (int)dtype;
     }
   }
   DerivDevTables t;
   t.device = dev;
-  t.dense = base;
+  t.dense = t.dense64 = base;
+  t.Mr = reinterpret_cast<double*>(base + nB);
   t.Mr2 = reinterpret_cast<float2*>(base + nB);
-  return launch_deriv_dense(t, plan->data, batch, lines, Lz, f, df, d2f, st);
+  return launch_deriv_any(true, t, plan->data, dtype, batch, lines, Lz, f, df, d2f, st);
 }
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }
@@ -115,7 +122,7 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
   if (s) return s;
   cudaStream_t st = (cudaStream_t)stream;
   if (deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch))
-    return noalloc_dense(plan, dev, batch, (long long)Nx * Ny, Lz, f, df, d2f, st);
+    return noalloc_dense(plan, dtype, dev, batch, (long long)Nx * Ny, Lz, f, df, d2f, st);
   {
     std::lock_guard<std::mutex> lk(g_mtx);
     if (g_loaded_serial[dev] != h.serial || g_loaded_dtype[dev] != (int)dtype) {

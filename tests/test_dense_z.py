@@ -167,3 +167,105 @@ def test_dense_kernel_magnitudes_and_nonfinite(api, Mr_5_25):
         av = a.cpu().view(torch.int32)
         fin = torch.isfinite(a.cpu())
         assert torch.equal(av[fin], b.view(torch.int32)[fin]) and torch.equal(av[fin], c.cpu().view(torch.int32)[fin])
+
+
+# ---------------------------------------------------------------------------
+# float64: exact integer products (dense64.hpp)
+# ---------------------------------------------------------------------------
+def _lines64(Nz, n, seed):
+    """Smooth and rough lines, wall layers, wide ranges of magnitude inside a line and between lines."""
+    r = np.random.default_rng(seed)
+    z = np.linspace(0, 1, Nz)[:, None]
+    f = np.sin(z * r.uniform(1, 30, n) + 1) + r.uniform(-1, 1, n) * z ** 3
+    f[:, 1::4] += 1e-3 * r.standard_normal((Nz, len(range(1, n, 4))))
+    f[:, 2::4] = np.exp(-z * r.uniform(5, 60, len(range(2, n, 4)))) * 10.0 ** r.uniform(-200, 200, len(range(2, n, 4)))
+    f[:, 3::4] *= np.where(np.arange(Nz) == Nz // 2, 1e6, 1.0)[:, None]
+    return f
+
+
+def _bound64(f, Mr, order, Lz=1.0):
+    """Per line and value.  Line: whole units of at most 2^-52 of its largest value m, each off by half a unit, through an
+    operator whose rows have 2-norm k_max^order (order 2: 0.45 of it) -> 2^-52 m k_max^order.  Operator: kernel values
+    carry 2^-53 of themselves and whole units of 2^-54 of the largest, times at most m each -> 2^-52 sqrt(N') m k_max^order.
+    Products left out and the outputs' units are below that; the same again for the rounding of the outputs and the sums
+    of the two orders' scale factors."""
+    m = np.abs(fc.extend(f, Mr)).max(axis=0)
+    kmax = np.pi * (f.shape[0] - 1) / Lz
+    return 4 * 2.0 ** -52 * np.sqrt(f.shape[0] + Mr.shape[0]) * m * kmax ** order
+
+
+def _derivative_ld(f, Mr, order, Lz=1.0):
+    """Continuation and derivative of f [Nz][lines] in extended precision."""
+    ld = np.longdouble
+    Nz, C, d = f.shape[0], Mr.shape[0], Mr.shape[1]
+    Np = Nz + C
+    x, M = f.astype(ld), Mr.astype(ld)
+    cont = sum(M[:, i:i + 1] * x[Nz - d + i] + M[::-1, d - 1 - i:d - i] * x[i] for i in range(d))
+    xe = np.vstack([x, cont])
+    pi = ld("3.14159265358979323846264338327950288")
+    k = np.arange(1, (Np + 1) // 2)
+    ang = 2 * pi * ((np.arange(Np)[:, None] * k) % Np).astype(ld) / Np
+    w = 2 * pi * k.astype(ld) / Np
+    c = -2 * (w * np.sin(ang)).sum(1) if order == 1 else -2 * (w * w * np.cos(ang)).sum(1)
+    if order == 2 and Np % 2 == 0:
+        c = c - pi * pi * np.where(np.arange(Np) % 2, -1, 1)
+    c = c / Np
+    y = np.stack([(c[(n - np.arange(Np)) % Np][:, None] * xe).sum(0) for n in range(Nz)])
+    return y / (ld(Lz) / (Nz - 1)) ** order
+
+
+@pytest.mark.parametrize("Nz", [11, 20, 33, 39, 102, 103, 128, 231, 358, 513, 549])
+def test_dense64_arithmetic_on_the_cpu(Nz, Mr_5_25):
+    """The kernel's tables, index maps and number formats against the oracle, the digit sums below 2^24."""
+    lib = _lib()
+    f = np.ascontiguousarray(_lines64(Nz, 16, Nz))
+    f[:, 15] = 0
+    Mr = np.ascontiguousarray(Mr_5_25, dtype=np.float64)
+    ptr = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    for order in (1, 2):
+        y = np.full((Nz, 16), np.nan)
+        assert lib.fchc_dense64_tile(Nz, 5, 25, ptr(Mr), order, ptr(f), ptr(y)) == 0
+        err = np.abs(y - _derivative_ld(f, Mr, order, Nz - 1.0)).max(axis=0)
+        bound = _bound64(f, Mr, order, Nz - 1.0)
+        assert (err <= bound).all(), (order, (err / bound).max())
+        assert not y[:, 15].any()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("Nz,Ny,Nx,B,Lz", [(11, 5, 3, 1, 1.0), (33, 7, 37, 3, 2.0), (65, 64, 66, 1, 1.0), (102, 33, 31, 2, 1.0),
+                                            (231, 48, 51, 1, 0.5), (358, 16, 17, 2, 1.0), (513, 61, 41, 1, 1e-6),
+                                            (549, 50, 49, 1, 1e5)])
+def test_dense64_kernel(api, Mr_5_25, Nz, Ny, Nx, B, Lz):
+    """Parts 4 and 2, tiles that end early or span fields, one output, wide magnitudes; NaN and Inf stay in their line;
+    the entry points that route the same call agree bitwise."""
+    import torch
+    n = B * Ny * Nx
+    f = np.ascontiguousarray(np.tile(_lines64(Nz, 64, Nz), (1, n // 64 + 1))[:, :n])
+    bad = [n // 2] if n < 40 else [17, n // 2]
+    f[Nz // 3, bad[0]] = np.nan
+    f[0, bad[-1]] = np.inf if len(bad) > 1 else np.nan
+    f[:, 3] = 0
+    ft = torch.from_numpy(np.ascontiguousarray(f.reshape(Nz, B, Ny, Nx).transpose(1, 0, 2, 3))).cuda()
+    plan = api.Plan(5, 25, Nz)
+    d = [torch.full_like(ft, 7.0) for _ in range(2)]
+    api.fc_deriv_z(plan, ft, *d, Lz=Lz)
+    one = [torch.full_like(ft, 7.0) for _ in range(2)]
+    api.fc_deriv_z(plan, ft, one[0], None, Lz=Lz)
+    api.fc_deriv_z(plan, ft, None, one[1], Lz=Lz)
+    noa = [torch.full_like(ft, 7.0) for _ in range(2)]
+    assert api._lib.fc_deriv_z_noalloc(plan.handle, api.FC_F64, B, Nx, Ny, ctypes.c_double(Lz), ft.data_ptr(),
+                                       noa[0].data_ptr(), noa[1].data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+    h = [torch.empty(ft.shape, dtype=torch.float64) for _ in range(2)]
+    api.fc_deriv_z_host(plan, ft.cpu(), *h, Lz=Lz, slab_bytes=2 * Nz * Nx * 8)
+    torch.cuda.synchronize()
+    good = np.setdiff1d(np.arange(n), bad)
+    pick = np.unique(np.r_[good[:40], good[-20:]])
+    for o in range(2):
+        y = d[o].cpu().numpy().transpose(1, 0, 2, 3).reshape(Nz, n)
+        assert np.isfinite(y[:, good]).all() and np.isnan(y[:, bad]).all() and not y[:, 3].any()
+        err = np.abs(y[:, pick] - _derivative_ld(f[:, pick], Mr_5_25, o + 1, Lz)).max(axis=0)
+        bound = _bound64(f[:, pick], Mr_5_25, o + 1, Lz)
+        assert (err <= bound).all(), (o, np.nanmax(err / np.maximum(bound, 1e-300)))
+        for other in (one[o], noa[o].cpu(), h[o]):
+            z = other.cpu().numpy().transpose(1, 0, 2, 3).reshape(Nz, n)
+            assert np.array_equal(z, y, equal_nan=True)
