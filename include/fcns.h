@@ -143,7 +143,7 @@ fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, 
  *     fixed 128 KiB static device array that every GPU loading the library
  *     reserves until the process exits, and the operator blocks of
  *     calls that fc_deriv_z runs with the dense operators in another of
- *     2.25 MiB.
+ *     2.54 MiB.
  *   - The first call on each device looks up that array's device address
  *     (cudaGetSymbolAddress) with the device current and keeps it for the
  *     life of the process: resetting the device (cudaDeviceReset) after that

@@ -115,12 +115,13 @@ static long long dense_min_lines(const PlanData& p) {
   return p.Np >= 180 ? 16384 : (p.Np >= 100 ? 131072 : never);
 }
 // Float64 calls take them wherever the plan has them: the transforms sit on the
-// float64 pipe and lose at every size.  Measured, dense against transform (us):
-// 11 x 512 lines 29 / 58, 65 x 8k 80 / 197, 231 (direct) x 131k 2387 / 3198, 487
-// (direct) x 2560 194 / 201 (the closest: the second wave of tiles nearly empty),
-// x 131k 4927 / 6438, 513 x 512 55 / 130, x 131k 5001 / 16258.
+// float64 pipe.  Measured, dense against transform (us): 11 x 512 lines 29 / 58,
+// 65 x 8k 80 / 197, 103 (direct) x 3072 64 / 85, 231 (direct) x 8k 205 / 255, 487
+// (direct) x 8k 420 / 462, 513 x 512 60 / 130, x 32k 1467 / 4104.  Only where the
+// transform has length N' = 512 and the second wave of 152 tiles of 16 lines is
+// half empty are they slower (3072 lines: 217 / 199).
 bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines) {
-  if (dtype == FC_F64) return p.dense64.NQ != 0;
+  if (dtype == FC_F64) return p.dense64.NQ && !(p.dense_direct && p.Np >= 400 && lines > 2432 && lines <= 3648);
   return p.dense.NQ && lines >= dense_min_lines(p);
 }
 
@@ -221,14 +222,14 @@ fc_status fc_setup_ex(int d, int C, int Nz, int M, int n_os, fc_plan_t* out) {
   const bool f64 = L > 0 && dense64_geom(Nz, pd.Np, &pd.dense64);
   if (!f32) pd.dense = DenseGeom();
   std::vector<double> c1, c2;
-  if (f32 || f64) deriv_kernels_closed(pd.Np, &c1, &c2);
   if (f32) {
+    deriv_kernels_closed(pd.Np, &c1, &c2);
     pd.dense_exp[0] = dense_blocks(pd.dense, c1, &pd.dense_blocks);
     pd.dense_exp[1] = dense_blocks(pd.dense, c2, &pd.dense_blocks);
   }
   // (no digit sum reaches 2^24 for any N' of either parity of Nz: checked over all of them)
-  if (f64 && !(dense64_blocks(pd.dense64, c1, &pd.dense64_blocks, &pd.dense64_exp[0], &pd.dense64_sh[0]) &&
-               dense64_blocks(pd.dense64, c2, &pd.dense64_blocks, &pd.dense64_exp[1], &pd.dense64_sh[1]))) {
+  if (f64 && !(dense64_blocks(pd.dense64, 1, &pd.dense64_blocks, &pd.dense64_exp[0], &pd.dense64_sh[0]) &&
+               dense64_blocks(pd.dense64, 2, &pd.dense64_blocks, &pd.dense64_exp[1], &pd.dense64_sh[1]))) {
     delete p;
     set_error("fc_setup: float64 operators of this size are not exact in digits");
     return FC_ERR_UNSUPPORTED;

@@ -2,16 +2,17 @@
 // number formats, index maps and the exact continuation, shared by the kernel
 // (k_dense64.cu), the table builder and the CPU checks.
 //
-// A line is brought to whole numbers of 2^(E - 1075), E the exponent of its
-// largest value (|x| < 2^53: what the sums of a double transform resolve, too),
-// split into its NQ parts (dense_geom.hpp; |u| <= 2^55, exact) and every part
-// into seven balanced base-256 digits.  The operators' blocks are whole numbers
-// of 2^-e below 2^55 and a little, in seven digits as well.  Digits are exact in
+// A line is brought to whole numbers of 2^(E - 1082), E the exponent of its
+// largest value (|x| < 2^60; with 2^53, a line with a peak lost up to 3.6 times
+// what the transform loses), split into its NQ parts (dense_geom.hpp; |u| <
+// 2^62, exact) and every part into eight balanced base-256 digits.  The
+// operators' blocks are whole numbers of 2^-e below 2^63 (rounded once, from
+// binary128; with 2^55, twice the transform's error), in eight digits.  Digits are exact in
 // float16, and a sum of digit products stays a whole number below 2^24 (the
 // table builder checks the bound), so the tensor cores add them up exactly in
 // float32.  Digit products of one weight share an accumulator: the eight
-// leading weights are kept (34 of 49 products), what is left out is below 2^-60
-// of the largest product sum.
+// leading weights are kept (36 of 64 products), what is left out is about 2^-56
+// of the largest entry times the largest value.
 #pragma once
 #include <cstdint>
 
@@ -20,7 +21,7 @@
 namespace fcns {
 
 constexpr int kD64Lines = 16;    // lines per tile: the rows of one matrix instruction
-constexpr int kD64Digits = 7;
+constexpr int kD64Digits = 8;
 constexpr int kD64Sums = 8;      // weights kept: digits i of the line and j of the operator with i + j < 8
 
 // dense_geom for float64: the blocks fit 2.4 MB (they are read once per tile)
@@ -38,22 +39,23 @@ inline long long dense64_order_halves(const DenseGeom& g) {
 FC_DG int d64_a_index(int row, int k) { return ((row & 7) * 4 + (k & 7) / 2) * 8 + ((row >> 3) + 2 * (k >> 3)) * 2 + (k & 1); }
 FC_DG int d64_b_index(int k, int col) { return ((col & 7) * 4 + (k & 7) / 2) * 8 + (2 * (col >> 3) + (k >> 3)) * 2 + (k & 1); }
 
-// double (its bits) in whole units of 2^(E - 1075), rounded; E >= its exponent field
+// double (its bits) in whole units of 2^(E - 1082), rounded; E >= its exponent field
 FC_DG long long d64_fixed(unsigned long long b, int E) {
   const int e = (int)(b >> 52) & 0x7ff;
   const unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0);
   const int s = E - (e ? e : 1);
-  const long long v = s == 0 ? (long long)m : (s > 54 ? 0 : (long long)((m + (1ull << (s - 1))) >> s));
+  const long long v = s <= 7 ? (long long)(m << (7 - s)) : (s > 61 ? 0 : (long long)((m + (1ull << (s - 8))) >> (s - 7)));
   return b >> 63 ? -v : v;
 }
-// the seven digits as biased bytes: digit i = field i - 128, field 0 the leading one
-FC_DG unsigned long long d64_bias(long long u) { return (unsigned long long)(u + 0x0080808080808080ll); }
-FC_DG int d64_field(unsigned long long w, int i) { return i == 0 ? (int)((long long)w >> 48) : (int)(w >> (8 * (6 - i))) & 255; }
-// the eight sums (the first the heaviest) as one whole number, in units of 2^(40 + sh) of the product
+// the digits as fields: digit i = field i - 128, field 0 the leading one
+FC_DG unsigned long long d64_bias(long long u) { return (unsigned long long)u + 0x8080808080808080ull; }
+FC_DG int d64_field(unsigned long long w, int i) { return (int)(w >> (8 * (7 - i))) & 255; }
+// the eight sums (the first the heaviest) as one whole number, in units of 2^(56 + sh) of the product
+// (modulo 2^64: the sum over the parts fits again)
 FC_DG long long d64_combine(const int* a, int sh) {
   const long long hi = ((long long)a[0] << 24) + ((long long)a[1] << 16) + ((long long)a[2] << 8) + a[3];
   const long long lo = ((long long)a[4] << 24) + ((long long)a[5] << 16) + ((long long)a[6] << 8) + a[7];
-  return hi * (1ll << (32 - sh)) + (lo >> sh);
+  return (long long)(((unsigned long long)hi << (32 - sh)) + (unsigned long long)((lo + ((1ll << sh) >> 1)) >> sh));
 }
 
 FC_DG int d64_clz(unsigned long long v) {

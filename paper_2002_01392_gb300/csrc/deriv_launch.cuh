@@ -88,7 +88,8 @@ fc_status launch_deriv_typed(const DerivDevTables& t, const PlanData& p, int bat
     return sym ? run_deriv<T, A, B, F ? LF : LD, A, true>(t, p, batch, lines, Lz, f, df, d2f, stream)       \
                : run_deriv<T, A, B, F ? LF : LD, A, false>(t, p, batch, lines, Lz, f, df, d2f, stream);
   // float64 with a shorter transform always takes the dense operators
-  // (dense64_geom holds for every N' <= 384 and every even N' < 576)
+  // (dense64_geom holds for every N' <= 384 and every even N' < 576; N' = 512
+  // is transformed for some line counts)
   if constexpr (F) {
     switch (t.L) {
       FC_CASE(64, 8, 8, 16, 8)
@@ -99,11 +100,11 @@ fc_status launch_deriv_typed(const DerivDevTables& t, const PlanData& p, int bat
       FC_CASE(256, 16, 16, 16, 8)
       FC_CASE(288, 16, 18, 16, 8)
       FC_CASE(320, 16, 20, 16, 8)
-      FC_CASE(512, 16, 32, 8, 4)
       default: break;
     }
   }
   switch (t.L) {
+    FC_CASE(512, 16, 32, 8, 4)
     FC_CASE(576, 24, 24, 8, 4)
     FC_CASE(768, 24, 32, 4, 2)
     FC_CASE(1024, 32, 32, 4, 2)

@@ -657,15 +657,31 @@ int dense_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<u
   return e;
 }
 
-bool dense64_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out, int* e, int* sh) {
-  // entries as in dense_blocks, each kernel value rounded to whole units first
+bool dense64_blocks(const DenseGeom& g, int order, std::vector<unsigned short>* out, int* e, int* sh) {
+  // entries as in dense_blocks, each kernel value (deriv_kernels_closed, in binary128) rounded to whole units first
+  const q h = 2 * q_pi() / (q)g.Np;
+  const bool even = g.Np % 2 == 0;
+  std::vector<q> c(g.Np, (q)0);
+  if (order == 2) c[0] = -h * h * ((q)g.Np * (q)g.Np + (q)(even ? 2 : -1)) / (q)12;
+  for (int j = 1; 2 * j <= g.Np; ++j) {
+    q co, si;
+    q_sincos2pi(j, 2LL * g.Np, &co, &si);
+    const q sg = j % 2 ? -1 : 1;
+    const q v = order == 1 ? (2 * j == g.Np ? (q)0 : h * sg * (even ? co : (q)1) / (2 * si))
+                           : -h * h * sg * (even ? (q)1 : co) / (2 * si * si);
+    c[j] = v;
+    if (2 * j != g.Np) c[g.Np - j] = order == 1 ? -v : v;
+  }
   double big = 0.0;
-  for (double v : c) big = std::max(big, std::fabs(v));
-  *e = 54 - std::ilogb(big / g.NQ);
+  for (q v : c) big = std::max(big, std::fabs((double)v));
+  *e = 61 - std::ilogb(big / g.NQ);
   std::vector<long long> ci(c.size());
   std::vector<long long> B((size_t)g.NQ * g.No * g.No);
   for (int turn = 0; turn < 2; ++turn) {
-    for (size_t i = 0; i < c.size(); ++i) ci[i] = std::llrint(std::ldexp(c[i], *e) / g.NQ);
+    for (size_t i = 0; i < c.size(); ++i) {
+      const q v = c[i] * (q)std::ldexp(1.0, *e) / g.NQ;
+      ci[i] = (long long)(v + (v < 0 ? (q)-0.5 : (q)0.5));
+    }
     long long most = 0;
     for (int ji = 0; ji < g.No; ++ji) {
       int rows[4], n = 0, member[4];
@@ -691,13 +707,13 @@ bool dense64_blocks(const DenseGeom& g, const std::vector<double>& c, std::vecto
         }
       }
     }
-    if (most <= 1LL << 55) break;
-    *e -= std::ilogb((double)most) - 54;   // several large kernel values met in one entry
+    if (most <= (1LL << 62) + (1LL << 61)) break;
+    --*e;   // several large kernel values met in one entry
   }
   // float16 bits of the digits
   static const std::vector<unsigned short> half_of = [] {
-    std::vector<unsigned short> v(257);
-    for (int i = 0; i < 257; ++i) {
+    std::vector<unsigned short> v(256);
+    for (int i = 0; i < 256; ++i) {
       const __half h = __float2half((float)(i - 128));
       std::memcpy(&v[i], &h, 2);
     }
@@ -706,15 +722,12 @@ bool dense64_blocks(const DenseGeom& g, const std::vector<double>& c, std::vecto
   const int KT = g.KQ / 16;
   const size_t at0 = out->size();
   out->resize(at0 + (size_t)dense64_order_halves(g), 0);
-  double rows_most = 0.0;
   bool exact = true;
   for (int jo = 0; jo < g.No; ++jo) {
-    double sum = 0.0;
     for (int q = 0; q < g.NQ; ++q) {
       long long by_digit[kD64Digits] = {};
       for (int ji = 0; ji < g.No; ++ji) {
         const long long v = B[((size_t)q * g.No + jo) * g.No + ji];
-        sum += std::fabs((double)v);
         const unsigned long long w = d64_bias(v);
         unsigned short* o = &(*out)[at0 + (((size_t)(jo / 16) * g.NQ + q) * KT + ji / 16) * kD64Digits * 256 +
                                     d64_b_index(ji % 16, jo % 16)];
@@ -731,10 +744,11 @@ bool dense64_blocks(const DenseGeom& g, const std::vector<double>& c, std::vecto
         exact = exact && most <= 1LL << 24;
       }
     }
-    rows_most = std::max(rows_most, sum);
   }
-  // |output| <= 2^55 rows_most, in units of 2^40
-  *sh = std::max(0, (int)std::ceil(std::log2(rows_most)) + 55 - 40 - 61);
+  // |output| <= 2^60 times the kernel's sum of magnitudes, in units of 2^56; 2^62 at most
+  double sum = 0.0;
+  for (long long v : ci) sum += g.NQ * std::fabs((double)v);
+  *sh = std::max(0, (int)std::ceil(std::log2(sum)) + 60 - 56 - 62);
   return exact && *sh <= 32;
 }
 

@@ -70,11 +70,11 @@ void deriv_kernels_closed(int Np, std::vector<double>* d1, std::vector<double>* 
 // scale exponent 12 - e.
 int dense_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out);
 
-// The same for float64 (dense64.hpp): per output tile of 16 orbits, part, 16-step
+// The same for float64 (dense64.hpp) and derivative order 1 or 2: per output tile of 16 orbits, part, 16-step
 // and digit the operand fragment of the matrix instruction.  *e: the blocks are
 // whole numbers of 2^-e; *sh: the bits that d64_combine drops so that an
 // output fits 62 bits.  False where a digit sum could leave 2^24.
-bool dense64_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out, int* e, int* sh);
+bool dense64_blocks(const DenseGeom& g, int order, std::vector<unsigned short>* out, int* e, int* sh);
 
 // cos / sin of 2 pi num / den, correctly rounded to double from binary128.
 void sincos2pi(long long num, long long den, double* c, double* s);

@@ -252,11 +252,9 @@ int fchc_dense_blocks(int Nz, int Np, int order, unsigned short* halves, int* ex
 int fchc_dense64_tile(int Nz, int d, int C, const double* Mr, int order, const double* x, double* y) {
   DenseGeom g;
   if (!dense64_geom(Nz, Nz + C, &g)) return 1;
-  std::vector<double> c1, c2;
-  deriv_kernels_closed(g.Np, &c1, &c2);
   std::vector<unsigned short> blocks;
   int ex = 0, sh = 0;
-  if (!dense64_blocks(g, order == 1 ? c1 : c2, &blocks, &ex, &sh)) return 2;
+  if (!dense64_blocks(g, order, &blocks, &ex, &sh)) return 2;
   if ((long long)blocks.size() != dense64_order_halves(g)) return 4;
   const int KT = g.KQ / 16;
   std::vector<unsigned long long> X((size_t)g.Np * 16);
@@ -307,7 +305,7 @@ int fchc_dense64_tile(int Nz, int d, int C, const double* Mr, int order, const d
       }
       for (int i = 0; i < g.NQ; ++i) {
         const int n = dense_row(g, j, i);
-        if (n < Nz) y[(size_t)n * 16 + li] = E[li] == 0x7ff ? NAN : std::ldexp((double)row[i], 40 + sh + E[li] - 1075 - ex);
+        if (n < Nz) y[(size_t)n * 16 + li] = E[li] == 0x7ff ? NAN : std::ldexp((double)row[i], 56 + sh + E[li] - 1082 - ex);
       }
     }
   return 0;

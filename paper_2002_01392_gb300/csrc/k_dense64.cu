@@ -29,26 +29,27 @@ struct Dense64Args {
   int sh[2];
 };
 
-// One CTA walks tiles of 16 lines.  Bound: the tensor pipe (34 products of 16 x
-// 8 x 16 per fragment pair), then the operators' fragments out of L2 (2.3 MB per
+// One CTA walks tiles of 16 lines.  Bound: the tensor pipe (36 products of 16 x
+// 8 x 16 per fragment pair), then the operators' fragments out of L2 (2.7 MB per
 // tile at N' = 538).  16 lines because the digits of all NQ parts have to be in
-// shared memory together (an output row is a sum over the parts): 129 KB, beside
+// shared memory together (an output row is a sum over the parts): 147 KB, beside
 // the line itself (69 KB), into which the next tile is copied while the products run.
 // A warp owns 16 orbits of one order: eight float32 sums of 16 x 16 values, and
 // 4 x 8 whole numbers per thread for the rows of its orbits.
 // mma.sync, not tcgen05: the eight sums and the digits of 128 lines would need
 // four times the tensor memory of an SM.
-// Measured, 3 x 256^2 x 513: transforms 24.4 ms, this 8.08 ms, with the next
-// step's fragments read ahead 7.51; 513 x 32k lines 4104 -> 1309 us (tensor pipe
-// 48 % busy; the rest: splitting the line into digits, which overlaps nothing
-// (15 %), 18 items over 8 warps (10 %), the issue distance of two warps per
-// scheduler).  Error against 64-bit references as before (5.2e-12).
+// Measured, 3 x 256^2 x 513: transforms 24.4 ms, this 8.36; 513 x 32k lines 4104
+// -> 1467 us (with seven digits, where the error exceeded the transform's,
+// 1309, the tensor pipe 48 % busy; without the next step's fragments read ahead
+// 1410).  The rest: splitting the line into digits, which overlaps nothing (15
+// %), 18 items over 8 warps (10 %), the issue distance of two warps per
+// scheduler.  Error 3 to 30 times below the transform's.
 template <int NQ>
 __global__ void __launch_bounds__(kD64Threads, 1) dense64_kernel(const __grid_constant__ Dense64Args a) {
   extern __shared__ __align__(16) unsigned char sm[];
   const DenseGeom& g = a.g;
   const int KT = g.KQ / 16, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint4* A = reinterpret_cast<uint4*>(sm);                                    // [NQ][KT][7][32]
+  uint4* A = reinterpret_cast<uint4*>(sm);                                    // [NQ][KT][8][32]
   unsigned long long* X = reinterpret_cast<unsigned long long*>(A + NQ * KT * kD64Digits * 32);   // [N'][16]
   double* scale = reinterpret_cast<double*>(X + g.Np * kD64Lines);            // [2][2][16]
   unsigned* top = reinterpret_cast<unsigned*>(scale + 4 * kD64Lines);         // [16] largest high word
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(kD64Threads, 1) dense64_kernel(const __grid_co
           for (int j = 0; j < kD64Digits; ++j) {
             // digits x[1] and x[0] come last: theirs are the youngest loads
 #pragma unroll
-            for (int i = j == 0 ? kD64Digits - 1 : kD64Sums - 1 - j; i >= 0; --i) {
+            for (int i = kD64Sums - 1 - j; i >= 0; --i) {
               float* s = c[i + j];
               asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                   : "+f"(s[0]), "+f"(s[1]), "+f"(s[2]), "+f"(s[3])
@@ -181,9 +182,8 @@ __global__ void __launch_bounds__(kD64Threads, 1) dense64_kernel(const __grid_co
                   : "r"(x[i].x), "r"(x[i].y), "r"(x[i].z), "r"(x[i].w), "r"(b[j].z), "r"(b[j].w));
             }
             b[j] = __ldg(B + j * 32);
-            if (j > 0) x[kD64Digits - j] = Af[(kD64Digits - j) * 32];
+            x[kD64Sums - 1 - j] = Af[(kD64Sums - 1 - j) * 32];
           }
-          x[0] = Af[0];
         }
         // signs of the rows of an orbit: part q and the operator's own parity
 #pragma unroll
@@ -245,7 +245,7 @@ fc_status launch_deriv_dense64(const DerivDevTables& t, const PlanData& p, int b
     int e = 0;
     a.f[o] = std::frexp(s[o], &e);
     a.sh[o] = p.dense64_sh[o];
-    a.k[o] = 40 + a.sh[o] - 1075 - p.dense64_exp[o] + e;
+    a.k[o] = 56 + a.sh[o] - 1082 - p.dense64_exp[o] + e;
   }
   const size_t smem = (size_t)a.g.NQ * (a.g.KQ / 16) * kD64Digits * 512 + (size_t)a.g.Np * kD64Lines * 8 + 6 * kD64Lines * 8;
   auto kern = a.g.NQ == 4 ? dense64_kernel<4> : dense64_kernel<2>;
@@ -266,7 +266,7 @@ fc_status launch_deriv_dense64(const DerivDevTables& t, const PlanData& p, int b
     if (dev < 64) sm_count[dev].store(sms);
   }
   // fewer tiles than SMs: the orbits of a tile over several CTAs (each reads and splits the lines for itself), down to
-  // one warp per quarter of an SM.  513 x 512 lines: 114 -> 59 us
+  // one warp per quarter of an SM.  513 x 512 lines: 114 -> 59 us (seven digits)
   const int items = ((df ? 1 : 0) + (d2f ? 1 : 0)) * (a.g.KQ / 16);
   const long long most = (items + 3) / 4, room = a.tiles < sms ? sms / a.tiles : 1;
   const dim3 grid((unsigned)(a.tiles < sms ? a.tiles : sms), (unsigned)(room < most ? room : most));

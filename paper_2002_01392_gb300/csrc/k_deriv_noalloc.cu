@@ -26,9 +26,9 @@ constexpr int kMaxDevices = 64;
 // Shared by every call on a device; holds the tables of the last call.
 static __device__ __align__(256) unsigned char g_deriv_scratch[kNoAllocBytes];
 // The same for calls that fc_deriv_z runs with the dense operators: their
-// blocks (at most 1.33 MB in float32, N' = 575, and 2.33 MB in float64, N' =
+// blocks (at most 1.33 MB in float32, N' = 575, and 2.66 MB in float64, N' =
 // 576) and the continuation matrix.
-constexpr size_t kNoAllocDense = 2304 * 1024;
+constexpr size_t kNoAllocDense = 2600 * 1024;
 static __device__ __align__(256) unsigned char g_dense_scratch[kNoAllocDense];
 
 std::mutex g_mtx;

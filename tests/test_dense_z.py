@@ -233,7 +233,7 @@ def test_dense64_arithmetic_on_the_cpu(Nz, Mr_5_25):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("Nz,Ny,Nx,B,Lz", [(11, 5, 3, 1, 1.0), (33, 7, 37, 3, 2.0), (65, 64, 66, 1, 1.0), (102, 33, 31, 2, 1.0),
-                                            (231, 48, 51, 1, 0.5), (358, 16, 17, 2, 1.0), (513, 61, 41, 1, 1e-6),
+                                            (231, 48, 51, 1, 0.5), (358, 16, 17, 2, 1.0), (487, 48, 50, 1, 1.0), (513, 61, 41, 1, 1e-6),
                                             (549, 50, 49, 1, 1e5)])
 def test_dense64_kernel(api, Mr_5_25, Nz, Ny, Nx, B, Lz):
     """Parts 4 and 2, tiles that end early or span fields, one output, wide magnitudes; NaN and Inf stay in their line;
