@@ -368,6 +368,8 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       dz::workers_sync();
       if (redo[it & 1]) {
         atomicMax(lmax + line, __float_as_int(mx));   // (non-negative floats order like their bits)
+        // the first pass's tensor-memory stores are asynchronous and go to the columns the second one writes again
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         dz::workers_sync();
         dz::line_scale(__int_as_float(lmax[line]), 12, s1, s2);
         tiny = __any_sync(0xffffffffu, s2 != 1.f);

@@ -169,6 +169,38 @@ def test_dense_kernel_magnitudes_and_nonfinite(api, Mr_5_25):
         assert torch.equal(av[fin], b.view(torch.int32)[fin]) and torch.equal(av[fin], c.cpu().view(torch.int32)[fin])
 
 
+def _field_with_peaks(Nz, n, seed):
+    """Smooth lines of magnitude about 1; every 37th has a peak of 300 to 3e5 on a row between two sampled ones."""
+    r = np.random.default_rng(seed)
+    z = np.arange(Nz) / (Nz - 1)
+    f = np.sin(np.outer(z, r.uniform(3, 40, n)) + 1)
+    at = np.arange(0, n, 37)
+    every = (Nz + 31) // 32
+    f[r.integers(1, Nz // every - 1, at.size) * every + r.integers(1, every, at.size), at] = 10.0 ** r.uniform(2.5, 5.5, at.size)
+    return f.astype(np.float32)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("Nz", [513, 350])
+def test_dense_kernel_reloaded_tiles(api, Mr_5_25, Nz):
+    """Tiles whose sampled scale turns out too small are loaded twice: every line to its own bound, the same bits in
+    repeated calls."""
+    import torch
+    Ny, Nx = 8, 2560
+    f = _field_with_peaks(Nz, Ny * Nx, Nz)
+    ft = torch.from_numpy(f).cuda().view(1, Nz, Ny, Nx)
+    plan = api.Plan(5, 25, Nz)
+    d = [torch.empty_like(ft) for _ in range(2)]
+    e = [torch.empty_like(ft) for _ in range(2)]
+    api.fc_deriv_z(plan, ft, *d)
+    for _ in range(5):
+        api.fc_deriv_z(plan, ft, *e)
+        assert torch.equal(d[0], e[0]) and torch.equal(d[1], e[1])
+    for order in (1, 2):
+        err = np.linalg.norm(d[order - 1].view(Nz, -1).cpu().numpy() - _oracle(f, Mr_5_25, order), axis=0)
+        assert (err <= _bound(f, Mr_5_25, order)).all()
+
+
 # ---------------------------------------------------------------------------
 # float64: exact integer products (dense64.hpp)
 # ---------------------------------------------------------------------------
