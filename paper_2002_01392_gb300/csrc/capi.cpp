@@ -218,7 +218,7 @@ fc_status fc_setup_ex(int d, int C, int Nz, int M, int n_os, fc_plan_t* out) {
   }
   PlanData& pd = p->data;
   pd.dense_direct = L == pd.Np;
-  const bool f32 = L > 0 && dense_min_lines(pd) < (1LL << 31) && dense_geom(Nz, pd.Np, &pd.dense);
+  const bool f32 = L > 0 && dense_min_lines(pd) < (1LL << 31) && dense_plan(Nz, d, C, &pd.dense);
   const bool f64 = L > 0 && dense64_geom(Nz, pd.Np, &pd.dense64);
   if (!f32) pd.dense = DenseGeom();
   std::vector<double> c1, c2;

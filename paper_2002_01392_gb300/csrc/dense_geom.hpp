@@ -79,4 +79,36 @@ inline long long dense_order_halves(const DenseGeom& g) { return dense_block_hal
 // largest slab in bytes
 FC_DG int dense_slab_bytes(const DenseGeom& g) { return (g.per < g.KQ / 16 ? g.per : g.KQ / 16) * 16 * g.NC * 4; }
 
+// shared memory of the kernel (byte offsets) with `stages` slabs in the ring
+constexpr int kDenseBars = 28;   // barriers: full[8], empty[8], accumulators full[4], free[4], A ready, scouts full, free, end
+constexpr int kDenseSmemMax = 227 * 1024;
+struct DenseSmem {
+  int lo, ring, cont, scale, lmax, mr, bars, total;
+};
+inline DenseSmem dense_smem(const DenseGeom& g, int d, int C, int stages) {
+  DenseSmem s;
+  s.lo = 0;
+  s.ring = g.NQ * g.KQ * 2 * kDenseLines;
+  s.cont = s.ring + stages * dense_slab_bytes(g);
+  s.scale = s.cont + C * kDenseLines * 4;
+  s.lmax = s.scale + 2 * kDenseLines * 4;
+  s.mr = s.lmax + kDenseLines * 4 + 16;
+  s.bars = (s.mr + C * d * 8 + 15) / 16 * 16;
+  s.total = s.bars + 8 * kDenseBars + 16;
+  return s;
+}
+// slabs that fit (at most 8)
+inline int dense_stages(const DenseGeom& g, int d, int C) {
+  const int n = (kDenseSmemMax - dense_smem(g, d, C, 0).total) / dense_slab_bytes(g);
+  return n < 8 ? n : 8;
+}
+// geometry of a plan: the ring needs two slabs, and the continuation of d, C takes shared memory too (with N' above 510
+// and C from 48 on there is room for one only: such plans have no dense operators)
+inline bool dense_plan(int Nz, int d, int C, DenseGeom* o) {
+  DenseGeom g;
+  if (!dense_geom(Nz, Nz + C, &g) || dense_stages(g, d, C) < 2) return false;
+  *o = g;
+  return true;
+}
+
 }  // namespace fcns

@@ -69,25 +69,6 @@ struct DenseArgs {
 
 constexpr int kDenseWorkers = 512, kDenseScouts = 64, kDenseThreads = 640;
 
-// barriers: full[8], empty[8], accumulators full[4], free[4], A ready, scouts full, free, end
-constexpr int kDenseBars = 28;
-
-struct DenseSmem {         // byte offsets
-  int lo, ring, cont, scale, lmax, mr, bars, total;
-};
-inline DenseSmem dense_smem(const DenseGeom& g, int d, int C, int stages) {
-  DenseSmem s;
-  s.lo = 0;
-  s.ring = g.NQ * g.KQ * 2 * kDenseLines;
-  s.cont = s.ring + stages * dense_slab_bytes(g);
-  s.scale = s.cont + C * kDenseLines * 4;
-  s.lmax = s.scale + 2 * kDenseLines * 4;
-  s.mr = s.lmax + kDenseLines * 4 + 16;
-  s.bars = (s.mr + C * d * 8 + 15) / 16 * 16;
-  s.total = s.bars + 8 * kDenseBars + 16;
-  return s;
-}
-
 constexpr float kDenseLimit = 8192.f;    // largest scaled magnitude: a part is a sum of four values, below 2^15
 constexpr int kDenseSampleTo = 6;        // the sampled maximum is scaled to [2^6, 2^7): true maxima may be 64 times larger
 

@@ -225,6 +225,14 @@ int fchc_dense_geom(int Nz, int Np, int* out) {
   for (int i = 0; i < 6; ++i) out[i] = v[i];
   return 0;
 }
+// slabs in the ring of a plan's kernel and its shared memory in bytes; 0 where the plan has no dense operators
+int fchc_dense_plan(int Nz, int d, int C, int* smem) {
+  DenseGeom g;
+  if (!dense_plan(Nz, d, C, &g)) return 0;
+  const int n = dense_stages(g, d, C);
+  *smem = dense_smem(g, d, C, n).total;
+  return n;
+}
 int fchc_dense_row(int Nz, int Np, int j, int i) {
   DenseGeom g;
   return dense_geom(Nz, Np, &g) ? dense_row(g, j, i) : -1;

@@ -9,11 +9,9 @@ namespace fcns {
 
 static fc_status launch_dense(DenseArgs a, cudaStream_t stream) {
   // as many slabs as fit beside the tile; a block set that fits whole is loaded once per CTA
-  const int slab = dense_slab_bytes(a.g), room = 227 * 1024 - dense_smem(a.g, a.d, a.Cc, 0).total;
   const int nord = (a.orders & 1) + (a.orders >> 1);
   const int all = nord * a.g.chunks * a.g.NQ * a.g.slabs;
-  a.stages = room / slab < 8 ? room / slab : 8;
-  if (a.stages < 2) return FC_ERR_UNSUPPORTED;
+  a.stages = dense_stages(a.g, a.d, a.Cc);   // (at least two: dense_plan)
   a.resident = all <= a.stages ? 1 : 0;
   const DenseSmem so = dense_smem(a.g, a.d, a.Cc, a.stages);
   // d = 5 (the default continuation) is compiled on its own
@@ -25,7 +23,7 @@ static fc_status launch_dense(DenseArgs a, cudaStream_t stream) {
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 64 || !(attr.load() >> dev & 1ull)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseSmemMax);
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(dense z)");
     if (dev < 64) attr.fetch_or(1ull << dev);
   }

@@ -64,6 +64,23 @@ def test_dense_tables_are_the_derivative_operators(Nz, C):
         assert np.abs(y - ref).max() < 2.0 ** -22 * np.pi ** order * np.abs(x).max() * np.sqrt(Np)
 
 
+def test_dense_plans_have_room_for_two_slabs():
+    """Every d, C and Nz that fc_setup accepts: the continuation's shared memory leaves two slabs, or the plan has no
+    dense operators (and its calls take the transforms)."""
+    lib = _lib()
+    smem, left_out = ctypes.c_int(), 0
+    o = (ctypes.c_int * 6)()
+    for d in range(2, 11):
+        for C in range(d, 65):
+            for Nz in range(2 * d, 577 - C):
+                n = lib.fchc_dense_plan(Nz, d, C, ctypes.byref(smem))
+                if n:
+                    assert 2 <= n <= 8 and smem.value <= 227 * 1024
+                else:
+                    left_out += lib.fchc_dense_geom(Nz, Nz + C, o) == 0
+    assert left_out > 0
+
+
 # ---------------------------------------------------------------------------
 # the kernel (GPU)
 # ---------------------------------------------------------------------------
@@ -167,6 +184,27 @@ def test_dense_kernel_magnitudes_and_nonfinite(api, Mr_5_25):
         av = a.cpu().view(torch.int32)
         fin = torch.isfinite(a.cpu())
         assert torch.equal(av[fin], b.view(torch.int32)[fin]) and torch.equal(av[fin], c.cpu().view(torch.int32)[fin])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,C,Nz", [(5, 60, 500), (10, 64, 480), (7, 64, 461),      # no room for two slabs: transforms
+                                    (7, 33, 513), (2, 40, 257), (10, 25, 350), (9, 64, 200)])   # other d and C, N' even and odd
+def test_dense_continuations(api, d, C, Nz):
+    """Calls of the dense operators' size with other continuations than (5, 25)."""
+    import torch
+    Ny, Nx = 8, 2049
+    r = np.random.default_rng(Nz)
+    z = np.arange(Nz) / (Nz - 1)
+    f = (np.sin(np.outer(z, r.uniform(3, 40, Ny * Nx)) + 1) + 0.1 * z[:, None] ** 2).astype(np.float32)
+    plan = api.Plan(d, C, Nz)
+    Mr = plan.matrix()
+    ft = torch.from_numpy(f).cuda().view(1, Nz, Ny, Nx)
+    out = [torch.empty_like(ft) for _ in range(2)]
+    api.fc_deriv_z(plan, ft, *out)
+    pick = np.r_[0:128, 8000:8128, Ny * Nx - 129:Ny * Nx]
+    for order in (1, 2):
+        err = np.linalg.norm(out[order - 1].view(Nz, -1)[:, pick].cpu().numpy() - _oracle(f[:, pick], Mr, order), axis=0)
+        assert (err <= _bound(f[:, pick], Mr, order)).all()
 
 
 def _field_with_peaks(Nz, n, seed):
