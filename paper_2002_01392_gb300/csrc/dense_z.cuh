@@ -343,16 +343,19 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       };
       load_tile();
       // the scale came from a sample of the line: where a value passes the limit all the same (the float16 parts of the
-      // sums have to stay below 2^16), the tile is loaded again with the scale of the true maxima
+      // sums have to stay below 2^16), the tile is loaded again, that line with the scale of its true maximum
+      auto too_large = [&](float m) { return m * s1 * s2 > kDenseLimit || (m > 0.f && s1 == 0x1p126f && s2 == 1.f); };
       if (tid == 0) redo[(it + 1) & 1] = 0;
-      if (mx * s1 * s2 > kDenseLimit || (mx > 0.f && s1 == 0x1p126f && s2 == 1.f)) redo[it & 1] = 1;
+      if (too_large(mx)) redo[it & 1] = 1;
       dz::workers_sync();
       if (redo[it & 1]) {
         atomicMax(lmax + line, __float_as_int(mx));   // (non-negative floats order like their bits)
         // the first pass's tensor-memory stores are asynchronous and go to the columns the second one writes again
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         dz::workers_sync();
-        dz::line_scale(__int_as_float(lmax[line]), 12, s1, s2);
+        // only the lines that passed it get another scale: a line's bits do not depend on its neighbours in the tile
+        const float all = __int_as_float(lmax[line]);
+        if (too_large(all)) dz::line_scale(all, 12, s1, s2);
         tiny = __any_sync(0xffffffffu, s2 != 1.f);
         load_tile();
         dz::workers_sync();

@@ -239,6 +239,29 @@ def test_dense_kernel_reloaded_tiles(api, Mr_5_25, Nz):
         assert (err <= _bound(f, Mr_5_25, order)).all()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["peaks"])
+def test_dense_lines_do_not_depend_on_their_neighbours(api, kind):
+    """The bits of a line are the same in any order of the lines, and in the slabs of a host call as in one call."""
+    import torch
+    Nz, Ny, Nx = 513, 10, 2050
+    f = _field_with_peaks(Nz, Ny * Nx, 3)
+    ft = torch.from_numpy(f).cuda().view(1, Nz, Ny, Nx)
+    plan = api.Plan(5, 25, Nz)
+    d = [torch.empty_like(ft) for _ in range(2)]
+    api.fc_deriv_z(plan, ft, *d)
+    h = [torch.empty(ft.shape) for _ in range(2)]
+    api.fc_deriv_z_host(plan, ft.cpu(), *h, slab_bytes=2 * Nz * Nx * 4)
+    order = torch.randperm(Ny * Nx, generator=torch.Generator().manual_seed(1)).cuda()
+    mixed = ft.view(Nz, -1)[:, order].contiguous().view(ft.shape)
+    m = [torch.empty_like(ft) for _ in range(2)]
+    api.fc_deriv_z(plan, mixed, *m)
+    for a, b, c in zip(d, h, m):
+        bits = a.view(torch.int32).view(Nz, -1)
+        assert torch.equal(bits.cpu(), b.view(torch.int32).view(Nz, -1))
+        assert torch.equal(bits[:, order], c.view(torch.int32).view(Nz, -1))
+
+
 # ---------------------------------------------------------------------------
 # float64: exact integer products (dense64.hpp)
 # ---------------------------------------------------------------------------
