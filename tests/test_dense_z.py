@@ -188,7 +188,7 @@ def test_dense_kernel_magnitudes_and_nonfinite(api, Mr_5_25):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("d,C,Nz", [(5, 60, 500), (10, 64, 480), (7, 64, 461),      # no room for two slabs: transforms
-                                    (7, 33, 513), (2, 40, 257), (10, 25, 350), (9, 64, 200)])   # other d and C, N' even and odd
+                                    (7, 33, 513), (4, 40, 257), (10, 25, 350), (9, 64, 200)])   # other d and C, N' even and odd
 def test_dense_continuations(api, d, C, Nz):
     """Calls of the dense operators' size with other continuations than (5, 25)."""
     import torch
