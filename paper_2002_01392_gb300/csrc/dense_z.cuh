@@ -61,7 +61,8 @@ struct DenseArgs {
   const __half* B;         // blocks of both orders
   long long order_halves;
   const float2* Mr2;
-  float f1, f2;            // output factors (grid spacing and the blocks' scale)
+  float f[2];              // output factors (grid spacing and the blocks' scale): a number in [1, 2) times 2^fe
+  int fe[2];
   unsigned* err;           // error word (host memory), may be null
 };
 
@@ -361,7 +362,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
         dz::workers_sync();
         if (sub == 0) lmax[line] = 0;
       }
-      const float r1 = __frcp_rn(s1), r2 = __frcp_rn(s2);   // (powers of two)
+      const int k = (__float_as_int(s1) >> 23) + (__float_as_int(s2) >> 23) - 254;   // the line is scaled by 2^k
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       dz::fence_before();
@@ -373,10 +374,11 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       for (int o = 0; o < 2; ++o) {
         if (!(a.orders >> o & 1)) continue;
         float* out = (o == 0 ? a.out1 : a.out2) + grp * a.out_outer + off;
-        // the factor undoes the line's scale (r1 r2); in steps where their product would leave float's range
-        const float f = o == 0 ? a.f1 : a.f2, fp = f * r1;
-        const bool steps = __any_sync(0xffffffffu, tiny || !(fp > 1e-36f && fp < 1e36f));
-        const float fa = steps ? 1.f : fp;
+        // the factor undoes the line's scale; where it or its products could leave float's range, in steps
+        const int K = a.fe[o] - k;
+        const bool far = K < -80 || K > 80;
+        const bool steps = __any_sync(0xffffffffu, far);
+        const float fa = far ? 1.f : __int_as_float(__float_as_int(a.f[o]) + (K << 23));
         const float par = o == 0 ? -1.f : 1.f;
         for (int c = 0; c < g.chunks; ++c, ++step) {
           // each part's accumulators are handed back as soon as they are read, so that the MMAs of the next chunk
@@ -414,9 +416,11 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
                   Y[0][e] = fmaf(R, fa, P);
                   Y[1][e] = par * fmaf(-R, fa, P);
                 }
-                if (steps) {
+                if (steps) {   // (by 1 for the other lines: a line's bits do not depend on its neighbours in the warp)
+                  const int K1 = far ? min(max(K, -126), 127) : 0, K2 = far ? min(max(K - K1, -126), 127) : 0;
+                  const float f0 = far ? a.f[o] : 1.f, f1 = __int_as_float((K1 + 127) << 23), f2 = __int_as_float((K2 + 127) << 23);
 #pragma unroll
-                  for (int i = 0; i < NQ; ++i) Y[i][e] = ((Y[i][e] * r1) * f) * r2;
+                  for (int i = 0; i < NQ; ++i) Y[i][e] = ((Y[i][e] * f0) * f1) * f2;
                 }
               }
 #pragma unroll

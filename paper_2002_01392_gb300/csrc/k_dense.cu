@@ -62,9 +62,16 @@ fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int bat
   a.B = static_cast<const __half*>(t.dense);
   a.order_halves = dense_order_halves(a.g);
   a.Mr2 = t.Mr2;
-  const double dz = Lz / (p.Nz - 1);
-  a.f1 = (float)std::ldexp(1.0 / dz, -p.dense_exp[0]);
-  a.f2 = (float)std::ldexp(1.0 / (dz * dz), -p.dense_exp[1]);
+  const double dz = Lz / (p.Nz - 1), sc[2] = {1.0 / dz, 1.0 / (dz * dz)};
+  for (int o = 0; o < 2; ++o) {   // (at least 1 after rounding: frexp's mantissa is in [1/2, 1))
+    int e = 0;
+    a.f[o] = (float)(2 * std::frexp(sc[o], &e));
+    a.fe[o] = e - 1 - p.dense_exp[o];
+    if (!(sc[o] > 0) || std::isinf(sc[o])) {   // (no exponent: as a product)
+      a.f[o] = (float)sc[o];
+      a.fe[o] = 1000;
+    }
+  }
   a.err = t.dense_err;
   return launch_dense(a, stream);
 }

@@ -240,12 +240,31 @@ def test_dense_kernel_reloaded_tiles(api, Mr_5_25, Nz):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("kind", ["peaks"])
+@pytest.mark.parametrize("Lz,scale", [(1e23, 1e25), (1e12, 1.0), (1e-15, 1e-10)])
+def test_dense_kernel_extreme_heights(api, Mr_5_25, Lz, scale):
+    """Output factors 1 / dz and 1 / dz^2 that, with the operators' scale, leave float's range while the outputs do not."""
+    import torch
+    Nz, Ny, Nx = 513, 8, 2048
+    z = np.arange(Nz) / (Nz - 1)
+    f = (np.sin(np.outer(z, np.random.default_rng(1).uniform(3, 40, Ny * Nx)) + 1) * scale).astype(np.float32)
+    ft = torch.from_numpy(f).cuda().view(1, Nz, Ny, Nx)
+    plan = api.Plan(5, 25, Nz)
+    out = [torch.empty_like(ft) for _ in range(2)]
+    api.fc_deriv_z(plan, ft, *out, Lz=Lz)
+    for order in (1, 2):
+        err = np.linalg.norm(out[order - 1].view(Nz, -1)[:, :256].cpu().numpy() - _oracle(f[:, :256], Mr_5_25, order, Lz), axis=0)
+        assert (err <= _bound(f[:, :256], Mr_5_25, order, Lz)).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["peaks", "tiny"])
 def test_dense_lines_do_not_depend_on_their_neighbours(api, kind):
     """The bits of a line are the same in any order of the lines, and in the slabs of a host call as in one call."""
     import torch
     Nz, Ny, Nx = 513, 10, 2050
     f = _field_with_peaks(Nz, Ny * Nx, 3)
+    if kind == "tiny":
+        f[:, ::97] *= np.float32(1e-36)
     ft = torch.from_numpy(f).cuda().view(1, Nz, Ny, Nx)
     plan = api.Plan(5, 25, Nz)
     d = [torch.empty_like(ft) for _ in range(2)]
