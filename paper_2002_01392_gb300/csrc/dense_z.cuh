@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
         dz::workers_sync();
         if (sub == 0) lmax[line] = 0;
       }
-      const int k = (__float_as_int(s1) >> 23) + (__float_as_int(s2) >> 23) - 254;   // the line is scaled by 2^k
+      const int scaled = (__float_as_int(s1) >> 23) + (__float_as_int(s2) >> 23) - 254;   // the line is scaled by 2^scaled
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       dz::fence_before();
@@ -374,11 +374,12 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       for (int o = 0; o < 2; ++o) {
         if (!(a.orders >> o & 1)) continue;
         float* out = (o == 0 ? a.out1 : a.out2) + grp * a.out_outer + off;
-        // the factor undoes the line's scale; where it or its products could leave float's range, in steps
-        const int K = a.fe[o] - k;
+        // the factor undoes the line's scale: a.f 2^K.  Where that or a part times it could leave float's range, the
+        // accumulators take most of it first (by 1 for the other lines of the warp: a line's bits do not depend on them)
+        const int K = a.fe[o] - scaled, K1 = min(max(K, -100), 100);
         const bool far = K < -80 || K > 80;
         const bool steps = __any_sync(0xffffffffu, far);
-        const float fa = far ? 1.f : __int_as_float(__float_as_int(a.f[o]) + (K << 23));
+        const float fa = far ? __int_as_float((min(max(K - K1, -126), 127) + 127) << 23) : __int_as_float(__float_as_int(a.f[o]) + (K << 23));
         const float par = o == 0 ? -1.f : 1.f;
         for (int c = 0; c < g.chunks; ++c, ++step) {
           // each part's accumulators are handed back as soon as they are read, so that the MMAs of the next chunk
@@ -394,6 +395,17 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             dz::fence_before();
             dz::mbar_arrive(bFree + 8 * q);
+          }
+          if (steps) {
+            const int K = a.fe[o] - scaled;
+            const float f1 = K < -80 || K > 80 ? a.f[o] * __int_as_float((min(max(K, -100), 100) + 127) << 23) : 1.f;
+#pragma unroll
+            for (int k = 0; k < MG; ++k)
+#pragma unroll
+              for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                  if (k < ng) y[k][q][e] *= f1;
           }
           if (!valid) continue;
 #pragma unroll
@@ -415,12 +427,6 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
                   const float P = Y[0][e] * fa, R = Y[1][e];
                   Y[0][e] = fmaf(R, fa, P);
                   Y[1][e] = par * fmaf(-R, fa, P);
-                }
-                if (steps) {   // (by 1 for the other lines: a line's bits do not depend on its neighbours in the warp)
-                  const int K1 = far ? min(max(K, -126), 127) : 0, K2 = far ? min(max(K - K1, -126), 127) : 0;
-                  const float f0 = far ? a.f[o] : 1.f, f1 = __int_as_float((K1 + 127) << 23), f2 = __int_as_float((K2 + 127) << 23);
-#pragma unroll
-                  for (int i = 0; i < NQ; ++i) Y[i][e] = ((Y[i][e] * f0) * f1) * f2;
                 }
               }
 #pragma unroll
