@@ -63,7 +63,7 @@ inline bool dense_geom(int Nz, int Np, DenseGeom* o) {
   g.No = (m + fixed) / 2;
   g.KQ = (g.No + 15) / 16 * 16;
   if (g.NQ * g.KQ > kDenseMaxK) return false;
-  const int most = g.NQ == 4 ? 48 : 96;                        // accumulator columns: NQ * NC <= 192
+  const int most = 48;   // accumulator columns: NQ * NC, twice that for NQ = 2 (dense_z.cuh), up to 192
   g.chunks = (g.No + most - 1) / most;
   g.NC = ((g.No + g.chunks - 1) / g.chunks + 15) / 16 * 16;
   const int kt = g.KQ / 16, fit = 9 * 48 / g.NC;  // slabs of at most 27 KB

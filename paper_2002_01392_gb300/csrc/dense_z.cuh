@@ -7,8 +7,14 @@
 //
 // Precision: every float32 operand is split into two float16 values, high and
 // low (22 bits and a sign, of a line scaled by a power of two into float16's
-// range: from a sample of the line, checked against every value), and the products high x high, high x low and low
-// x high are accumulated in float32 (per slab, the small ones first).
+// range: from a sample of the line, checked against every value), and the
+// products high x high, high x low and low x high are accumulated in float32,
+// the small ones first (of NQ = 2, whose blocks come in several slabs, apart
+// from the large ones) and, where the contraction is short and the time of a
+// tile is its loads (KQ <= 48), low x low too.  Error of d/dz against the
+// transforms', 2-norm over rough lines: 0.47 to 0.95 for N' from 125 to 575
+// (1.01 and 0.92 at N' = 384); with the small products of NQ = 2 added to the
+// large sums it was up to 1.16.
 //
 // On-chip memory sets the shape: the split tile takes 4 bytes per value, 128 x
 // 576 x 4 = 288 KB, more than the 227 KB of shared memory, so the high parts
@@ -24,7 +30,7 @@
 //   warps 16-17 scouts: scale and continuation values of the next tile's lines,
 //               and its rows into L2
 //   warp 18     issues the MMAs;  warp 19 issues the bulk copies
-// Measured, d/dz and d2/dz2 of 3 x 512^2 x 513 float32: 1.70 ms (0.42 of the
+// Measured, d/dz and d2/dz2 of 3 x 512^2 x 513 float32: 1.69 ms (0.42 of the
 // measured HBM rate), against 2.91 ms for the length-1080 transforms, whose
 // arithmetic alone is bounded at 1.25 ms; error against 64 bits 2.1e-6 (2.7e-6).
 // A tile takes about 45 us on its SM: 13 us of loading and splitting (latency
@@ -49,7 +55,7 @@ namespace fcns {
 
 struct DenseArgs {
   DenseGeom g;
-  int d, Cc, stages, resident, orders;   // orders: bit 0 d/dz, bit 1 d2/dz2
+  int d, Cc, stages, resident, low_low, orders;   // orders: bit 0 d/dz, bit 1 d2/dz2
   int Zin;                 // rows of the input: Nz (the rest continued here) or N'
   long long per;           // lines of one group: adjacent in memory; the z stride
   long long in_outer, out_outer;   // elements between groups
@@ -156,28 +162,47 @@ __device__ __forceinline__ void mma_ss(unsigned d, unsigned a, unsigned b, unsig
       "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(kDescHi)
       : "memory");
 }
-__device__ __forceinline__ void mma_ts(unsigned d, unsigned a, unsigned b, unsigned idesc) {
+__device__ __forceinline__ void mma_ts(unsigned d, unsigned a, unsigned b, unsigned idesc, unsigned acc) {
   asm volatile(
-      "{\n.reg .pred p;\n.reg .b64 db;\nsetp.eq.u32 p, 0, 0;\nmov.b64 db, {%2, %4};\n"
+      "{\n.reg .pred p;\n.reg .b64 db;\nsetp.ne.u32 p, %4, 0;\nmov.b64 db, {%2, %5};\n"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n}" ::"r"(d),
-      "r"(a), "r"(b), "r"(idesc), "r"(kDescHi)
+      "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(kDescHi)
       : "memory");
 }
 // the products of one slab of n 16-steps (straight-line code: what one lane issues per MMA has to stay below the 31 cycles
-// it takes), then the arrivals on barriers be (slab read) and ba (accumulators done), where not 0
-template <int n>
-__device__ __forceinline__ void issue_slab(unsigned d, unsigned as, unsigned at, unsigned bh, unsigned bl, unsigned inc,
-                                           unsigned idesc, unsigned acc, unsigned be, unsigned ba) {
+// it takes): the small ones, low x high and high x low (and low x low where LL), into ds, then high x high into d, which may
+// be the same; then the arrivals on barriers be (slab read) and ba (accumulators done), where not 0
+template <int n, bool LL>
+__device__ __forceinline__ void issue_slab(unsigned d, unsigned ds, unsigned as, unsigned at, unsigned bh, unsigned bl,
+                                           unsigned inc, unsigned idesc, unsigned acc, unsigned be, unsigned ba) {
   if (elect()) {
-    mma_ss(d, as, bh, idesc, acc);
+    if (LL) {
 #pragma unroll
-    for (int k = 1; k < n; ++k) mma_ss(d, as + k * (kDenseLines * 2), bh + k * inc, idesc, 1);
+      for (int k = 0; k < n; ++k) mma_ss(ds, as + k * (kDenseLines * 2), bl + k * inc, idesc, k > 0 ? 1 : acc);
+    }
 #pragma unroll
-    for (int k = 0; k < n; ++k) mma_ts(d, at + 8 * k, bl + k * inc, idesc);
+    for (int k = 0; k < n; ++k) mma_ss(ds, as + k * (kDenseLines * 2), bh + k * inc, idesc, LL || k > 0 ? 1 : acc);
 #pragma unroll
-    for (int k = 0; k < n; ++k) mma_ts(d, at + 8 * k, bh + k * inc, idesc);
+    for (int k = 0; k < n; ++k) mma_ts(ds, at + 8 * k, bl + k * inc, idesc, 1);
+#pragma unroll
+    for (int k = 0; k < n; ++k) mma_ts(d, at + 8 * k, bh + k * inc, idesc, k > 0 || d == ds ? 1 : acc);
     if (be) mma_commit(be);
     if (ba) mma_commit(ba);
+  }
+}
+template <bool LL>
+__device__ __forceinline__ void issue_slab(int n, unsigned d, unsigned ds, unsigned as, unsigned at, unsigned bh, unsigned bl,
+                                           unsigned inc, unsigned idesc, unsigned acc, unsigned be, unsigned ba) {
+  switch (n) {
+    case 1: issue_slab<1, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    case 2: issue_slab<2, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    case 3: issue_slab<3, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    case 4: issue_slab<4, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    case 5: issue_slab<5, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    case 6: issue_slab<6, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    case 7: issue_slab<7, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    case 8: issue_slab<8, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
+    default: issue_slab<9, LL>(d, ds, as, at, bh, bl, inc, idesc, acc, be, ba); break;
   }
 }
 __device__ __forceinline__ void tmem_st4(unsigned addr, const unsigned (&v)[4]) {
@@ -258,6 +283,9 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
   const unsigned hiw = (unsigned)(NQ * g.KQ / 2);          // columns of the high parts; the accumulators follow
   const int nord = (a.orders & 1) + (a.orders >> 1);
   const int slabB = dense_slab_bytes(g);
+  // Of NQ = 2, the small products have accumulators of their own: added to the large sums of the slabs before, they would
+  // lose what the tensor cores cut off (not rounded) below 2^-24 of the sum.  A block of NQ = 4 is one slab.
+  constexpr int acc_sets = NQ == 2 ? 2 : 1;
 
   if (warp < 16) {
     // ------------------------------------------------------------- workers
@@ -370,7 +398,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       dz::mbar_arrive(bA);
       // --- outputs, chunk by chunk
       const int ng = g.NC / 16;   // groups of 4 orbits of this thread's quarter of a chunk
-      constexpr int MG = NQ == 4 ? 3 : 6;
+      constexpr int MG = 3;
       for (int o = 0; o < 2; ++o) {
         if (!(a.orders >> o & 1)) continue;
         float* out = (o == 0 ? a.out1 : a.out2) + grp * a.out_outer + off;
@@ -391,8 +419,23 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
             dz::fence_after();
 #pragma unroll
             for (int k = 0; k < MG; ++k)
-              if (k < ng) dz::tmem_ld4(tl + hiw + (unsigned)(q * g.NC + (sub * ng + k) * 4), y[k][q]);
+              if (k < ng) dz::tmem_ld4(tl + hiw + (unsigned)(q * acc_sets * g.NC + (sub * ng + k) * 4), y[k][q]);
+            float small[MG][4];
+            if constexpr (acc_sets == 2) {
+#pragma unroll
+              for (int k = 0; k < MG; ++k)
+                if (k < ng) dz::tmem_ld4(tl + hiw + (unsigned)((2 * q + 1) * g.NC + (sub * ng + k) * 4), small[k]);
+            }
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if constexpr (acc_sets == 2) {
+#pragma unroll
+              for (int k = 0; k < MG; ++k)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  asm volatile("" : "+f"(y[k][q][e]), "+f"(small[k][e]));   // (the sum stays behind the wait)
+                  if (k < ng) y[k][q][e] += small[k][e];
+                }
+            }
             dz::fence_before();
             dz::mbar_arrive(bFree + 8 * q);
           }
@@ -548,19 +591,10 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
             const int n = dense_slab(g, s);
             const unsigned bh = smb + so.ring + st * slabB, bl = bh + (unsigned)n * kstep;
             const unsigned da = dz::desc_lo(alo, kDenseLines * 16), dh = dz::desc_lo(bh, lbo), dl = dz::desc_lo(bl, lbo);
-            const bool last = s == g.slabs - 1;
-            const unsigned be = a.resident ? 0u : bempty + 8 * st, ba = last ? bAcc + 8 * q : 0u;
-            switch (n) {
-              case 1: dz::issue_slab<1>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              case 2: dz::issue_slab<2>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              case 3: dz::issue_slab<3>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              case 4: dz::issue_slab<4>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              case 5: dz::issue_slab<5>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              case 6: dz::issue_slab<6>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              case 7: dz::issue_slab<7>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              case 8: dz::issue_slab<8>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-              default: dz::issue_slab<9>(dcol, da, ahi, dh, dl, inc, idesc, acc, be, ba); break;
-            }
+            const unsigned ds = dcol + (NQ == 2 ? (unsigned)g.NC : 0u);
+            const unsigned be = a.resident ? 0u : bempty + 8 * st, ba = s == g.slabs - 1 ? bAcc + 8 * q : 0u;
+            if (NQ == 4 && a.low_low) dz::issue_slab<true>(n, dcol, ds, da, ahi, dh, dl, inc, idesc, acc, be, ba);
+            else dz::issue_slab<false>(n, dcol, ds, da, ahi, dh, dl, inc, idesc, acc, be, ba);
             __syncwarp();
             acc = 1;
             alo += (unsigned)n * (2 * kDenseLines * 16);
@@ -570,7 +604,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
               ph ^= 1;
             }
           }
-          dcol += (unsigned)g.NC;
+          dcol += (unsigned)(acc_sets * g.NC);
         }
       }
     }

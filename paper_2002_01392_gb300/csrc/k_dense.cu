@@ -13,6 +13,8 @@ static fc_status launch_dense(DenseArgs a, cudaStream_t stream) {
   const int all = nord * a.g.chunks * a.g.NQ * a.g.slabs;
   a.stages = dense_stages(a.g, a.d, a.Cc);   // (at least two: dense_plan)
   a.resident = all <= a.stages ? 1 : 0;
+  // low x low products where the contraction is short and the tile's time is its loads: see the header
+  a.low_low = a.g.NQ == 4 && a.g.KQ <= 48 ? 1 : 0;
   const DenseSmem so = dense_smem(a.g, a.d, a.Cc, a.stages);
   // d = 5 (the default continuation) is compiled on its own
   const int form = (a.g.NQ == 4 ? 1 : 0) + (a.d == 5 ? 2 : 0);

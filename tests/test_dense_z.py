@@ -240,6 +240,32 @@ def test_dense_kernel_reloaded_tiles(api, Mr_5_25, Nz):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("Nz,lines", [(129, 131072), (512, 16384), (513, 16384), (520, 16384)])
+def test_dense_kernel_is_no_less_exact_than_the_transforms(api, Nz, lines):
+    """Rough lines (an inertial-range spectrum, smooth at the walls): the error against the float64 derivatives, in the
+    2-norm, of the dense operators and of the transforms, which a call of few lines takes."""
+    import torch
+    r = np.random.default_rng(Nz)
+    z = np.arange(Nz) / (Nz - 1)
+    k = np.arange(1, 2 * (Nz - 1) // 3 + 1)
+    i = np.minimum(np.arange(Nz), np.arange(Nz)[::-1])
+    damp = np.sin(0.5 * np.pi * np.clip((i - 5) / 10, 0, 1)) ** 2
+    prof = [damp * (k[:, None] ** (-5 / 6) * np.cos(np.pi * np.outer(k, z) + 2 * np.pi * r.random((k.size, 1)))).sum(0)
+            + np.cos(r.uniform(1, 9) * z + r.uniform(0, 6)) for _ in range(8)]
+    f = torch.from_numpy((np.array(prof).T @ r.standard_normal((8, lines))).astype(np.float32)).cuda().view(1, Nz, 1, lines)
+    part = f[..., :4096].contiguous()
+    plan = api.Plan(5, 25, Nz)
+    outs = []
+    for x in (f, part, part.double()):
+        o = [torch.empty_like(x) for _ in range(2)]
+        api.fc_deriv_z(plan, x, *o)
+        outs.append([t[..., :4096].double() for t in o])
+    for dense, transform, exact in zip(*outs):
+        assert not torch.equal(dense, transform)      # two routes
+        assert (dense - exact).norm() <= (transform - exact).norm()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("Lz,scale", [(1e23, 1e25), (1e12, 1.0), (1e-15, 1e-10)])
 def test_dense_kernel_extreme_heights(api, Mr_5_25, Lz, scale):
     """Output factors 1 / dz and 1 / dz^2 that, with the operators' scale, leave float's range while the outputs do not."""
