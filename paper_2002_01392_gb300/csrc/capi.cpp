@@ -221,19 +221,8 @@ fc_status fc_setup_ex(int d, int C, int Nz, int M, int n_os, fc_plan_t* out) {
   const bool f32 = L > 0 && dense_min_lines(pd) < (1LL << 31) && dense_plan(Nz, d, C, &pd.dense);
   const bool f64 = L > 0 && dense64_geom(Nz, pd.Np, &pd.dense64);
   if (!f32) pd.dense = DenseGeom();
-  std::vector<double> c1, c2;
-  if (f32) {
-    deriv_kernels_closed(pd.Np, &c1, &c2);
-    pd.dense_exp[0] = dense_blocks(pd.dense, c1, &pd.dense_blocks);
-    pd.dense_exp[1] = dense_blocks(pd.dense, c2, &pd.dense_blocks);
-  }
-  // (no digit sum reaches 2^24 for any N' of either parity of Nz: checked over all of them)
-  if (f64 && !(dense64_blocks(pd.dense64, 1, &pd.dense64_blocks, &pd.dense64_exp[0], &pd.dense64_sh[0]) &&
-               dense64_blocks(pd.dense64, 2, &pd.dense64_blocks, &pd.dense64_exp[1], &pd.dense64_sh[1]))) {
-    delete p;
-    set_error("fc_setup: float64 operators of this size are not exact in digits");
-    return FC_ERR_UNSUPPORTED;
-  }
+  if (!f64) pd.dense64 = DenseGeom();
+  if (f32 || f64) dense_kernels(f32 ? pd.dense : pd.dense64, &pd.kern);
   *out = p;
   return FC_OK;
 }
@@ -266,9 +255,7 @@ fc_status fc_destroy(fc_plan_t plan) {
     for (auto& t : plan->data.dev) {
       cudaSetDevice(t.device);
       cudaDeviceSynchronize();
-      cudaFree(t.Mr); cudaFree(t.Mr2); cudaFree(t.tw32); cudaFree(t.tw64);
-      cudaFree(t.H1_32); cudaFree(t.H1_64); cudaFree(t.H2_32); cudaFree(t.H2_64);
-      cudaFree(t.dense); cudaFree(t.dense64);
+      cudaFree(t.block);
       if (t.dense_err) cudaFreeHost(t.dense_err);
       for (auto& slot : t.stage)
         for (void* b : slot) cudaFree(b);
@@ -291,15 +278,6 @@ fc_status fc_destroy(fc_plan_t plan) {
 
 namespace fcns {
 
-template <class C>
-static fc_status upload(const std::vector<std::complex<double>>& v, void** dst) {
-  std::vector<C> h(v.size());
-  for (size_t i = 0; i < v.size(); ++i) { h[i].x = (decltype(h[i].x))v[i].real(); h[i].y = (decltype(h[i].y))v[i].imag(); }
-  fc_status s = cuda_status(cudaMalloc(dst, sizeof(C) * h.size()), "cudaMalloc(tables)");
-  if (s) return s;
-  return cuda_status(cudaMemcpy(*dst, h.data(), sizeof(C) * h.size(), cudaMemcpyHostToDevice), "cudaMemcpy(tables)");
-}
-
 static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
   int dev = -1;
   fc_status s = cuda_status(cudaGetDevice(&dev), "cudaGetDevice");
@@ -310,38 +288,49 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
     set_error("fc_deriv_z: more devices than the plan supports (64)");
     return FC_ERR_UNSUPPORTED;
   }
+  // every table in one allocation and one copy; the dense operators' blocks behind them, built on the device
+  const PlanData& pd = plan->data;
+  const PlanHostTables& h = plan->deriv;
+  std::vector<unsigned char> up;
+  auto put = [&up](const void* src, size_t bytes) {
+    const size_t at = (up.size() + 255) & ~(size_t)255;
+    up.resize(at + bytes);
+    std::memcpy(up.data() + at, src, bytes);
+    return at;
+  };
+  const size_t L = h.L;
+  const size_t oMr = put(pd.Mr.data(), sizeof(double) * pd.Mr.size()), oMr2 = put(h.Mr2.data(), sizeof(float2) * h.Mr2.size());
+  const size_t oH1 = put(h.H1_32.data(), 8 * L), oH2 = put(h.H2_32.data(), 8 * L), oT = put(h.tw32.data(), 16 * L);
+  const size_t oG1 = put(h.H1_64.data(), 16 * L), oG2 = put(h.H2_64.data(), 16 * L), oU = put(h.tw64.data(), 32 * L);
+  const size_t oC = pd.dense.NQ ? put(pd.kern.c.data(), 8 * pd.kern.c.size()) : 0;
+  const size_t oI = pd.dense64.NQ ? put(pd.kern.ci.data(), 8 * pd.kern.ci.size()) : 0;
+  const size_t oB = (up.size() + 255) & ~(size_t)255, oB64 = oB + dense_bytes(pd), total = oB64 + dense64_bytes(pd);
   DerivDevTables t;
   t.device = dev;
-  t.L = plan->deriv.L;
-  s = cuda_status(cudaMalloc((void**)&t.Mr, sizeof(double) * plan->data.Mr.size()), "cudaMalloc(Mr)");
-  if (!s) s = cuda_status(cudaMemcpy(t.Mr, plan->data.Mr.data(), sizeof(double) * plan->data.Mr.size(),
-                                     cudaMemcpyHostToDevice), "cudaMemcpy(Mr)");
-  if (!s) s = cuda_status(cudaMalloc((void**)&t.Mr2, sizeof(float2) * plan->deriv.Mr2.size()), "cudaMalloc(Mr2)");
-  if (!s) s = cuda_status(cudaMemcpy(t.Mr2, plan->deriv.Mr2.data(), sizeof(float2) * plan->deriv.Mr2.size(),
-                                     cudaMemcpyHostToDevice), "cudaMemcpy(Mr2)");
-  auto up = [&](const void* src, size_t bytes, void** dst) {
-    fc_status st = cuda_status(cudaMalloc(dst, bytes), "cudaMalloc(tables)");
-    if (!st) st = cuda_status(cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice), "cudaMemcpy(tables)");
-    return st;
-  };
-  const size_t L = plan->deriv.L;
-  if (!s) s = up(plan->deriv.H1_32.data(), 8 * L, &t.H1_32);
-  if (!s) s = up(plan->deriv.H2_32.data(), 8 * L, &t.H2_32);
-  if (!s) s = up(plan->deriv.H1_64.data(), 16 * L, &t.H1_64);
-  if (!s) s = up(plan->deriv.H2_64.data(), 16 * L, &t.H2_64);
-  if (!s) s = upload<float2>(plan->deriv.tw, &t.tw32);
-  if (!s) s = upload<double2>(plan->deriv.tw, &t.tw64);
-  if (!s && plan->data.dense.NQ) {
-    s = up(plan->data.dense_blocks.data(), 2 * plan->data.dense_blocks.size(), &t.dense);
+  t.L = h.L;
+  s = cuda_status(cudaMalloc(&t.block, total), "cudaMalloc(tables)");
+  if (s) return s;
+  unsigned char* at = static_cast<unsigned char*>(t.block);
+  t.Mr = reinterpret_cast<double*>(at + oMr);
+  t.Mr2 = reinterpret_cast<float2*>(at + oMr2);
+  t.H1_32 = at + oH1; t.H2_32 = at + oH2; t.tw32 = at + oT;
+  t.H1_64 = at + oG1; t.H2_64 = at + oG2; t.tw64 = at + oU;
+  s = cuda_status(cudaMemcpy(at, up.data(), up.size(), cudaMemcpyHostToDevice), "cudaMemcpy(tables)");
+  if (!s && pd.dense.NQ) {
+    t.dense = at + oB;
+    s = launch_dense_build(pd, reinterpret_cast<const double*>(at + oC), t.dense, nullptr);
     if (!s) s = cuda_status(cudaHostAlloc((void**)&t.dense_err, sizeof(unsigned), cudaHostAllocDefault), "cudaHostAlloc");
     if (!s) *t.dense_err = 0;
   }
-  if (!s && plan->data.dense64.NQ) s = up(plan->data.dense64_blocks.data(), 2 * plan->data.dense64_blocks.size(), &t.dense64);
+  if (!s && pd.dense64.NQ) {
+    t.dense64 = at + oB64;
+    s = launch_dense64_build(pd, reinterpret_cast<const long long*>(at + oI), t.dense64, nullptr);
+  }
+  // in place before any stream reads them, non-blocking ones too
+  if (!s) s = cuda_status(cudaStreamSynchronize(nullptr), "cudaStreamSynchronize(tables)");
   if (s) {
-    cudaFree(t.Mr); cudaFree(t.Mr2); cudaFree(t.tw32); cudaFree(t.tw64);
-      cudaFree(t.H1_32); cudaFree(t.H1_64); cudaFree(t.H2_32); cudaFree(t.H2_64);
-      cudaFree(t.dense); cudaFree(t.dense64);
-      if (t.dense_err) cudaFreeHost(t.dense_err);
+    cudaFree(t.block);
+    if (t.dense_err) cudaFreeHost(t.dense_err);
     return s;
   }
   plan->data.dev.push_back(t);

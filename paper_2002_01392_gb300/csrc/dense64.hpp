@@ -31,7 +31,7 @@ inline bool dense64_geom(int Nz, int Np, DenseGeom* o) {
   *o = g;
   return true;
 }
-inline long long dense64_order_halves(const DenseGeom& g) {
+FC_DG long long dense64_order_halves(const DenseGeom& g) {
   return (long long)(g.KQ / 16) * g.NQ * (g.KQ / 16) * kD64Digits * 32 * 8;
 }
 // operand fragments of the 16 x 8 x 16 matrix instruction: lane and half of

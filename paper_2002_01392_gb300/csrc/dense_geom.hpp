@@ -74,8 +74,8 @@ inline bool dense_geom(int Nz, int Np, DenseGeom* o) {
   return true;
 }
 // halves of one slab's high (or low) part, of a block, and of one order
-inline long long dense_block_halves(const DenseGeom& g) { return 2LL * g.KQ * g.NC; }
-inline long long dense_order_halves(const DenseGeom& g) { return dense_block_halves(g) * g.chunks * g.NQ; }
+FC_DG long long dense_block_halves(const DenseGeom& g) { return 2LL * g.KQ * g.NC; }
+FC_DG long long dense_order_halves(const DenseGeom& g) { return dense_block_halves(g) * g.chunks * g.NQ; }
 // largest slab in bytes
 FC_DG int dense_slab_bytes(const DenseGeom& g) { return (g.per < g.KQ / 16 ? g.per : g.KQ / 16) * 16 * g.NC * 4; }
 

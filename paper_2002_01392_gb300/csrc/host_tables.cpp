@@ -9,13 +9,8 @@
 // [1 - delta_r, 2b - (1 - delta_r)] (2(d + C) grid spacings).  The right-end
 // matrix is M_r = A_r Q_r^T (App. B, eq. Af).
 #include "host_tables.hpp"
-#include "dense64.hpp"
-
-#include <cuda_fp16.h>
-
 
 #include <cmath>
-#include <cstring>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -579,177 +574,78 @@ void engine_twiddles(int L1, int L2, std::vector<std::complex<double>>* tw) {
     }
 }
 
-void deriv_kernels_closed(int Np, std::vector<double>* d1, std::vector<double>* d2) {
-  // sums over the modes of i k e^{ikj} / N' and -k^2 e^{ikj} / N', k = 2 pi l / N'
-  const double h = 2 * M_PI / Np;
-  d1->assign(Np, 0.0);
-  d2->assign(Np, 0.0);
+void dense_kernels(const DenseGeom& g, DenseKernels* o) {
+  const int Np = g.Np;
   const bool even = Np % 2 == 0;
-  (*d2)[0] = -h * h * ((double)Np * Np + (even ? 2.0 : -1.0)) / 12.0;
+  // sums over the modes of i k e^{ikj} / N' and -k^2 e^{ikj} / N', k = 2 pi l / N', in closed form, in binary128
+  // (cosine and sine of pi j / N' by angle addition: 2^-113 per step)
+  const q h = 2 * q_pi() / (q)Np;
+  q c1, s1;
+  q_sincos2pi(1, 2LL * Np, &c1, &s1);
+  std::vector<q> c[2] = {std::vector<q>(Np, (q)0), std::vector<q>(Np, (q)0)};
+  c[1][0] = -h * h * ((q)Np * (q)Np + (q)(even ? 2 : -1)) / (q)12;
+  q co = c1, si = s1;
   for (int j = 1; 2 * j <= Np; ++j) {
-    double c, s;   // of pi j / N'
-    sincos2pi(j, 2LL * Np, &c, &s);
-    const double sg = j % 2 ? -1.0 : 1.0;
-    const double v1 = 2 * j == Np ? 0.0 : 0.5 * h * sg * (even ? c : 1.0) / s;
-    const double v2 = -h * h * sg * (even ? 1.0 : c) / (2 * s * s);
-    (*d1)[j] = v1;
-    if (2 * j != Np) (*d1)[Np - j] = -v1;
-    (*d2)[j] = (*d2)[Np - j] = v2;
+    const q w = (j % 2 ? -h : h) / (2 * si), v = -h * w / si;   // -+ h / (2 s), +- h^2 / (2 s^2)
+    const q d1 = 2 * j == Np ? (q)0 : (even ? w * co : w), d2 = even ? v : v * co;
+    c[0][j] = d1;
+    if (2 * j != Np) c[0][Np - j] = -d1;
+    c[1][j] = c[1][Np - j] = d2;
+    const q t = co * c1 - si * s1;
+    si = si * c1 + co * s1;
+    co = t;
   }
-}
-
-int dense_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out) {
-  // B(jo, ji) of part (s, m): sum over the distinct rows n of orbit ji of
-  // sign(n) c(n0(jo) - n) / NQ, sign = 1, m, s, s m for the four members
-  std::vector<double> B((size_t)g.NQ * g.No * g.No);
-  double most = 0.0;
-  for (int ji = 0; ji < g.No; ++ji) {
-    int rows[4], n = 0, member[4];
-    for (int i = 0; i < g.NQ; ++i) {
-      const int r = dense_row(g, ji, i);
-      bool seen = false;
-      for (int k = 0; k < n; ++k) seen = seen || rows[k] == r;
-      if (seen) continue;
-      rows[n] = r;
-      member[n++] = i;
+  o->c.resize(2 * (size_t)Np);
+  o->ci.resize(2 * (size_t)Np);
+  for (int k = 0; k < 2; ++k) {
+    double* d = o->c.data() + (size_t)k * Np;
+    double big = 0.0, sum = 0.0;
+    for (int j = 0; j < Np; ++j) {
+      d[j] = (double)c[k][j];
+      big = std::max(big, std::fabs(d[j]));
+      sum += std::fabs(d[j]);
     }
-    for (int jo = 0; jo < g.No; ++jo) {
-      const int n0 = dense_row(g, jo, 0);
-      for (int q = 0; q < g.NQ; ++q) {   // q & 1: m = -1, q & 2: s = -1
-        double v = 0.0;
-        for (int k = 0; k < n; ++k) {
-          const int neg = ((q & member[k] & 1) + ((q & member[k] & 2) >> 1)) & 1;
-          const double x = c[((n0 - rows[k]) % g.Np + g.Np) % g.Np];
-          v += neg ? -x : x;
-        }
-        v /= g.NQ;
-        B[((size_t)q * g.No + jo) * g.No + ji] = v;
-        most = std::max(most, std::fabs(v));
-      }
-    }
-  }
-  const int e = 12 - (most > 0.0 ? std::ilogb(most) : 0);
-  const double sc = std::ldexp(1.0, e);
-  auto half_bits = [](double v, double* back) {
-    const __half h = __double2half(v);
-    *back = (double)__half2float(h);
-    unsigned short b;
-    std::memcpy(&b, &h, 2);
-    return b;
-  };
-  out->reserve(out->size() + (size_t)dense_order_halves(g));
-  std::vector<unsigned short> low;
-  for (int ch = 0; ch < g.chunks; ++ch)
-    for (int q = 0; q < g.NQ; ++q)
-      for (int s = 0; s < g.slabs; ++s) {
-        low.clear();
-        for (int kc = 2 * s * g.per; kc < 2 * (s * g.per + dense_slab(g, s)); ++kc)
-          for (int r = 0; r < g.NC; ++r)
-            for (int k = 0; k < 8; ++k) {
-              const int jo = ch * g.NC + r, ji = kc * 8 + k;
-              const double v = jo < g.No && ji < g.No ? sc * B[((size_t)q * g.No + jo) * g.No + ji] : 0.0;
-              double hv, lv;
-              out->push_back(half_bits(v, &hv));
-              low.push_back(half_bits(v - hv, &lv));
-            }
-        out->insert(out->end(), low.begin(), low.end());
-      }
-  return e;
-}
-
-bool dense64_blocks(const DenseGeom& g, int order, std::vector<unsigned short>* out, int* e, int* sh) {
-  // entries as in dense_blocks, each kernel value (deriv_kernels_closed, in binary128) rounded to whole units first
-  const q h = 2 * q_pi() / (q)g.Np;
-  const bool even = g.Np % 2 == 0;
-  std::vector<q> c(g.Np, (q)0);
-  if (order == 2) c[0] = -h * h * ((q)g.Np * (q)g.Np + (q)(even ? 2 : -1)) / (q)12;
-  for (int j = 1; 2 * j <= g.Np; ++j) {
-    q co, si;
-    q_sincos2pi(j, 2LL * g.Np, &co, &si);
-    const q sg = j % 2 ? -1 : 1;
-    const q v = order == 1 ? (2 * j == g.Np ? (q)0 : h * sg * (even ? co : (q)1) / (2 * si))
-                           : -h * h * sg * (even ? (q)1 : co) / (2 * si * si);
-    c[j] = v;
-    if (2 * j != g.Np) c[g.Np - j] = order == 1 ? -v : v;
-  }
-  double big = 0.0;
-  for (q v : c) big = std::max(big, std::fabs((double)v));
-  *e = 61 - std::ilogb(big / g.NQ);
-  std::vector<long long> ci(c.size());
-  std::vector<long long> B((size_t)g.NQ * g.No * g.No);
-  for (int turn = 0; turn < 2; ++turn) {
-    for (size_t i = 0; i < c.size(); ++i) {
-      const q v = c[i] * (q)std::ldexp(1.0, *e) / g.NQ;
-      ci[i] = (long long)(v + (v < 0 ? (q)-0.5 : (q)0.5));
-    }
-    long long most = 0;
+    // largest entry of the blocks: the kernel twice in a row, so that a row of entries is read in order
+    std::vector<double> two(d, d + Np);
+    two.insert(two.end(), d, d + Np);
+    double most = 0.0;
+    const int first = dense_row(g, 0, 0);
     for (int ji = 0; ji < g.No; ++ji) {
-      int rows[4], n = 0, member[4];
+      const double* at[4];
+      double on[4];
+      int rows[4];
       for (int i = 0; i < g.NQ; ++i) {
-        const int r = dense_row(g, ji, i);
-        bool seen = false;
-        for (int k = 0; k < n; ++k) seen = seen || rows[k] == r;
-        if (seen) continue;
-        rows[n] = r;
-        member[n++] = i;
+        rows[i] = dense_row(g, ji, i);
+        on[i] = 1.0;
+        for (int p = 0; p < i; ++p)
+          if (rows[p] == rows[i]) on[i] = 0.0;
+        at[i] = two.data() + ((first - rows[i]) % Np + Np) % Np;
       }
+      // (first + jo stays below N' + N'/2, so an index stays within the two copies)
       for (int jo = 0; jo < g.No; ++jo) {
-        const int n0 = dense_row(g, jo, 0);
-        for (int q = 0; q < g.NQ; ++q) {
-          long long v = 0;
-          for (int k = 0; k < n; ++k) {
-            const int neg = ((q & member[k] & 1) + ((q & member[k] & 2) >> 1)) & 1;
-            const long long x = ci[n0 - rows[k] + (n0 < rows[k] ? g.Np : 0)];
-            v += neg ? -x : x;
-          }
-          B[((size_t)q * g.No + jo) * g.No + ji] = v;
-          most = std::max(most, v < 0 ? -v : v);
+        const double x0 = on[0] * at[0][jo], x1 = on[1] * at[1][jo];
+        if (g.NQ == 4) {   // the largest of the four parts' |(x0 +- x1) +- (x2 +- x3)|, equal signs inside
+          const double x2 = on[2] * at[2][jo], x3 = on[3] * at[3][jo];
+          most = std::max(most, std::max(std::fabs(x0 + x1) + std::fabs(x2 + x3), std::fabs(x0 - x1) + std::fabs(x2 - x3)));
+        } else {
+          most = std::max(most, std::fabs(x0) + std::fabs(x1));
         }
       }
     }
-    if (most <= (1LL << 62) + (1LL << 61)) break;
-    --*e;   // several large kernel values met in one entry
-  }
-  // float16 bits of the digits
-  static const std::vector<unsigned short> half_of = [] {
-    std::vector<unsigned short> v(256);
-    for (int i = 0; i < 256; ++i) {
-      const __half h = __float2half((float)(i - 128));
-      std::memcpy(&v[i], &h, 2);
+    most /= g.NQ;
+    o->e[k] = 12 - (most > 0.0 ? std::ilogb(most) : 0);
+    // float64: whole units of 2^-e64, entries below 1.5 2^62 (several large kernel values can meet in one)
+    int e = 61 - std::ilogb(big / g.NQ);
+    if (std::ldexp(most, e) > std::ldexp(1.5, 62)) --e;
+    o->e64[k] = e;
+    const q unit = (q)std::ldexp(1.0, e) / g.NQ;
+    for (int j = 0; j < Np; ++j) {
+      const q v = c[k][j] * unit;
+      o->ci[(size_t)k * Np + j] = (long long)(v + (v < 0 ? (q)-0.5 : (q)0.5));
     }
-    return v;
-  }();
-  const int KT = g.KQ / 16;
-  const size_t at0 = out->size();
-  out->resize(at0 + (size_t)dense64_order_halves(g), 0);
-  bool exact = true;
-  for (int jo = 0; jo < g.No; ++jo) {
-    for (int q = 0; q < g.NQ; ++q) {
-      long long by_digit[kD64Digits] = {};
-      for (int ji = 0; ji < g.No; ++ji) {
-        const long long v = B[((size_t)q * g.No + jo) * g.No + ji];
-        const unsigned long long w = d64_bias(v);
-        unsigned short* o = &(*out)[at0 + (((size_t)(jo / 16) * g.NQ + q) * KT + ji / 16) * kD64Digits * 256 +
-                                    d64_b_index(ji % 16, jo % 16)];
-        for (int i = 0; i < kD64Digits; ++i) {
-          const int field = d64_field(w, i);
-          by_digit[i] += std::abs(field - 128);
-          o[i * 256] = half_of[field];
-        }
-      }
-      // the line's digits are at most 128
-      for (int s = 0; s < kD64Sums; ++s) {
-        long long most = 0;
-        for (int j = std::max(0, s - kD64Digits + 1); j <= std::min(s, kD64Digits - 1); ++j) most += 128 * by_digit[j];
-        exact = exact && most <= 1LL << 24;
-      }
-    }
+    // |output| <= 2^60 times the kernel's sum of magnitudes, in units of 2^56; 2^62 at most
+    o->sh[k] = std::max(0, (int)std::ceil(std::log2(std::ldexp(sum, e))) + 60 - 56 - 62);
   }
-  // |output| <= 2^60 times the kernel's sum of magnitudes, in units of 2^56; 2^62 at most
-  double sum = 0.0;
-  for (long long v : ci) sum += g.NQ * std::fabs((double)v);
-  *sh = std::max(0, (int)std::ceil(std::log2(sum)) + 60 - 56 - 62);
-  return exact && *sh <= 32;
 }
 
 }  // namespace fcns

@@ -56,25 +56,16 @@ void engine_twiddles(int L1, int L2, std::vector<std::complex<double>>* tw);
 // e^{-2 pi i k / N}, k = 0 .. N/2 (computed in binary128, rounded to double)
 void split_twiddles(int N, std::vector<std::complex<double>>* tw);
 
-// Derivative kernels of the N'-periodic unit grid, c[j] for j = 0..N'-1
-// (d1 odd and d2 even exactly; the Nyquist mode zeroed in d1, kept in d2), from
-// their closed forms.
-void deriv_kernels_closed(int Np, std::vector<double>* d1, std::vector<double>* d2);
-
-// Blocks of the dense z operator with kernel c (c[j], j modulo N'; odd or
-// even) on the geometry g, scaled by 2^(12 - e), e the exponent of the largest
-// entry, and split into float16 high and low parts: per output chunk, part and
-// contraction slab the high values and then the low values, each as groups of
-// eight contraction indexes x NC outputs (the shared-memory image the kernel
-// copies).  `out` gets dense_order_halves(g) values appended; returns the
-// scale exponent 12 - e.
-int dense_blocks(const DenseGeom& g, const std::vector<double>& c, std::vector<unsigned short>* out);
-
-// The same for float64 (dense64.hpp) and derivative order 1 or 2: per output tile of 16 orbits, part, 16-step
-// and digit the operand fragment of the matrix instruction.  *e: the blocks are
-// whole numbers of 2^-e; *sh: the bits that d64_combine drops so that an
-// output fits 62 bits.  False where a digit sum could leave 2^24.
-bool dense64_blocks(const DenseGeom& g, int order, std::vector<unsigned short>* out, int* e, int* sh);
+// Derivative kernels d/dz and d2/dz2 of the N'-periodic unit grid, c[j] for j = 0..N'-1 (d1 odd and d2 even exactly; the
+// Nyquist mode zeroed in d1, kept in d2), for the dense operators' blocks (dense_build.cuh).
+struct DenseKernels {
+  std::vector<double> c;       // [2][N'], order 1 first
+  std::vector<long long> ci;   // [2][N'], float64: c / NQ in whole units of 2^-e64
+  int e[2];                    // float32 blocks: entries are scaled by 2^e, the largest to [2^12, 2^13)
+  int e64[2];
+  int sh[2];                   // the bits that d64_combine drops so that an output fits 62 bits
+};
+void dense_kernels(const DenseGeom& g, DenseKernels* o);
 
 // cos / sin of 2 pi num / den, correctly rounded to double from binary128.
 void sincos2pi(long long num, long long den, double* c, double* s);

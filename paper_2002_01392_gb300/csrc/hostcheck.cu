@@ -10,7 +10,7 @@
 #include <vector>
 
 #include "deriv_kernel.cuh"
-#include "dense64.hpp"
+#include "dense_build.cuh"
 #include "host_tables.hpp"
 #include "slabs.hpp"
 
@@ -245,25 +245,50 @@ int fchc_dense_slab(int Nz, int Np, int s) {
 int fchc_dense_blocks(int Nz, int Np, int order, unsigned short* halves, int* exponent) {
   DenseGeom g;
   if (!dense_geom(Nz, Np, &g)) return 1;
-  std::vector<double> c1, c2;
-  deriv_kernels_closed(Np, &c1, &c2);
-  std::vector<unsigned short> out;
-  *exponent = dense_blocks(g, order == 1 ? c1 : c2, &out);
-  std::memcpy(halves, out.data(), 2 * out.size());
-  return (long long)out.size() == dense_order_halves(g) ? 0 : 2;
+  DenseKernels k;
+  dense_kernels(g, &k);
+  *exponent = k.e[order - 1];
+  for (long long i = 0; i < dense_groups(g); ++i)
+    dense_group(g, k.c.data() + (order - 1) * Np, k.e[order - 1], i, reinterpret_cast<__half*>(halves));
+  return 0;
+}
+static void dense64_order(const DenseGeom& g, const DenseKernels& k, int order, std::vector<__half>* out) {
+  out->resize(dense64_order_halves(g));
+  for (long long i = 0; i < dense64_lanes(g); ++i) dense64_lane(g, k.ci.data() + (order - 1) * g.Np, i, out->data());
+}
+// The sums of digit products that the float64 kernel adds in float32 are exact: the largest possible magnitude of one, for
+// line digits of at most 128, over all outputs, parts and weights of an order; 0 where there is no geometry.
+long long fchc_dense64_largest_sum(int Nz, int Np, int order) {
+  DenseGeom g;
+  if (!dense64_geom(Nz, Np, &g)) return 0;
+  DenseKernels k;
+  dense_kernels(g, &k);
+  long long most = 0;
+  for (int jo = 0; jo < g.No; ++jo)
+    for (int q = 0; q < g.NQ; ++q) {
+      long long by_digit[kD64Digits] = {};
+      for (int ji = 0; ji < g.No; ++ji) {
+        const unsigned long long w = d64_bias(dense_entry(g, q, jo, ji, k.ci.data() + (order - 1) * Np));
+        for (int i = 0; i < kD64Digits; ++i) by_digit[i] += std::abs(d64_field(w, i) - 128);
+      }
+      long long sum = 0;   // the last weight has all digits
+      for (int i = 0; i < kD64Digits; ++i) sum += 128 * by_digit[i];
+      most = std::max(most, sum);
+    }
+  return most;
 }
 // Float64 derivative of order 1 or 2 (unit spacing) of a tile of 16 lines x
 // [Nz][16] by the dense operators, y [Nz][16]: the kernel's own tables, index
 // maps and number formats, the products and sums in 64-bit integers.  Returns
-// 1 where there is no geometry, 2 where the digit sums could be inexact, 3
-// where one left 2^24.
+// 1 where there is no geometry, 3 where a digit sum left 2^24.
 int fchc_dense64_tile(int Nz, int d, int C, const double* Mr, int order, const double* x, double* y) {
   DenseGeom g;
   if (!dense64_geom(Nz, Nz + C, &g)) return 1;
-  std::vector<unsigned short> blocks;
-  int ex = 0, sh = 0;
-  if (!dense64_blocks(g, order, &blocks, &ex, &sh)) return 2;
-  if ((long long)blocks.size() != dense64_order_halves(g)) return 4;
+  DenseKernels kern;
+  dense_kernels(g, &kern);
+  const int ex = kern.e64[order - 1], sh = kern.sh[order - 1];
+  std::vector<__half> blocks;
+  dense64_order(g, kern, order, &blocks);
   const int KT = g.KQ / 16;
   std::vector<unsigned long long> X((size_t)g.Np * 16);
   std::memcpy(X.data(), x, sizeof(double) * Nz * 16);
@@ -287,11 +312,7 @@ int fchc_dense64_tile(int Nz, int d, int C, const double* Mr, int order, const d
       }
   }
   std::vector<int> B(blocks.size());
-  for (size_t i = 0; i < blocks.size(); ++i) {
-    __half h;
-    std::memcpy(&h, &blocks[i], 2);
-    B[i] = (int)__half2float(h);
-  }
+  for (size_t i = 0; i < blocks.size(); ++i) B[i] = (int)__half2float(blocks[i]);
   for (int li = 0; li < 16; ++li)
     for (int j = 0; j < g.No; ++j) {
       long long row[4] = {};

@@ -9,6 +9,7 @@
 #include "../../include/fcns.h"
 #include "dense64.hpp"
 #include "dense_geom.hpp"
+#include "host_tables.hpp"
 
 namespace fcns {
 
@@ -28,6 +29,7 @@ int pick_engine_length(int need);
 struct DerivDevTables {
   int device = -1;
   int L = 0;
+  void* block = nullptr;  // one allocation holds all of the following
   double* Mr = nullptr;
   float2* Mr2 = nullptr;  // (hi, lo) float split of Mr
   void* tw32 = nullptr;  // float2[L]
@@ -52,12 +54,9 @@ struct PlanData {
   double ls_residual;
   std::vector<double> Mr;
   DenseGeom dense;                        // dense operators (NQ = 0: none)
-  int dense_exp[2] = {0, 0};
-  bool dense_direct = false;              // the transform kernel would run at length N' itself
-  std::vector<unsigned short> dense_blocks;
   DenseGeom dense64;                      // the same for float64 (dense64.hpp)
-  int dense64_exp[2] = {0, 0}, dense64_sh[2] = {0, 0};
-  std::vector<unsigned short> dense64_blocks;
+  bool dense_direct = false;              // the transform kernel would run at length N' itself
+  DenseKernels kern;                      // what the blocks are built from, where either exists
   std::mutex mtx;
   std::mutex host_mtx;   // serialises fc_deriv_z_host calls on the plan (shared staging)
   std::vector<DerivDevTables> dev;
@@ -101,6 +100,12 @@ inline fc_status launch_deriv_any(bool dense, const DerivDevTables& t, const Pla
   return dtype == FC_F64 ? launch_deriv_dense64(t, p, batch, lines, Lz, f, df, d2f, stream)
                          : launch_deriv_dense(t, p, batch, lines, Lz, f, df, d2f, stream);
 }
+// builds the blocks of both orders in `out` (bytes: dense_bytes / dense64_bytes) from the kernels `c` (plan.kern.c or
+// plan.kern.ci, both orders, on the device)
+fc_status launch_dense_build(const PlanData& p, const double* c, void* out, cudaStream_t stream);
+fc_status launch_dense64_build(const PlanData& p, const long long* c, void* out, cudaStream_t stream);
+inline size_t dense_bytes(const PlanData& p) { return p.dense.NQ ? 4 * (size_t)dense_order_halves(p.dense) : 0; }
+inline size_t dense64_bytes(const PlanData& p) { return p.dense64.NQ ? 4 * (size_t)dense64_order_halves(p.dense64) : 0; }
 // whether a whole call (all its lines) takes the dense operators
 bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines);
 

@@ -2,6 +2,7 @@
 #include <atomic>
 #include <cmath>
 
+#include "dense_build.cuh"
 #include "dense_z.cuh"
 #include "internal.hpp"
 
@@ -68,7 +69,7 @@ fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int bat
   for (int o = 0; o < 2; ++o) {   // (at least 1 after rounding: frexp's mantissa is in [1/2, 1))
     int e = 0;
     a.f[o] = (float)(2 * std::frexp(sc[o], &e));
-    a.fe[o] = e - 1 - p.dense_exp[o];
+    a.fe[o] = e - 1 - p.kern.e[o];
     if (!(sc[o] > 0) || std::isinf(sc[o])) {   // (no exponent: as a product)
       a.f[o] = (float)sc[o];
       a.fe[o] = 1000;
@@ -76,6 +77,19 @@ fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int bat
   }
   a.err = t.dense_err;
   return launch_dense(a, stream);
+}
+
+__global__ void dense_build_kernel(const __grid_constant__ DenseGeom g, const double* __restrict__ c, int e1, int e2, __half* out) {
+  const long long n = dense_groups(g), i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 2 * n) return;
+  const int o = i >= n;
+  dense_group(g, c + o * g.Np, o ? e2 : e1, i - o * n, out + o * dense_order_halves(g));
+}
+
+fc_status launch_dense_build(const PlanData& p, const double* c, void* out, cudaStream_t stream) {
+  const long long n = 2 * dense_groups(p.dense);
+  dense_build_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(p.dense, c, p.kern.e[0], p.kern.e[1], static_cast<__half*>(out));
+  return cuda_status(cudaGetLastError(), "dense z blocks launch");
 }
 
 }  // namespace fcns

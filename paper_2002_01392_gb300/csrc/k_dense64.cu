@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 
 #include "dense64.hpp"
+#include "dense_build.cuh"
 #include "internal.hpp"
 
 namespace fcns {
@@ -221,6 +222,13 @@ __global__ void __launch_bounds__(kD64Threads, 1) dense64_kernel(const __grid_co
   }
 }
 
+__global__ void dense64_build_kernel(const __grid_constant__ DenseGeom g, const long long* __restrict__ c, __half* out) {
+  const long long n = dense64_lanes(g), i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 2 * n) return;
+  const int o = i >= n;
+  dense64_lane(g, c + o * g.Np, i - o * n, out + o * dense64_order_halves(g));
+}
+
 }  // namespace
 
 fc_status launch_deriv_dense64(const DerivDevTables& t, const PlanData& p, int batch, long long lines, double Lz,
@@ -244,8 +252,8 @@ fc_status launch_deriv_dense64(const DerivDevTables& t, const PlanData& p, int b
   for (int o = 0; o < 2; ++o) {
     int e = 0;
     a.f[o] = std::frexp(s[o], &e);
-    a.sh[o] = p.dense64_sh[o];
-    a.k[o] = 56 + a.sh[o] - 1082 - p.dense64_exp[o] + e;
+    a.sh[o] = p.kern.sh[o];
+    a.k[o] = 56 + a.sh[o] - 1082 - p.kern.e64[o] + e;
   }
   const size_t smem = (size_t)a.g.NQ * (a.g.KQ / 16) * kD64Digits * 512 + (size_t)a.g.Np * kD64Lines * 8 + 6 * kD64Lines * 8;
   auto kern = a.g.NQ == 4 ? dense64_kernel<4> : dense64_kernel<2>;
@@ -272,6 +280,12 @@ fc_status launch_deriv_dense64(const DerivDevTables& t, const PlanData& p, int b
   const dim3 grid((unsigned)(a.tiles < sms ? a.tiles : sms), (unsigned)(room < most ? room : most));
   kern<<<grid, kD64Threads, smem, stream>>>(a);
   return cuda_status(cudaGetLastError(), "dense z launch (float64)");
+}
+
+fc_status launch_dense64_build(const PlanData& p, const long long* c, void* out, cudaStream_t stream) {
+  const long long n = 2 * dense64_lanes(p.dense64);
+  dense64_build_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(p.dense64, c, static_cast<__half*>(out));
+  return cuda_status(cudaGetLastError(), "dense z blocks launch (float64)");
 }
 
 }  // namespace fcns

@@ -11,8 +11,8 @@
 // until the process exits).  A call whose plan and precision differ from the
 // tables the array holds on this device copies the plan's tables into it on
 // the caller's stream first; a call with the same plan and precision as the
-// previous call on the device launches the kernel at once.  Calls that
-// fc_deriv_z runs with the dense operators have a second array of their own.
+// previous call on the device launches the kernel at once.  The dense
+// operators' blocks are built in a second array by a kernel on that stream.
 #include <mutex>
 
 #include "internal.hpp"
@@ -25,71 +25,35 @@ constexpr int kMaxDevices = 64;
 
 // Shared by every call on a device; holds the tables of the last call.
 static __device__ __align__(256) unsigned char g_deriv_scratch[kNoAllocBytes];
-// The same for calls that fc_deriv_z runs with the dense operators: their
-// blocks (at most 1.33 MB in float32, N' = 575, and 2.66 MB in float64, N' =
-// 576) and the continuation matrix.
-constexpr size_t kNoAllocDense = 2600 * 1024;
+// The dense operators' blocks of the same plan and precision (at most 1.33 MB
+// in float32, N' = 575, and 2.66 MB in float64, N' = 576).
+constexpr size_t kNoAllocDense = 2592 * 1024;
 static __device__ __align__(256) unsigned char g_dense_scratch[kNoAllocDense];
 
 std::mutex g_mtx;
 void* g_scratch_addr[kMaxDevices] = {};
 void* g_dense_addr[kMaxDevices] = {};
-unsigned long long g_dense_serial[kMaxDevices] = {};
-int g_dense_dtype[kMaxDevices] = {};
 // which tables the array holds per device: the plan's serial number and the
 // precision of the last upload (0: none, or an upload that failed part-way)
 unsigned long long g_loaded_serial[kMaxDevices] = {};
 int g_loaded_dtype[kMaxDevices] = {};
 
-// Device address of g_deriv_scratch on the current device (the host-side
-// symbol is only a stand-in and must never be passed to a kernel).
-fc_status scratch_address(int dev, unsigned char** out) {
+// Device addresses of the two arrays on the current device (the host-side
+// symbols are only stand-ins and must never be passed to a kernel).
+fc_status scratch_addresses(int dev, unsigned char** tables, unsigned char** blocks) {
   if (dev < 0 || dev >= kMaxDevices) { set_error("fc_deriv_z_noalloc: device index out of range"); return FC_ERR_UNSUPPORTED; }
   std::lock_guard<std::mutex> lk(g_mtx);
-  if (!g_scratch_addr[dev]) {
-    void* p = nullptr;
+  if (!g_scratch_addr[dev] || !g_dense_addr[dev]) {
+    void *p = nullptr, *d = nullptr;
     fc_status s = cuda_status(cudaGetSymbolAddress(&p, g_deriv_scratch), "cudaGetSymbolAddress(g_deriv_scratch)");
+    if (!s) s = cuda_status(cudaGetSymbolAddress(&d, g_dense_scratch), "cudaGetSymbolAddress(g_dense_scratch)");
     if (s) return s;
     g_scratch_addr[dev] = p;
+    g_dense_addr[dev] = d;
   }
-  *out = static_cast<unsigned char*>(g_scratch_addr[dev]);
+  *tables = static_cast<unsigned char*>(g_scratch_addr[dev]);
+  *blocks = static_cast<unsigned char*>(g_dense_addr[dev]);
   return FC_OK;
-}
-
-// the dense-operator call: blocks and matrix copied when the plan or precision differs from the previous such call's
-fc_status noalloc_dense(fc_plan* plan, fc_dtype dtype, int dev, int batch, long long lines, double Lz, const void* f, void* df, void* d2f,
-                        cudaStream_t st) {
-  const bool f64 = dtype == FC_F64;
-  const std::vector<unsigned short>& blocks = f64 ? plan->data.dense64_blocks : plan->data.dense_blocks;
-  const void* Mr = f64 ? (const void*)plan->data.Mr.data() : (const void*)plan->deriv.Mr2.data();
-  const size_t nB = 2 * blocks.size(), nM = sizeof(double) * plan->data.Mr.size();   // (a float pair per entry in float32)
-  if (nB + nM > kNoAllocDense) {
-    set_error("fc_deriv_z_noalloc: dense blocks of this plan exceed the static scratch");
-    return FC_ERR_UNSUPPORTED;
-  }
-  unsigned char* base = nullptr;
-  {
-    std::lock_guard<std::mutex> lk(g_mtx);
-    fc_status s = FC_OK;
-    if (!g_dense_addr[dev])
-      s = cuda_status(cudaGetSymbolAddress(&g_dense_addr[dev], g_dense_scratch), "cudaGetSymbolAddress(g_dense_scratch)");
-    if (s) return s;
-    base = static_cast<unsigned char*>(g_dense_addr[dev]);
-    if (g_dense_serial[dev] != plan->deriv.serial || g_dense_dtype[dev] != (int)dtype) {
-      g_dense_serial[dev] = 0;
-      s = cuda_status(cudaMemcpyAsync(base, blocks.data(), nB, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(dense)");
-      if (!s) s = cuda_status(cudaMemcpyAsync(base + nB, Mr, nM, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(M_r)");
-      if (s) return s;
-      g_dense_serial[dev] = plan->deriv.serial;
-      g_dense_dtype[dev] = (int)dtype;
-    }
-  }
-  DerivDevTables t;
-  t.device = dev;
-  t.dense = t.dense64 = base;
-  t.Mr = reinterpret_cast<double*>(base + nB);
-  t.Mr2 = reinterpret_cast<float2*>(base + nB);
-  return launch_deriv_any(true, t, plan->data, dtype, batch, lines, Lz, f, df, d2f, st);
 }
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }
@@ -109,20 +73,21 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
   const size_t cs = dtype == FC_F32 ? sizeof(float2) : sizeof(double2);
   const size_t nMr = plan->data.Mr.size();
   const size_t oMr = 0, oMr2 = align256(sizeof(double) * nMr), oH1 = oMr2 + align256(sizeof(float2) * nMr);
-  const size_t oH2 = oH1 + align256(cs * h.L), oTw = oH2 + align256(cs * h.L), need = oTw + align256(cs * 2 * h.L);
-  if (need > kNoAllocBytes) {
-    set_error("fc_deriv_z_noalloc: tables of this plan exceed the 128 KiB static scratch");
+  const size_t oH2 = oH1 + align256(cs * h.L), oTw = oH2 + align256(cs * h.L), oC = oTw + align256(cs * 2 * h.L);
+  // the kernels that the dense blocks of this precision are built from
+  const PlanData& pd = plan->data;
+  const size_t nB = dtype == FC_F32 ? dense_bytes(pd) : dense64_bytes(pd), nC = nB ? sizeof(double) * pd.kern.c.size() : 0;
+  if (oC + nC > kNoAllocBytes || nB > kNoAllocDense) {
+    set_error("fc_deriv_z_noalloc: tables of this plan exceed the static scratch");
     return FC_ERR_UNSUPPORTED;
   }
   int dev = -1;
   s = cuda_status(cudaGetDevice(&dev), "cudaGetDevice");
   if (s) return s;
-  unsigned char* base = nullptr;
-  s = scratch_address(dev, &base);
+  unsigned char *base = nullptr, *blocks = nullptr;
+  s = scratch_addresses(dev, &base, &blocks);
   if (s) return s;
   cudaStream_t st = (cudaStream_t)stream;
-  if (deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch))
-    return noalloc_dense(plan, dtype, dev, batch, (long long)Nx * Ny, Lz, f, df, d2f, st);
   {
     std::lock_guard<std::mutex> lk(g_mtx);
     if (g_loaded_serial[dev] != h.serial || g_loaded_dtype[dev] != (int)dtype) {
@@ -137,6 +102,13 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
       if (!s) s = cuda_status(cudaMemcpyAsync(base + oH1, H1src, cs * h.L, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(H1)");
       if (!s) s = cuda_status(cudaMemcpyAsync(base + oH2, H2src, cs * h.L, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(H2)");
       if (!s) s = cuda_status(cudaMemcpyAsync(base + oTw, Tsrc, cs * 2 * h.L, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(tw)");
+      // (whatever the size of this call, so that the next one copies nothing)
+      if (!s && nB) {
+        const void* C = dtype == FC_F32 ? (const void*)pd.kern.c.data() : (const void*)pd.kern.ci.data();
+        s = cuda_status(cudaMemcpyAsync(base + oC, C, nC, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync(kernels)");
+        if (!s) s = dtype == FC_F32 ? launch_dense_build(pd, reinterpret_cast<const double*>(base + oC), blocks, st)
+                                    : launch_dense64_build(pd, reinterpret_cast<const long long*>(base + oC), blocks, st);
+      }
       if (s) return s;
       g_loaded_serial[dev] = h.serial;
       g_loaded_dtype[dev] = (int)dtype;
@@ -150,5 +122,7 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
   t.H1_32 = t.H1_64 = base + oH1;
   t.H2_32 = t.H2_64 = base + oH2;
   t.tw32 = t.tw64 = base + oTw;
-  return launch_deriv_z(t, plan->data, dtype, batch, (long long)Nx * Ny, Lz, f, df, d2f, st);
+  t.dense = t.dense64 = blocks;
+  const long long lines = (long long)Nx * Ny;
+  return launch_deriv_any(deriv_is_dense(pd, dtype, lines * batch), t, pd, dtype, batch, lines, Lz, f, df, d2f, st);
 }

@@ -369,6 +369,53 @@ def test_dense64_arithmetic_on_the_cpu(Nz, Mr_5_25):
         assert not y[:, 15].any()
 
 
+def test_dense64_digit_sums_are_exact():
+    """No sum of digit products of any operator that the float64 kernel takes can leave 2^24, where float32 still holds
+    every whole number."""
+    lib = _lib()
+    lib.fchc_dense64_largest_sum.restype = ctypes.c_longlong
+    most = [lib.fchc_dense64_largest_sum(Np - C, Np, order) for Np in range(6, 577) for C in (2, 3) for order in (1, 2)]
+    assert sum(m > 0 for m in most) > 1800 and max(most) <= 2 ** 24
+
+
+@pytest.mark.gpu
+def test_a_plans_first_call_prepares_all_others(api):
+    """After one small call on a plan, large ones, of the other precision too, can be captured (nothing is allocated or
+    copied), and fc_deriv_z_noalloc, whose tables are one precision's, only launches after a small call of the same."""
+    import torch
+    Nz, Ny, Nx = 513, 8, 2560
+    plan = api.Plan(5, 25, Nz)
+    f = torch.randn((1, Nz, Ny, Nx), device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    ref = api.Plan(5, 25, Nz)
+    for name in ("fc_deriv_z", "fc_deriv_z_noalloc"):
+        for dt, code in ((torch.float32, api.FC_F32), (torch.float64, api.FC_F64)):
+            x = f.to(dt)
+            want = [torch.empty_like(x) for _ in range(2)]
+            api.fc_deriv_z(ref, x, *want)
+            small = x[:, :, :1, :64].contiguous()
+            so, out = [torch.empty_like(small) for _ in range(2)], [torch.zeros_like(x) for _ in range(2)]
+
+            def call(a, o):
+                st = getattr(api._lib, name)(plan.handle, code, 1, a.shape[3], a.shape[2], ctypes.c_double(1.0), a.data_ptr(),
+                                             o[0].data_ptr(), o[1].data_ptr(), torch.cuda.current_stream().cuda_stream)
+                assert st == 0, api._lib.fc_last_error().decode()
+
+            if name == "fc_deriv_z_noalloc" or dt == torch.float32:
+                call(small, so)
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                call(x, out)
+            call(x, out)       # not captured: whatever the capture would have copied is not there
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(out, want)), (name, dt)
+            out[0].zero_()
+            out[1].zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(out, want)), (name, dt)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("Nz,Ny,Nx,B,Lz", [(11, 5, 3, 1, 1.0), (33, 7, 37, 3, 2.0), (65, 64, 66, 1, 1.0), (102, 33, 31, 2, 1.0),
                                             (231, 48, 51, 1, 0.5), (358, 16, 17, 2, 1.0), (487, 48, 50, 1, 1.0), (513, 61, 41, 1, 1e-6),
