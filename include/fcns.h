@@ -96,7 +96,9 @@ fc_status fc_plan_matrix(fc_plan_t plan, double* Mr_out);
 fc_status fc_plan_info(fc_plan_t plan, int* d, int* C, int* Nz, int* M, int* n_os,
                        double* ls_residual);
 
-/* Release a plan and its device tables (synchronises the devices it used). */
+/* Release a plan and its device tables (synchronises the devices it used).
+ * FC_ERR_TIMEOUT where a kernel of the plan had given up a wait that no call
+ * has reported (see fc_deriv_z); the plan is released all the same. */
 fc_status fc_destroy(fc_plan_t plan);
 
 /*
@@ -123,8 +125,11 @@ fc_status fc_destroy(fc_plan_t plan);
  * even N' < 576, take the derivative operators as dense blocks on the tensor
  * cores instead of transforms (same accuracy, float64 through exact integer
  * sums); a NaN or Inf then spoils the outputs of its own line only.
- * FC_ERR_TIMEOUT: the float32 dense kernel of an earlier call of the plan gave
- * up a bounded wait (its outputs are not valid); the state is cleared.
+ * FC_ERR_TIMEOUT: a float32 dense kernel of an earlier call of the plan gave up
+ * a bounded wait; its outputs are NaN from there on.  Reported once, by the
+ * next fc_deriv_z, fc_deriv_z_noalloc or fc_deriv_z_host call of the plan,
+ * which then does nothing, or by fc_destroy; fc_deriv_z_host reports its own
+ * kernels' when it returns.
  */
 fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, double Lz,
                      const void* f, void* df, void* d2f, fc_stream_t stream);
@@ -541,7 +546,9 @@ fc_status ns_set_finite_check(ns_sim_t sim, int every);
  * fc_count_nonfinite, fc_noise, ns_create,
  * ns_set_fields, ns_get_fields, ns_get_state, ns_put_state, ns_rhs,
  * fc_poisson_project, rk_step, ns_diagnostics, ns_profiles, ns_interpolate,
- * ns_tune, ns_check_finite, ns_batch_create and ns_batch_step.
+ * ns_tune, ns_check_finite, ns_batch_create and ns_batch_step.  The name
+ * dense_z_kernel (not matched by "*") makes a float32 dense kernel of
+ * fc_deriv_z count as one that gave up a wait; its outputs are valid.
  * FC_ERR_ARG for a NULL-free rule with status FC_OK, skip < 0 or count = 0.
  */
 fc_status fc_inject_failure(const char* entry, fc_status status, long long skip, long long count);

@@ -96,6 +96,18 @@ fc_status injected(const char* entry) {
   return out;
 }
 
+bool injected_event(const char* name) {
+  if (g_inj_state.load(std::memory_order_acquire) <= 0) return false;
+  std::lock_guard<std::mutex> lk(g_inj_mtx);
+  for (auto& r : g_inj) {
+    if (r.entry != name || r.count == 0) continue;
+    if (r.skip > 0) { --r.skip; continue; }
+    if (r.count > 0) --r.count;
+    return true;
+  }
+  return false;
+}
+
 // Which float32 calls take the dense operators instead of the transforms.  A
 // tile of 128 lines passes through one SM in 10 us (N' = 115) to 45 us (538), so
 // a call needs a wave of tiles (152 x 128 lines) or more, and the gain depends
@@ -175,7 +187,7 @@ fc_status fc_setup_ex(int d, int C, int Nz, int M, int n_os, fc_plan_t* out) {
   fc_plan* p = new (std::nothrow) fc_plan;
   if (!p) return FC_ERR_NOMEM;
   static std::atomic<unsigned long long> next_serial{1};
-  p->deriv.serial = next_serial.fetch_add(1);
+  p->data.serial = next_serial.fetch_add(1);
   FcTables T;
   if (!build_fc_tables(d, C, M, n_os, &T)) { delete p; set_error("fc_setup: table construction failed"); return FC_ERR_ARG; }
   p->data.d = d; p->data.C = C; p->data.Nz = Nz; p->data.Np = Nz + C;
@@ -256,7 +268,6 @@ fc_status fc_destroy(fc_plan_t plan) {
       cudaSetDevice(t.device);
       cudaDeviceSynchronize();
       cudaFree(t.block);
-      if (t.dense_err) cudaFreeHost(t.dense_err);
       for (auto& slot : t.stage)
         for (void* b : slot) cudaFree(b);
       for (int k = 0; k < 3; ++k) {
@@ -270,8 +281,10 @@ fc_status fc_destroy(fc_plan_t plan) {
     }
     cudaSetDevice(cur);
   }
+  // (the devices have finished: what no later call has reported)
+  const fc_status s = dense_gave_up(plan->data, "fc_destroy");
   delete plan;
-  return FC_OK;
+  return s;
 }
 
 }  // extern "C"
@@ -319,8 +332,6 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
   if (!s && pd.dense.NQ) {
     t.dense = at + oB;
     s = launch_dense_build(pd, reinterpret_cast<const double*>(at + oC), t.dense, nullptr);
-    if (!s) s = cuda_status(cudaHostAlloc((void**)&t.dense_err, sizeof(unsigned), cudaHostAllocDefault), "cudaHostAlloc");
-    if (!s) *t.dense_err = 0;
   }
   if (!s && pd.dense64.NQ) {
     t.dense64 = at + oB64;
@@ -330,7 +341,6 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
   if (!s) s = cuda_status(cudaStreamSynchronize(nullptr), "cudaStreamSynchronize(tables)");
   if (s) {
     cudaFree(t.block);
-    if (t.dense_err) cudaFreeHost(t.dense_err);
     return s;
   }
   plan->data.dev.push_back(t);
@@ -366,6 +376,7 @@ extern "C" fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int N
   if (fc_status inj = injected("fc_deriv_z")) return inj;
   if (!plan) { set_error("fc_deriv_z: NULL plan"); return FC_ERR_ARG; }
   fc_status s = check_deriv_args(plan->data, plan->deriv, dtype, batch, Nx, Ny, Lz, f, df, d2f, "fc_deriv_z");
+  if (!s) s = dense_gave_up(plan->data, "fc_deriv_z");
   if (s) return s;
   DerivDevTables* t = nullptr;
   {
@@ -417,6 +428,7 @@ extern "C" fc_status fc_deriv_z_host_ex(fc_plan_t plan, fc_dtype dtype, int batc
   if (fc_status inj = injected("fc_deriv_z_host")) return inj;
   if (!plan) { set_error("fc_deriv_z_host: NULL plan"); return FC_ERR_ARG; }
   fc_status s = check_deriv_args(plan->data, plan->deriv, dtype, batch, Nx, Ny, Lz, f, df, d2f, "fc_deriv_z_host");
+  if (!s) s = dense_gave_up(plan->data, "fc_deriv_z_host");
   if (s) return s;
   DerivDevTables* t = nullptr;
   {
@@ -470,7 +482,8 @@ extern "C" fc_status fc_deriv_z_host_ex(fc_plan_t plan, fc_dtype dtype, int batc
   const fc_status s2 = cuda_status(cudaStreamSynchronize(t->st_run), "cudaStreamSynchronize");
   const fc_status s3 = cuda_status(cudaStreamSynchronize(t->st_out), "cudaStreamSynchronize");
   if (e0) cudaEventDestroy(e0);
-  return s ? s : (s1 ? s1 : (s2 ? s2 : s3));
+  const fc_status s4 = dense_gave_up(plan->data, "fc_deriv_z_host");
+  return s ? s : (s1 ? s1 : (s2 ? s2 : (s3 ? s3 : s4)));
 }
 
 extern "C" fc_status fc_deriv_z_host(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, double Lz,

@@ -43,8 +43,8 @@
 // rows in L2 (1.97 -> 1.70 together with the sampled scale, which saves a
 // second pass over the tile).
 //
-// Every wait is bounded (dz::mbar_wait): one that runs out sets the error word in
-// host memory, and the next call on the plan reports it.
+// Every wait is bounded (dz::mbar_wait): after one that runs out the outputs are
+// NaN, and the error word is set, which the plan's next call reports.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -69,7 +69,7 @@ struct DenseArgs {
   const float2* Mr2;
   float f[2];              // output factors (grid spacing and the blocks' scale): a number in [1, 2) times 2^fe
   int fe[2];
-  unsigned* err;           // error word (host memory), may be null
+  unsigned* err;           // error word (managed memory), may be null
 };
 
 #if defined(__CUDACC__) && !defined(FC_HOSTCHECK)
@@ -439,6 +439,8 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
             dz::fence_before();
             dz::mbar_arrive(bFree + 8 * q);
           }
+          // (a role that gives up sets the flag before it goes on, so what came of it is read behind it)
+          const float fb = *abort ? __int_as_float(0x7fc00000) : fa;
           if (steps) {
             const int K = a.fe[o] - scaled;
             const float f1 = K < -80 || K > 80 ? a.f[o] * __int_as_float((min(max(K, -100), 100) + 127) << 23) : 1.f;
@@ -460,16 +462,16 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
               for (int e = 0; e < 4; ++e) {
                 float(&Y)[NQ][4] = y[k];
                 if constexpr (NQ == 4) {
-                  const float P = (Y[0][e] + Y[2][e]) * fa, M = (Y[0][e] - Y[2][e]) * fa;
+                  const float P = (Y[0][e] + Y[2][e]) * fb, M = (Y[0][e] - Y[2][e]) * fb;
                   const float R = Y[1][e] + Y[3][e], S = Y[1][e] - Y[3][e];
-                  Y[0][e] = fmaf(R, fa, P);
-                  Y[1][e] = par * fmaf(-R, fa, P);
-                  Y[2][e] = fmaf(S, fa, M);
-                  Y[3][e] = par * fmaf(-S, fa, M);
+                  Y[0][e] = fmaf(R, fb, P);
+                  Y[1][e] = par * fmaf(-R, fb, P);
+                  Y[2][e] = fmaf(S, fb, M);
+                  Y[3][e] = par * fmaf(-S, fb, M);
                 } else {
-                  const float P = Y[0][e] * fa, R = Y[1][e];
-                  Y[0][e] = fmaf(R, fa, P);
-                  Y[1][e] = par * fmaf(-R, fa, P);
+                  const float P = Y[0][e] * fb, R = Y[1][e];
+                  Y[0][e] = fmaf(R, fb, P);
+                  Y[1][e] = par * fmaf(-R, fb, P);
                 }
               }
 #pragma unroll

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <complex>
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -40,7 +41,6 @@ struct DerivDevTables {
   void* H2_64 = nullptr;
   void* dense = nullptr;          // blocks of the dense operators (float16 pairs), both orders; null: not used
   void* dense64 = nullptr;        // the same for float64 (digit fragments)
-  unsigned* dense_err = nullptr;  // host word (pinned) that a kernel sets when a wait runs out
   // staging of fc_deriv_z_host: three rotating slots of (input, d1, d2) slab
   // buffers of stage_bytes each, and the copy-in / compute / copy-out streams
   size_t stage_bytes = 0;
@@ -50,6 +50,7 @@ struct DerivDevTables {
 };
 
 struct PlanData {
+  unsigned long long serial = 0;          // unique per plan in the process (never reused)
   int d, C, Nz, Np, M, n_os;
   double ls_residual;
   std::vector<double> Mr;
@@ -57,6 +58,8 @@ struct PlanData {
   DenseGeom dense64;                      // the same for float64 (dense64.hpp)
   bool dense_direct = false;              // the transform kernel would run at length N' itself
   DenseKernels kern;                      // what the blocks are built from, where either exists
+  // word that a float32 dense kernel of the plan sets when a wait runs out (null before the first one)
+  mutable std::atomic<unsigned*> gave_up{nullptr};
   std::mutex mtx;
   std::mutex host_mtx;   // serialises fc_deriv_z_host calls on the plan (shared staging)
   std::vector<DerivDevTables> dev;
@@ -65,7 +68,6 @@ struct PlanData {
 
 // host copies of the derivative tables of one plan, in both precisions
 struct PlanHostTables {
-  unsigned long long serial = 0;  // unique per plan in the process (never reused)
   int L = 0, L1 = 0, L2 = 0;
   std::vector<std::complex<double>> tw;
   std::vector<float2> tw32, Mr2, H1_32, H2_32;
@@ -106,6 +108,10 @@ fc_status launch_dense_build(const PlanData& p, const double* c, void* out, cuda
 fc_status launch_dense64_build(const PlanData& p, const long long* c, void* out, cudaStream_t stream);
 inline size_t dense_bytes(const PlanData& p) { return p.dense.NQ ? 4 * (size_t)dense_order_halves(p.dense) : 0; }
 inline size_t dense64_bytes(const PlanData& p) { return p.dense64.NQ ? 4 * (size_t)dense64_order_halves(p.dense64) : 0; }
+// FC_ERR_TIMEOUT (once) where a float32 dense kernel of the plan gave up a bounded wait
+fc_status dense_gave_up(const PlanData& p, const char* who);
+// whether a rule of fc_inject_failure for exactly this name fires; sets no error text
+bool injected_event(const char* name);
 // whether a whole call (all its lines) takes the dense operators
 bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines);
 

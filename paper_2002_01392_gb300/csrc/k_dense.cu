@@ -42,14 +42,34 @@ static fc_status launch_dense(DenseArgs a, cudaStream_t stream) {
   return cuda_status(cudaGetLastError(), "dense z launch");
 }
 
+// The words that kernels set when a wait runs out, one per plan (by its serial number; two of a thousand plans in use
+// share one).  Managed: a kernel's store reaches the host without a call, a host's read of a page that no kernel has written
+// is an ordinary one, and nothing is allocated (a pinned word of its own cost a plan's first call 107 us).
+constexpr int kErrWords = 1024;
+static __managed__ unsigned g_dense_err[kErrWords];
+
+static unsigned* err_word(const PlanData& p) {
+  unsigned* w = p.gave_up.load();
+  if (w) return w;
+  // (where the host may not read managed memory while kernels run, there is no word; the outputs are NaN all the same)
+  int dev = 0, ok = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&ok, cudaDevAttrConcurrentManagedAccess, dev) != cudaSuccess || !ok) return nullptr;
+  w = &g_dense_err[p.serial % kErrWords];
+  p.gave_up.store(w);
+  return w;
+}
+
+fc_status dense_gave_up(const PlanData& p, const char* who) {
+  unsigned* w = p.gave_up.load();
+  const unsigned id = w ? *static_cast<volatile unsigned*>(w) : 0;
+  if (!id) return FC_OK;
+  *static_cast<volatile unsigned*>(w) = 0;
+  set_error(std::string(who) + ": a kernel of the plan gave up wait " + std::to_string(id));
+  return FC_ERR_TIMEOUT;
+}
+
 fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int batch, long long lines, double Lz,
                              const void* f, void* df, void* d2f, cudaStream_t stream) {
-  const unsigned gave_up = t.dense_err ? *static_cast<volatile unsigned*>(t.dense_err) : 0;
-  if (gave_up) {
-    *static_cast<volatile unsigned*>(t.dense_err) = 0;
-    set_error("fc_deriv_z: an earlier call's kernel gave up wait " + std::to_string(gave_up));
-    return FC_ERR_TIMEOUT;
-  }
   DenseArgs a = {};
   a.g = p.dense;
   a.d = p.d;
@@ -75,8 +95,10 @@ fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int bat
       a.fe[o] = 1000;
     }
   }
-  a.err = t.dense_err;
-  return launch_dense(a, stream);
+  a.err = err_word(p);
+  const fc_status s = launch_dense(a, stream);
+  if (!s && a.err && injected_event("dense_z_kernel")) *static_cast<volatile unsigned*>(a.err) = 1;   // (as the kernel would)
+  return s;
 }
 
 __global__ void dense_build_kernel(const __grid_constant__ DenseGeom g, const double* __restrict__ c, int e1, int e2, __half* out) {

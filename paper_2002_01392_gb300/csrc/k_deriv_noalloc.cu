@@ -69,6 +69,8 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
   if (!plan) { set_error("fc_deriv_z_noalloc: NULL plan"); return FC_ERR_ARG; }
   fc_status s = check_deriv_args(plan->data, plan->deriv, dtype, batch, Nx, Ny, Lz, f, df, d2f, "fc_deriv_z_noalloc");
   if (s) return s;
+  s = dense_gave_up(plan->data, "fc_deriv_z_noalloc");
+  if (s) return s;
   const PlanHostTables& h = plan->deriv;
   const size_t cs = dtype == FC_F32 ? sizeof(float2) : sizeof(double2);
   const size_t nMr = plan->data.Mr.size();
@@ -90,7 +92,7 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
   cudaStream_t st = (cudaStream_t)stream;
   {
     std::lock_guard<std::mutex> lk(g_mtx);
-    if (g_loaded_serial[dev] != h.serial || g_loaded_dtype[dev] != (int)dtype) {
+    if (g_loaded_serial[dev] != pd.serial || g_loaded_dtype[dev] != (int)dtype) {
       g_loaded_serial[dev] = 0;
       const void* H1src = dtype == FC_F32 ? (const void*)h.H1_32.data() : (const void*)h.H1_64.data();
       const void* H2src = dtype == FC_F32 ? (const void*)h.H2_32.data() : (const void*)h.H2_64.data();
@@ -110,7 +112,7 @@ extern "C" fc_status fc_deriv_z_noalloc(fc_plan_t plan, fc_dtype dtype, int batc
                                     : launch_dense64_build(pd, reinterpret_cast<const long long*>(base + oC), blocks, st);
       }
       if (s) return s;
-      g_loaded_serial[dev] = h.serial;
+      g_loaded_serial[dev] = pd.serial;
       g_loaded_dtype[dev] = (int)dtype;
     }
   }

@@ -379,6 +379,45 @@ def test_dense64_digit_sums_are_exact():
 
 
 @pytest.mark.gpu
+def test_given_up_waits_are_reported(api):
+    """A kernel that gave up a wait (set on the host here) is reported once, by whatever call of the plan comes next, by the
+    call itself where it is synchronous, or by fc_destroy; another plan is not concerned."""
+    import torch
+    Nz, Ny, Nx = 257, 8, 2560
+    plan, other = api.Plan(5, 25, Nz), api.Plan(5, 25, Nz)
+    f = torch.randn((1, Nz, Ny, Nx), device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+
+    def call(p, name, x):
+        o = [torch.empty_like(x) for _ in range(2)]
+        st = getattr(api._lib, name)(p.handle, api.FC_F32 if x.dtype == torch.float32 else api.FC_F64, 1, x.shape[3], x.shape[2],
+                                     ctypes.c_double(1.0), x.data_ptr(), o[0].data_ptr(), o[1].data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        return st, o
+
+    small, host = f[:, :, :1, :64].contiguous(), f.cpu()
+    timeout = api.STATUS["FC_ERR_TIMEOUT"]
+    good = call(plan, "fc_deriv_z", f)[1]
+    for first in ("fc_deriv_z", "fc_deriv_z_noalloc"):
+        for name, x in (("fc_deriv_z", small), ("fc_deriv_z", f.double()), ("fc_deriv_z_noalloc", f), ("fc_deriv_z_host", host)):
+            api.inject_failure("dense_z_kernel", "FC_ERR_TIMEOUT")
+            assert call(plan, first, f)[0] == 0
+            assert call(other, name, x)[0] == 0
+            assert call(plan, name, x)[0] == timeout and b"gave up" in api._lib.fc_last_error()
+            assert call(plan, name, x)[0] == 0
+    api.inject_failure("dense_z_kernel", "FC_ERR_TIMEOUT")
+    assert call(plan, "fc_deriv_z_host", host)[0] == timeout
+    st, o = call(plan, "fc_deriv_z_host", host)
+    assert st == 0 and all(torch.equal(a, b.cpu()) for a, b in zip(o, good))
+    api.inject_failure("dense_z_kernel", "FC_ERR_TIMEOUT")
+    assert call(plan, "fc_deriv_z", f)[0] == 0
+    assert api._lib.fc_destroy(plan.handle) == timeout
+    plan.handle = None
+    assert api._lib.fc_destroy(other.handle) == 0
+    other.handle = None
+
+
+@pytest.mark.gpu
 def test_a_plans_first_call_prepares_all_others(api):
     """After one small call on a plan, large ones, of the other precision too, can be captured (nothing is allocated or
     copied), and fc_deriv_z_noalloc, whose tables are one precision's, only launches after a small call of the same."""
