@@ -248,13 +248,13 @@ int fchc_dense_blocks(int Nz, int Np, int order, unsigned short* halves, int* ex
   DenseKernels k;
   dense_kernels(g, &k);
   *exponent = k.e[order - 1];
-  for (long long i = 0; i < dense_groups(g); ++i)
-    dense_group(g, k.c.data() + (order - 1) * Np, k.e[order - 1], i, reinterpret_cast<__half*>(halves));
+  for (long long i = 0; i < dense_pairs(g); ++i)
+    dense_pair(g, k.c.data() + (order - 1) * Np, k.e[order - 1], i, reinterpret_cast<__half*>(halves));
   return 0;
 }
 static void dense64_order(const DenseGeom& g, const DenseKernels& k, int order, std::vector<__half>* out) {
   out->resize(dense64_order_halves(g));
-  for (long long i = 0; i < dense64_lanes(g); ++i) dense64_lane(g, k.ci.data() + (order - 1) * g.Np, i, out->data());
+  for (long long i = 0; i < dense64_pairs(g); ++i) dense64_pair(g, k.ci.data() + (order - 1) * g.Np, i, out->data());
 }
 // The sums of digit products that the float64 kernel adds in float32 are exact: the largest possible magnitude of one, for
 // line digits of at most 128, over all outputs, parts and weights of an order; 0 where there is no geometry.

@@ -102,14 +102,14 @@ fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int bat
 }
 
 __global__ void dense_build_kernel(const __grid_constant__ DenseGeom g, const double* __restrict__ c, int e1, int e2, __half* out) {
-  const long long n = dense_groups(g), i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long n = dense_pairs(g), i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * n) return;
   const int o = i >= n;
-  dense_group(g, c + o * g.Np, o ? e2 : e1, i - o * n, out + o * dense_order_halves(g));
+  dense_pair(g, c + o * g.Np, o ? e2 : e1, i - o * n, out + o * dense_order_halves(g));
 }
 
 fc_status launch_dense_build(const PlanData& p, const double* c, void* out, cudaStream_t stream) {
-  const long long n = 2 * dense_groups(p.dense);
+  const long long n = 2 * dense_pairs(p.dense);
   dense_build_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(p.dense, c, p.kern.e[0], p.kern.e[1], static_cast<__half*>(out));
   return cuda_status(cudaGetLastError(), "dense z blocks launch");
 }

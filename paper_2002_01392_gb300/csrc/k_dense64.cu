@@ -223,10 +223,10 @@ __global__ void __launch_bounds__(kD64Threads, 1) dense64_kernel(const __grid_co
 }
 
 __global__ void dense64_build_kernel(const __grid_constant__ DenseGeom g, const long long* __restrict__ c, __half* out) {
-  const long long n = dense64_lanes(g), i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long n = dense64_pairs(g), i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * n) return;
   const int o = i >= n;
-  dense64_lane(g, c + o * g.Np, i - o * n, out + o * dense64_order_halves(g));
+  dense64_pair(g, c + o * g.Np, i - o * n, out + o * dense64_order_halves(g));
 }
 
 }  // namespace
@@ -283,7 +283,7 @@ fc_status launch_deriv_dense64(const DerivDevTables& t, const PlanData& p, int b
 }
 
 fc_status launch_dense64_build(const PlanData& p, const long long* c, void* out, cudaStream_t stream) {
-  const long long n = 2 * dense64_lanes(p.dense64);
+  const long long n = 2 * dense64_pairs(p.dense64);
   dense64_build_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(p.dense64, c, static_cast<__half*>(out));
   return cuda_status(cudaGetLastError(), "dense z blocks launch (float64)");
 }
