@@ -188,7 +188,7 @@ constexpr int kNoiseThreads = 128;
 // output, whole call: 1.09 ms, against 16.0 ms for one float64 sum over +-n
 // per point and passes of their own for the maximum and the scaling; error
 // against 64 bits 2.5e-8 (before: 3.7e-8, two roundings).
-template <class A, bool QUARTER, bool MAX, bool WRITE>
+template <class A, bool QUARTER, bool MAX, bool WRITE, bool SHIFT = false>
 __global__ void __launch_bounds__(kNoiseThreads) noise_rows(int nmax, int Nx, int ni, int Ny, int Nz, int rows,
                                                             const int* __restrict__ start, const int* __restrict__ ml,
                                                             const typename A::W* __restrict__ P,
@@ -223,8 +223,15 @@ __global__ void __launch_bounds__(kNoiseThreads) noise_rows(int nmax, int Nx, in
   }
   __syncthreads();
   float2 f = make_float2(0.f, 0.f);
+  int shift = 0;
   if constexpr (WRITE && !MAX) {
-    const double mx = __longlong_as_double((long long)*word), fd = mx > 0.0 ? amplitude / mx : 1.0;
+    const double mx = __longlong_as_double((long long)*word);
+    double fd = mx > 0.0 ? amplitude / mx : 1.0;
+    if constexpr (SHIFT) {   // the exponent apart
+      int ea = 0, em = 0;
+      fd = mx > 0.0 ? frexp(amplitude, &ea) / frexp(mx, &em) : 1.0;
+      shift = ea - em;
+    }
     f.x = (float)fd;
     f.y = (float)(fd - (double)f.x);
   }
@@ -261,7 +268,7 @@ __global__ void __launch_bounds__(kNoiseThreads) noise_rows(int nmax, int Nx, in
       typename A::T* o = row + c * plane;
       auto put = [&](int x, V v) {
         if constexpr (MAX) m.take(v);
-        if constexpr (WRITE) o[x] = noise_out(v, f);
+        if constexpr (WRITE) o[x] = SHIFT ? (typename A::T)ldexp(noise_out(v, f), shift) : noise_out(v, f);
       };
       if constexpr (QUARTER) {
         // cos n(pi -+ x) = (-1)^n cos nx, sin n(pi - x) = -(-1)^n sin nx
@@ -328,7 +335,12 @@ void noise_launch(const NoiseGrid& g, const NoiseDev& d, typename A::T* out, cud
   if constexpr (std::is_same_v<A, NoiseF32>) {
     noise_rows<A, QUARTER, true, false><<<grid, kNoiseThreads, per * rows, st>>>(
         g.nmax, g.Nx, g.ni, g.Ny, g.Nz, rows, d.start, d.ml, P, Ex, Ey, out, d.word, g.amplitude);
-    noise_rows<A, QUARTER, false, true><<<grid, kNoiseThreads, per * rows, st>>>(
+    // amplitude / max has to stay in float's range as a pair (the sums are near 1); far amplitudes have their exponent apart
+    // (for all of them, ldexp on every value would cost 5 %)
+    const double amp = std::fabs(g.amplitude);
+    auto kern = amp > 0.0 && (amp < 0x1p-60 || amp > 0x1p60) ? noise_rows<A, QUARTER, false, true, true>
+                                                            : noise_rows<A, QUARTER, false, true, false>;
+    kern<<<grid, kNoiseThreads, per * rows, st>>>(
         g.nmax, g.Nx, g.ni, g.Ny, g.Nz, rows, d.start, d.ml, P, Ex, Ey, out, d.word, g.amplitude);
   } else {
     noise_rows<A, QUARTER, true, true><<<grid, kNoiseThreads, per * rows, st>>>(
@@ -485,9 +497,16 @@ extern "C" fc_status fc_noise(const fc_noise_params* p, fc_dtype dtype, int Nx, 
       ab[2 * j] = make_double2(ra * std::cos(2 * pi * draws[2 * j]), ra * std::sin(2 * pi * draws[2 * j]));
       ab[2 * j + 1] = make_double2(rb * std::cos(2 * pi * draws[2 * j + 1]), rb * std::sin(2 * pi * draws[2 * j + 1]));
     }
-  // the largest magnitude is scaled away at the end: keep the sums near 1 by a power of two, whatever the slopes
+  // the largest magnitude is scaled away at the end: keep the vertical profiles (g_m and g_m' / lambda_m are below about 2)
+  // near 1 by a power of two, whatever the slopes and the box
   double big = 0.0;
-  for (const double2& v : ab) big = std::max(big, std::max(std::fabs(v.x), std::fabs(v.y)));
+  for (int h = 0; h < H; ++h)
+    for (int mi = 0; mi < nm; ++mi) {
+      const double2 a = ab[2 * ((size_t)h * nm + mi)], b = ab[2 * ((size_t)h * nm + mi) + 1];
+      const double kx = md.kxy[h].x, ky = md.kxy[h].y, kp = std::sqrt(kx * kx + ky * ky);
+      big = std::max(big, std::hypot(a.x, a.y) * std::max(kp * kp, kp * lam[mi] / p->Lz));
+      big = std::max(big, std::hypot(b.x, b.y) * kp);
+    }
   if (big > 0.0 && std::isfinite(big)) {
     const int e = std::ilogb(big);
     for (double2& v : ab) v = make_double2(std::ldexp(v.x, -e), std::ldexp(v.y, -e));

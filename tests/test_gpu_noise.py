@@ -103,3 +103,15 @@ def test_noise_folded_rows_match_oracle(api, Nx, Ny, Nz, kw):
     assert np.abs(out64 - ref).max() < 1e-13
     # one float32 rounding of values <= 1; the pairs' own error is below 1e-12
     assert np.abs(out32 - ref).max() <= 2.0 ** -24 + 1e-12
+
+
+@pytest.mark.parametrize("size,amplitude", [(1e-18, 1e-25), (1e18, 1e25), (1e-12, 1e30), (1.0, 2e-38), (1.0, 3e38)])
+def test_noise_box_sizes_and_amplitudes(api, size, amplitude):
+    """Boxes and amplitudes whose ratio to the unscaled sums leaves float's range: float32 output is the float64 one,
+    rounded (2^-24 of a value, 2^-150 where it is subnormal, each twice for the shift)."""
+    kw = {"Lx": 2 * np.pi * size, "Ly": 2 * np.pi * size, "Lz": size, "kperp2_min": 4.0 / size ** 2,
+          "kperp2_max": 25.0 / size ** 2, "amplitude": amplitude}
+    out64, _ = _run(api, 14, 12, 9, torch.float64, 5, **kw)
+    out32, _ = _run(api, 14, 12, 9, torch.float32, 5, **kw)
+    assert abs(np.abs(out64).max() / amplitude - 1) < 1e-14
+    assert np.abs(out32 - out64).max() <= 2.0 ** -23 * amplitude + 2.0 ** -149
