@@ -56,9 +56,8 @@ namespace fcns {
 struct DenseArgs {
   DenseGeom g;
   int d, Cc, stages, resident, low_low, orders;   // orders: bit 0 d/dz, bit 1 d2/dz2
-  int Zin;                 // rows of the input: Nz (the rest continued here) or N'
-  long long per;           // lines of one group: adjacent in memory; the z stride
-  long long in_outer, out_outer;   // elements between groups
+  long long per;           // lines of one field: adjacent in memory; the z stride
+  long long outer;         // elements between fields
   long long lines;         // all lines
   long long tiles;
   const float* in;
@@ -297,7 +296,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       const long long L = tile * kDenseLines + line;
       const bool valid = L < a.lines;
       const long long grp = valid ? L / a.per : 0, off = valid ? L % a.per : 0;
-      const float* in = a.in + grp * a.in_outer + off;
+      const float* in = a.in + grp * a.outer + off;
       dz::mbar_wait<64>(bSf, it & 1, abort, 1);
       float s1 = scale[line], s2 = scale[kDenseLines + line];
       bool tiny = __any_sync(0xffffffffu, s2 != 1.f);
@@ -312,7 +311,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
         for (int i = 0; i < NQ; ++i) {   // rows move by one per orbit: the group's ends (and a wrap between them)
           r0[i] = dense_row(g, j0, i);
           const int r1 = dense_row(g, j0 + 7, i);
-          pure = pure && r0[i] < a.Zin && r1 < a.Zin && (r1 - r0[i] == 7 || r0[i] - r1 == 7);
+          pure = pure && r0[i] < g.Nz && r1 < g.Nz && (r1 - r0[i] == 7 || r0[i] - r1 == 7);
         }
         if (pure) {
 #pragma unroll
@@ -329,7 +328,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
             for (int i = 0; i < NQ; ++i) {
               const int r = dense_row(g, j0 + k, i);
               float v = 0.f;
-              if (j0 + k < g.No) v = r < a.Zin ? __ldcg(in + (long long)r * a.per) : cont[(r - g.Nz) * kDenseLines + line];
+              if (j0 + k < g.No) v = r < g.Nz ? __ldcg(in + (long long)r * a.per) : cont[(r - g.Nz) * kDenseLines + line];
               x[i][k] = v;
             }
         }
@@ -401,7 +400,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       constexpr int MG = 3;
       for (int o = 0; o < 2; ++o) {
         if (!(a.orders >> o & 1)) continue;
-        float* out = (o == 0 ? a.out1 : a.out2) + grp * a.out_outer + off;
+        float* out = (o == 0 ? a.out1 : a.out2) + grp * a.outer + off;
         // the factor undoes the line's scale: a.f 2^K.  Where that or a part times it could leave float's range, the
         // accumulators take most of it first (by 1 for the other lines of the warp: a line's bits do not depend on them)
         const int K = a.fe[o] - scaled, K1 = min(max(K, -100), 100);
@@ -507,59 +506,57 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_z_kernel(const __grid_
       for (int u = 0; u < 2; ++u) {
         const long long L = tile * kDenseLines + line0 + 64 * u;
         valid[u] = L < a.lines;
-        in[u] = a.in + (valid[u] ? (L / a.per) * a.in_outer + L % a.per : 0);   // (an absent line reads the first one)
+        in[u] = a.in + (valid[u] ? (L / a.per) * a.outer + L % a.per : 0);   // (an absent line reads the first one)
       }
       // this tile's rows into L2 while the workers are busy with the one before: a prefetch per 128 bytes, eight rows at
       // a time
       const long long Ln = tile * kDenseLines + 32 * (lane & 3);
       if (Ln < a.lines) {
-        const float* nx = a.in + (Ln / a.per) * a.in_outer + Ln % a.per;
-        for (int n = (warp - 16) * 8 + (lane >> 2); n < a.Zin; n += 16) prefetch_l2(nx + (long long)n * a.per);
+        const float* nx = a.in + (Ln / a.per) * a.outer + Ln % a.per;
+        for (int n = (warp - 16) * 8 + (lane >> 2); n < g.Nz; n += 16) prefetch_l2(nx + (long long)n * a.per);
       }
       // a sample of the line for its scale: at most 32 rows
-      const int every = (a.Zin + 31) / 32;
+      const int every = (g.Nz + 31) / 32;
       const long long skip = a.per * every;
       const float *p0 = in[0], *p1 = in[1];
 #pragma unroll 16
-      for (int n = 0; n < a.Zin; n += every, p0 += skip, p1 += skip) {
+      for (int n = 0; n < g.Nz; n += every, p0 += skip, p1 += skip) {
         mx[0] = fmaxf(mx[0], fabsf(__ldcg(p0)));
         mx[1] = fmaxf(mx[1], fabsf(__ldcg(p1)));
       }
       if (it > 0) dz::mbar_wait<64>(bSe, (it - 1) & 1, abort, 3);
-      if (a.Zin < g.Np) {
-        // continuation (Sec. 3): M_r f_last + its mirror on f_first, in float
-        // pairs, both lines in one packed operation; values jj and C - 1 - jj
-        // share their matrix entries
-        constexpr int DM = D > 0 ? D : 10;
-        const int d = D > 0 ? D : a.d;
-        float2 first[DM], last[DM];
+      // continuation (Sec. 3): M_r f_last + its mirror on f_first, in float
+      // pairs, both lines in one packed operation; values jj and C - 1 - jj
+      // share their matrix entries
+      constexpr int DM = D > 0 ? D : 10;
+      const int d = D > 0 ? D : a.d;
+      float2 first[DM], last[DM];
 #pragma unroll
-        for (int i = 0; i < DM; ++i) {
-          const long long of = (long long)i * a.per, ol = (long long)(g.Nz - d + i) * a.per;
-          first[i] = i < d ? make_float2(__ldcg(in[0] + of), __ldcg(in[1] + of)) : make_float2(0.f, 0.f);
-          last[i] = i < d ? make_float2(__ldcg(in[0] + ol), __ldcg(in[1] + ol)) : make_float2(0.f, 0.f);
-        }
-        for (int jj = 0; 2 * jj < a.Cc; ++jj) {
-          float2 h[2] = {}, l[2] = {};   // value jj and its mirror: high and low sums
+      for (int i = 0; i < DM; ++i) {
+        const long long of = (long long)i * a.per, ol = (long long)(g.Nz - d + i) * a.per;
+        first[i] = i < d ? make_float2(__ldcg(in[0] + of), __ldcg(in[1] + of)) : make_float2(0.f, 0.f);
+        last[i] = i < d ? make_float2(__ldcg(in[0] + ol), __ldcg(in[1] + ol)) : make_float2(0.f, 0.f);
+      }
+      for (int jj = 0; 2 * jj < a.Cc; ++jj) {
+        float2 h[2] = {}, l[2] = {};   // value jj and its mirror: high and low sums
 #pragma unroll
-          for (int i = 0; i < DM; ++i)
-            if (i < d) {
-              const float2 m1 = mr[jj * d + i], m2 = mr[(a.Cc - 1 - jj) * d + (d - 1 - i)];
-              const float2 n1 = mr[(a.Cc - 1 - jj) * d + i], n2 = mr[jj * d + (d - 1 - i)];
-              dz::ff2_fma(h[0], l[0], m1, last[i]);
-              dz::ff2_fma(h[1], l[1], n1, last[i]);
-              dz::ff2_fma(h[0], l[0], m2, first[i]);
-              dz::ff2_fma(h[1], l[1], n2, first[i]);
-            }
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const float2 v = dz::add2(h[u], l[u]);
-            const int row = u == 0 ? jj : a.Cc - 1 - jj;
-            mx[0] = fmaxf(mx[0], fabsf(v.x));
-            mx[1] = fmaxf(mx[1], fabsf(v.y));
-            cont[row * kDenseLines + line0] = v.x;
-            cont[row * kDenseLines + line0 + 64] = v.y;
+        for (int i = 0; i < DM; ++i)
+          if (i < d) {
+            const float2 m1 = mr[jj * d + i], m2 = mr[(a.Cc - 1 - jj) * d + (d - 1 - i)];
+            const float2 n1 = mr[(a.Cc - 1 - jj) * d + i], n2 = mr[jj * d + (d - 1 - i)];
+            dz::ff2_fma(h[0], l[0], m1, last[i]);
+            dz::ff2_fma(h[1], l[1], n1, last[i]);
+            dz::ff2_fma(h[0], l[0], m2, first[i]);
+            dz::ff2_fma(h[1], l[1], n2, first[i]);
           }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float2 v = dz::add2(h[u], l[u]);
+          const int row = u == 0 ? jj : a.Cc - 1 - jj;
+          mx[0] = fmaxf(mx[0], fabsf(v.x));
+          mx[1] = fmaxf(mx[1], fabsf(v.y));
+          cont[row * kDenseLines + line0] = v.x;
+          cont[row * kDenseLines + line0 + 64] = v.y;
         }
       }
 #pragma unroll

@@ -75,9 +75,8 @@ fc_status launch_deriv_dense(const DerivDevTables& t, const PlanData& p, int bat
   a.d = p.d;
   a.Cc = p.C;
   a.orders = (df ? 1 : 0) | (d2f ? 2 : 0);
-  a.Zin = p.Nz;
   a.per = lines;
-  a.in_outer = a.out_outer = lines * p.Nz;
+  a.outer = lines * p.Nz;
   a.lines = lines * batch;
   a.in = static_cast<const float*>(f);
   a.out1 = static_cast<float*>(df);
