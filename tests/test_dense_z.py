@@ -369,6 +369,34 @@ def test_dense64_arithmetic_on_the_cpu(Nz, Mr_5_25):
         assert not y[:, 15].any()
 
 
+@pytest.mark.parametrize("d,C,Nz", [(3, 15, 40), (7, 33, 103), (10, 64, 201), (10, 64, 448), (4, 64, 512)])
+def test_dense64_other_continuations_on_the_cpu(d, C, Nz):
+    """test_dense64_arithmetic_on_the_cpu with other d and C, N' even and odd up to the largest.  The reference continues
+    the lines in rational numbers: the weights of d = 10, C = 64 reach 1e10 and cancel."""
+    from fractions import Fraction
+    lib = _lib()
+    from paper_2002_01392_gb300 import api as a
+    f = np.ascontiguousarray(_lines64(Nz, 16, Nz))
+    Mr = np.ascontiguousarray(a.Plan(d, C, Nz).matrix())
+    M, F = [[Fraction(v) for v in row] for row in Mr.tolist()], [[Fraction(v) for v in row] for row in f.tolist()]
+
+    def extended(v):   # to 64 bits
+        hi = float(v)
+        return np.longdouble(hi) + np.longdouble(float(v - Fraction(hi)))
+
+    cont = np.array([[extended(sum(M[j][i] * F[Nz - d + i][n] + M[C - 1 - j][d - 1 - i] * F[i][n] for i in range(d)))
+                      for n in range(16)] for j in range(C)])
+    # the derivative of the line that is continued already: N' points, none added
+    xe = np.vstack([f.astype(np.longdouble), cont])
+    ptr = lambda x: x.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    for order in (1, 2):
+        y = np.full((Nz, 16), np.nan)
+        assert lib.fchc_dense64_tile(Nz, d, C, ptr(Mr), order, ptr(f), ptr(y)) == 0
+        ref = _derivative_ld(xe, np.zeros((0, d)), order, Nz + C - 1.0)[:Nz]
+        err = np.abs(y - ref).max(axis=0)
+        assert (err <= _bound64(f, Mr, order, Nz - 1.0)).all()
+
+
 def test_dense64_digit_sums_are_exact():
     """No sum of digit products of any operator that the float64 kernel takes can leave 2^24, where float32 still holds
     every whole number."""
