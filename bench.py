@@ -53,8 +53,25 @@ def _measured_traffic(key):
     return None
 
 
+def _deriv_tensor_roofline(r, digit_products, Nz=513, C=25):
+    """fc_deriv_z by the dense operators against the tensor cores: per line and order NQ blocks of No x No entries
+    (the parts of a line under its mirror and, for even N', the half shift), each entry times a value as
+    ``digit_products`` products (3 of float16 pairs, 36 of eight-digit numbers), 2 flops each, without padding, over the
+    CUDA-event time; peak = the measured cuBLAS bf16 burst rate."""
+    Np = Nz + C
+    NQ, m = (4, Np // 2) if Np % 2 == 0 else (2, Np)
+    No = (m + (1 if m % 2 else (2 if Nz % 2 else 0))) // 2
+    line = 2 * NQ * No * No * digit_products * 2
+    achieved = line * (r["points"] / Nz) / r["seconds_per_call_mean"] / 1e12
+    p = os.path.join(ROOT, "MEASURED_PEAKS.json")
+    peak, kind = (json.load(open(p)).get("bf16_tflops"), "measured") if os.path.exists(p) else (None, None)
+    peak, kind = (float(peak), kind) if peak else (1900.0, "fallback")
+    return {"bound": "tensor", "achieved": float(achieved), "peak": peak, "unit": "TFLOP/s", "frac": float(achieved / peak),
+            "flops_per_line": float(line), "peak_kind": kind + " cuBLAS bf16 burst"}
+
+
 def _deriv_alu_roofline(r, peak_tflops, peak_kind, L=1080, Nz=513, C=25, d=5):
-    """fc_deriv_z against the arithmetic pipe: algorithmic flops per line pair
+    """fc_deriv_z by transforms (float32 calls of few lines) against the arithmetic pipe: algorithmic flops per line pair
     (two real z-lines as one complex line) = three length-L FFTs at
     5 L log2 L, two spectrum products (6 flops per complex multiply), the
     continuation of both lines (2 C d multiply-adds each) and the output
@@ -1171,7 +1188,7 @@ def main():
         nz = bench_noise(api, torch)
     alu = measure_alu_peaks(api, torch)
     if r64:
-        r64["roofline_alu"] = _deriv_alu_roofline(r64, alu["dfma"]["tflops"], "measured DFMA rate (fc_alu_probe)")
+        r64["roofline_tensor"] = _deriv_tensor_roofline(r64, 36)
     value = replica_value(torch, r32["points"] * args.steps, r32["seconds_total"])
     ms_per_step = _max_over_ranks(torch, r32["seconds_total"]) / args.steps * 1e3
     out = {
@@ -1179,7 +1196,8 @@ def main():
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": dict(DERIV_CONFIG, parallelism="replicas" if world > 1 else "single",
-                       arm="FP32 transforms, continuation in float-float (FP64-level)"),
+                       arm="FP32 lines, dense z operators in float16 pairs on the tensor cores (FP32-level), "
+                           "continuation in float-float (FP64-level)"),
         "p50_ms": r32["p50_ms"], "p99_ms": r32["p99_ms"],
         "fc_deriv_z": {"fp32": {k: v for k, v in r32.items() if k != "e2e"}, "fp64": r64,
                        "fp32_smooth_Np512_3x512x512x487": rs, "cufft_fp64_plain": rc,
@@ -1195,9 +1213,9 @@ def main():
                      "peak": hbm_peak, "unit": "GB/s",
                      "frac": r32["alg_bytes_per_call"] / r32["seconds_per_call_mean"] / 1e9 / hbm_peak,
                      "traffic": _measured_traffic("fc_deriv_z_f32"), "peak_kind": peak_kind,
-                     "kernel": "fc_deriv_z conv L=1080 FP32, paired lines, real-valued kernel spectra, registers j >= 16 known zero, rows j < 13 without bounds checks, whole tiles (phased_kernel<DerivPair<float,30,36,4,16,1,13,1>>)",
+                     "kernel": "fc_deriv_z dense operators f32: 128-line tiles, tcgen05.mma on float16 pairs (dense_z_kernel<4, 5>)",
                      "algorithmic_bytes_per_point": 12, "traffic_source": "profiles/traffic.txt (ncu, small case scaled x6)"},
-        "roofline_alu": _deriv_alu_roofline(r32, alu["ffma"]["tflops"], "measured FFMA rate (fc_alu_probe)"),
+        "roofline_tensor": _deriv_tensor_roofline(r32, 3),
         "alu_peaks_measured": alu,
         "e2e": r32.get("e2e"),
         "gpu_launches": r32["launches"],

@@ -121,10 +121,22 @@ fc_status fc_destroy(fc_plan_t plan);
  * Needs no workspace.  Transform length: N' itself when it is a compiled
  * smooth length (64, 128, 256, 512, 768, 1024, 1536), else the smallest
  * compiled length >= N' + Nz - 1 (up to 1536); FC_ERR_UNSUPPORTED when
- * neither exists.  Large float32 calls, and float64 calls for N' <= 384 or
- * even N' < 576, take the derivative operators as dense blocks on the tensor
- * cores instead of transforms (same accuracy, float64 through exact integer
- * sums); a NaN or Inf then spoils the outputs of its own line only.
+ * neither exists.
+ * Some calls take the derivative operators as dense blocks on the tensor cores
+ * instead of transforms, by their number of lines batch*Nx*Ny:
+ *   float32, from 16384 lines on for padded N' >= 180, from 131072 on for padded
+ *     N' >= 100 whose transform has 288 points or more (256 for odd N') and
+ *     from 98304 on for N' = 512, up to N' = 576 (575 for odd Nz) and while
+ *     the continuation leaves room (any C < 48);
+ *   float64, at any number (but 2433 to 3648 for N' = 512), for N' <= 384 and even
+ *     N' <= 576 (574 for odd Nz).
+ * The bits of a line therefore depend on the size of the call, and not on the
+ * other lines; splitting a call into smaller ones can change them.  Float64 is
+ * exact integer sums, rounded once.  Float32 carries 22 bits of every factor;
+ * its error is that of the transforms or less in the 2-norm (0.5 to 0.95 of it
+ * on rough lines), while the largest single error, which the transforms spread
+ * over the line, can be up to 2.5 times theirs next to steep ends.  A NaN or Inf
+ * spoils the outputs of its own line only (of its pair, in the transforms).
  * FC_ERR_TIMEOUT: a float32 dense kernel of an earlier call of the plan gave up
  * a bounded wait; its outputs are NaN from there on.  Reported once, by the
  * next fc_deriv_z, fc_deriv_z_noalloc or fc_deriv_z_host call of the plan,
@@ -148,7 +160,7 @@ fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, 
  *     fixed 128 KiB static device array that every GPU loading the library
  *     reserves until the process exits, and the operator blocks of
  *     calls that fc_deriv_z runs with the dense operators in another of
- *     2.54 MiB.
+ *     2.53 MiB.
  *   - The first call on each device looks up that array's device address
  *     (cudaGetSymbolAddress) with the device current and keeps it for the
  *     life of the process: resetting the device (cudaDeviceReset) after that
@@ -156,14 +168,15 @@ fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, 
  *   - When the plan or the precision differs from those of the previous call
  *     on the device, the call first copies the plan's tables into the array
  *     on `stream` from the plan's (pageable) host memory; such a copy waits
- *     for the work already queued on `stream` before the call returns.  A
- *     call with the same plan and precision as the previous call on the
- *     device copies nothing and only enqueues the kernel.
+ *     for the work already queued on `stream` before the call returns; a
+ *     kernel then builds the operator blocks of that plan and precision, if it
+ *     has any.  A call with the same plan and precision as the previous call
+ *     on the device copies nothing and only enqueues the kernel.
  *   - Every call shares the array and the tables stay there after the call:
  *     calls whose copies and kernels can overlap on the GPU (on other
  *     streams, from other host threads) race on it and must be serialised by
  *     the caller.
- *   - A plan whose tables would not fit the 128 KiB array returns
+ *   - A plan whose tables would not fit the arrays returns
  *     FC_ERR_UNSUPPORTED (the tables of every compiled transform length fit:
  *     at most 100 KiB, float64 at length 1536); arguments are checked as in
  *     fc_deriv_z.

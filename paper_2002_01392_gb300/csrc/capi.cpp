@@ -112,19 +112,23 @@ bool injected_event(const char* name) {
 // tile of 128 lines passes through one SM in 10 us (N' = 115) to 45 us (538), so
 // a call needs a wave of tiles (152 x 128 lines) or more, and the gain depends
 // on how far the transform length lies above N'.  Measured, dense against
-// transform (us):
-//   padded, N' >= 180   257 x 16k lines 34 / 37, 513 x 16k 51 / 65, 513 x 41k
-//                       131 / 156, 400 x 82k 180 / 333, 513 x 400k 881 / 1578;
-//                       8k lines: 33 / 22 and 46 / 31, so from 16384 lines on
-//   padded, N' >= 100   90 x 132k 88 / 94, 129 x 132k 113 / 131; 129 x 41k 51 /
-//                       42, 65 x 132k 80 / 74: from 131072 lines on
-//   direct, N' >= 400   (the transform has length N') 487 x 82k 206 / 228, 41k
+// transform (us, inputs that rotate over more than the L2):
+//   padded, N' >= 180   Nz = 155 x 16k lines 29 / 34, 257 x 16k 39 / 48, 400 x 16k 52 /
+//                       80, 513 x 16k 58 / 65, 400 x 98k 221 / 395; 8k lines: about
+//                       33 / 22 and 46 / 31, so from 16384 lines on
+//   padded, N' >= 100   from 131072 lines on (129 x 41k 51 / 42), and where the
+//                       transform has 288 points or more (129 x 131k 112 / 132, 150
+//                       101 / 208), or 256 and the line two parts, which short lines
+//                       prefer to four (N' odd: 104 89 / 97, but 115 105 / 99); below
+//                       that the transforms are even or faster (75 x 131k 87 / 81)
+//   direct, N' >= 400   (the transform has length N') 487 x 98k 245 / 272, 41k
 //                       124 / 121: from 98304 lines on
 //   direct, shorter     231 x 132k 167 / 139: transforms
-static long long dense_min_lines(const PlanData& p) {
+static long long dense_min_lines(const PlanData& p, int L) {
   const long long never = 1LL << 62;
   if (p.dense_direct) return p.Np >= 400 ? 98304 : never;
-  return p.Np >= 180 ? 16384 : (p.Np >= 100 ? 131072 : never);
+  if (p.Np >= 180) return 16384;
+  return p.Np >= 100 && (L >= 288 || (L == 256 && p.Np % 2)) ? 131072 : never;
 }
 // Float64 calls take them wherever the plan has them: the transforms sit on the
 // float64 pipe.  Measured, dense against transform (us): 11 x 512 lines 29 / 58,
@@ -134,7 +138,7 @@ static long long dense_min_lines(const PlanData& p) {
 // half empty are they slower (3072 lines: 217 / 199).
 bool deriv_is_dense(const PlanData& p, fc_dtype dtype, long long lines) {
   if (dtype == FC_F64) return p.dense64.NQ && !(p.dense_direct && p.Np >= 400 && lines > 2432 && lines <= 3648);
-  return p.dense.NQ && lines >= dense_min_lines(p);
+  return p.dense.NQ && lines >= p.dense_lines;
 }
 
 }  // namespace fcns
@@ -230,7 +234,8 @@ fc_status fc_setup_ex(int d, int C, int Nz, int M, int n_os, fc_plan_t* out) {
   }
   PlanData& pd = p->data;
   pd.dense_direct = L == pd.Np;
-  const bool f32 = L > 0 && dense_min_lines(pd) < (1LL << 31) && dense_plan(Nz, d, C, &pd.dense);
+  pd.dense_lines = dense_min_lines(pd, L);
+  const bool f32 = L > 0 && pd.dense_lines < (1LL << 31) && dense_plan(Nz, d, C, &pd.dense);
   const bool f64 = L > 0 && dense64_geom(Nz, pd.Np, &pd.dense64);
   if (!f32) pd.dense = DenseGeom();
   if (!f64) pd.dense64 = DenseGeom();

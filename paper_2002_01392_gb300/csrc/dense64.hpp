@@ -9,7 +9,7 @@
 // operators' blocks are whole numbers of 2^-e below 2^63 (rounded once, from
 // binary128; with 2^55, twice the transform's error), in eight digits.  Digits are exact in
 // float16, and a sum of digit products stays a whole number below 2^24 (the
-// table builder checks the bound), so the tensor cores add them up exactly in
+// CPU tests check the bound for every N'), so the tensor cores add them up exactly in
 // float32.  Digit products of one weight share an accumulator: the eight
 // leading weights are kept (36 of 64 products), what is left out is about 2^-56
 // of the largest entry times the largest value.
@@ -24,7 +24,7 @@ constexpr int kD64Lines = 16;    // lines per tile: the rows of one matrix instr
 constexpr int kD64Digits = 8;
 constexpr int kD64Sums = 8;      // weights kept: digits i of the line and j of the operator with i + j < 8
 
-// dense_geom for float64: the blocks fit 2.4 MB (they are read once per tile)
+// dense_geom for float64: both orders' blocks take 2.65 MB at most (they are read once per tile)
 inline bool dense64_geom(int Nz, int Np, DenseGeom* o) {
   DenseGeom g;
   if (!dense_geom(Nz, Np, &g) || (g.NQ == 2 && g.KQ > 192)) return false;

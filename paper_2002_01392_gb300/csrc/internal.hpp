@@ -55,6 +55,7 @@ struct PlanData {
   double ls_residual;
   std::vector<double> Mr;
   DenseGeom dense;                        // dense operators (NQ = 0: none)
+  long long dense_lines = 0;              // float32 calls of this many lines or more take them
   DenseGeom dense64;                      // the same for float64 (dense64.hpp)
   bool dense_direct = false;              // the transform kernel would run at length N' itself
   DenseKernels kern;                      // what the blocks are built from, where either exists

@@ -31,7 +31,7 @@ struct Dense64Args {
 };
 
 // One CTA walks tiles of 16 lines.  Bound: the tensor pipe (36 products of 16 x
-// 8 x 16 per fragment pair), then the operators' fragments out of L2 (2.7 MB per
+// 8 x 16 per fragment pair), then the operators' fragments out of L2 (2.65 MB per
 // tile at N' = 538).  16 lines because the digits of all NQ parts have to be in
 // shared memory together (an output row is a sum over the parts): 147 KB, beside
 // the line itself (69 KB), into which the next tile is copied while the products run.
