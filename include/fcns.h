@@ -133,9 +133,10 @@ fc_status fc_destroy(fc_plan_t plan);
  * The bits of a line therefore depend on the size of the call, and not on the
  * other lines; splitting a call into smaller ones can change them.  Float64 is
  * exact integer sums, rounded once.  Float32 carries 22 bits of every factor;
- * its error is that of the transforms or less in the 2-norm (0.5 to 0.95 of it
- * on rough lines), while the largest single error, which the transforms spread
- * over the line, can be up to 2.5 times theirs next to steep ends.  A NaN or Inf
+ * its error in the 2-norm is 0.3 to 1.0 times that of the transforms on rough
+ * lines (up to 1.3 for N' = 512 on parabolas and lines with a large mean),
+ * while the largest single error, which the transforms spread over the line,
+ * can be up to 2.5 times theirs where the values are large.  A NaN or Inf
  * spoils the outputs of its own line only (of its pair, in the transforms).
  * FC_ERR_TIMEOUT: a float32 dense kernel of an earlier call of the plan gave up
  * a bounded wait; its outputs are NaN from there on.  Reported once, by the

@@ -12,7 +12,7 @@
 // the small ones first (of NQ = 2, whose blocks come in several slabs, apart
 // from the large ones) and, where the contraction is short and the time of a
 // tile is its loads (KQ <= 48), low x low too.  Error of d/dz against the
-// transforms', 2-norm over rough lines: 0.47 to 0.95 for N' from 125 to 575
+// transforms', 2-norm over rough lines: 0.33 to 0.97 for N' from 125 to 575
 // (1.01 and 0.92 at N' = 384); with the small products of NQ = 2 added to the
 // large sums it was up to 1.16.
 //
