@@ -154,7 +154,8 @@ fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int Nx, int Ny, 
  * fixed-size arena and that forbid allocations by plug-ins, and programs
  * running under a device-memory budget that a library must not grow.
  * (fc_deriv_z allocates its tables with cudaMalloc on the first call of a
- * plan on a device.)  The paper has no counterpart; this is a deployment
+ * plan on a device, and a precision's operator blocks on the first call that
+ * takes the dense operators in it.)  The paper has no counterpart; this is a deployment
  * variant of fc_deriv_z, and its results are bitwise those of fc_deriv_z.
  *   - Calls no cudaMalloc, cudaFree or other allocating routine.  The plan's
  *     tables (continuation matrix, kernel spectra, twiddles) live in one

@@ -273,6 +273,7 @@ fc_status fc_destroy(fc_plan_t plan) {
       cudaSetDevice(t.device);
       cudaDeviceSynchronize();
       cudaFree(t.block);
+      cudaFree(t.dense); cudaFree(t.dense64);
       for (auto& slot : t.stage)
         for (void* b : slot) cudaFree(b);
       for (int k = 0; k < 3; ++k) {
@@ -306,7 +307,7 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
     set_error("fc_deriv_z: more devices than the plan supports (64)");
     return FC_ERR_UNSUPPORTED;
   }
-  // every table in one allocation and one copy; the dense operators' blocks behind them, built on the device
+  // every table in one allocation and one copy (the dense operators' blocks follow when a call takes them)
   const PlanData& pd = plan->data;
   const PlanHostTables& h = plan->deriv;
   std::vector<unsigned char> up;
@@ -322,11 +323,10 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
   const size_t oG1 = put(h.H1_64.data(), 16 * L), oG2 = put(h.H2_64.data(), 16 * L), oU = put(h.tw64.data(), 32 * L);
   const size_t oC = pd.dense.NQ ? put(pd.kern.c.data(), 8 * pd.kern.c.size()) : 0;
   const size_t oI = pd.dense64.NQ ? put(pd.kern.ci.data(), 8 * pd.kern.ci.size()) : 0;
-  const size_t oB = (up.size() + 255) & ~(size_t)255, oB64 = oB + dense_bytes(pd), total = oB64 + dense64_bytes(pd);
   DerivDevTables t;
   t.device = dev;
   t.L = h.L;
-  s = cuda_status(cudaMalloc(&t.block, total), "cudaMalloc(tables)");
+  s = cuda_status(cudaMalloc(&t.block, up.size()), "cudaMalloc(tables)");
   if (s) return s;
   unsigned char* at = static_cast<unsigned char*>(t.block);
   t.Mr = reinterpret_cast<double*>(at + oMr);
@@ -334,14 +334,8 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
   t.H1_32 = at + oH1; t.H2_32 = at + oH2; t.tw32 = at + oT;
   t.H1_64 = at + oG1; t.H2_64 = at + oG2; t.tw64 = at + oU;
   s = cuda_status(cudaMemcpy(at, up.data(), up.size(), cudaMemcpyHostToDevice), "cudaMemcpy(tables)");
-  if (!s && pd.dense.NQ) {
-    t.dense = at + oB;
-    s = launch_dense_build(pd, reinterpret_cast<const double*>(at + oC), t.dense, nullptr);
-  }
-  if (!s && pd.dense64.NQ) {
-    t.dense64 = at + oB64;
-    s = launch_dense64_build(pd, reinterpret_cast<const long long*>(at + oI), t.dense64, nullptr);
-  }
+  if (pd.dense.NQ) t.kern = reinterpret_cast<const double*>(at + oC);
+  if (pd.dense64.NQ) t.kern64 = reinterpret_cast<const long long*>(at + oI);
   // in place before any stream reads them, non-blocking ones too
   if (!s) s = cuda_status(cudaStreamSynchronize(nullptr), "cudaStreamSynchronize(tables)");
   if (s) {
@@ -351,6 +345,28 @@ static fc_status deriv_tables_locked(fc_plan* plan, DerivDevTables** out) {
   plan->data.dev.push_back(t);
   *out = &plan->data.dev.back();
   return FC_OK;
+}
+
+// The dense operators' blocks of a precision, at its first call that takes them (an allocation of more than 2 MB is 90 us,
+// and most plans are used in one precision).  On a stream of its own and with the thread's capture mode relaxed, so that
+// the call may be a captured one: the blocks belong to the plan, not to the graph.
+static fc_status dense_blocks_locked(const PlanData& pd, DerivDevTables* t, fc_dtype dtype) {
+  void*& slot = dtype == FC_F64 ? t->dense64 : t->dense;
+  if (slot) return FC_OK;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  fc_status s = cuda_status(cudaThreadExchangeStreamCaptureMode(&mode), "cudaThreadExchangeStreamCaptureMode");
+  if (s) return s;
+  void* b = nullptr;
+  cudaStream_t st = nullptr;
+  s = cuda_status(cudaMalloc(&b, dtype == FC_F64 ? dense64_bytes(pd) : dense_bytes(pd)), "cudaMalloc(blocks)");
+  if (!s) s = cuda_status(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking), "cudaStreamCreate");
+  if (!s) s = dtype == FC_F64 ? launch_dense64_build(pd, t->kern64, b, st) : launch_dense_build(pd, t->kern, b, st);
+  if (!s) s = cuda_status(cudaStreamSynchronize(st), "cudaStreamSynchronize(blocks)");
+  if (st) cudaStreamDestroy(st);
+  if (s) cudaFree(b);
+  else slot = b;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return s;
 }
 
 }  // namespace fcns
@@ -383,13 +399,14 @@ extern "C" fc_status fc_deriv_z(fc_plan_t plan, fc_dtype dtype, int batch, int N
   fc_status s = check_deriv_args(plan->data, plan->deriv, dtype, batch, Nx, Ny, Lz, f, df, d2f, "fc_deriv_z");
   if (!s) s = dense_gave_up(plan->data, "fc_deriv_z");
   if (s) return s;
+  const bool dense = deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch);
   DerivDevTables* t = nullptr;
   {
     std::lock_guard<std::mutex> lk(plan->data.mtx);
     s = deriv_tables_locked(plan, &t);
+    if (!s && dense) s = dense_blocks_locked(plan->data, t, dtype);
   }
   if (s) return s;
-  const bool dense = deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch);
   return launch_deriv_any(dense, *t, plan->data, dtype, batch, (long long)Nx * Ny, Lz, f, df, d2f, (cudaStream_t)stream);
 }
 
@@ -435,10 +452,13 @@ extern "C" fc_status fc_deriv_z_host_ex(fc_plan_t plan, fc_dtype dtype, int batc
   fc_status s = check_deriv_args(plan->data, plan->deriv, dtype, batch, Nx, Ny, Lz, f, df, d2f, "fc_deriv_z_host");
   if (!s) s = dense_gave_up(plan->data, "fc_deriv_z_host");
   if (s) return s;
+  // the whole call picks the kernel, so that the slabs give what one call on device arrays gives
+  const bool dense = deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch);
   DerivDevTables* t = nullptr;
   {
     std::lock_guard<std::mutex> lk(plan->data.mtx);
     s = deriv_tables_locked(plan, &t);
+    if (!s && dense) s = dense_blocks_locked(plan->data, t, dtype);
   }
   if (s) return s;
   std::lock_guard<std::mutex> hl(plan->data.host_mtx);
@@ -457,8 +477,6 @@ extern "C" fc_status fc_deriv_z_host_ex(fc_plan_t plan, fc_dtype dtype, int batc
   const char* fh = static_cast<const char*>(f);
   char* oh[2] = {static_cast<char*>(df), static_cast<char*>(d2f)};
   const size_t hp = (size_t)Ny * Nx * es;     // host pitch between z rows
-  // the whole call picks the kernel, so that the slabs give what one call on device arrays gives
-  const bool dense = deriv_is_dense(plan->data, dtype, (long long)Nx * Ny * batch);
   long long i = 0;
   for (size_t si = 0; si < slabs.size() && !s; ++si, ++i) {
     {  // slab si in staging slot i % 3

@@ -30,7 +30,7 @@ int pick_engine_length(int need);
 struct DerivDevTables {
   int device = -1;
   int L = 0;
-  void* block = nullptr;  // one allocation holds all of the following
+  void* block = nullptr;  // one allocation holds all of the following but the blocks
   double* Mr = nullptr;
   float2* Mr2 = nullptr;  // (hi, lo) float split of Mr
   void* tw32 = nullptr;  // float2[L]
@@ -39,6 +39,8 @@ struct DerivDevTables {
   void* H1_64 = nullptr;
   void* H2_32 = nullptr;
   void* H2_64 = nullptr;
+  const double* kern = nullptr;      // what the blocks are built from (PlanData::kern)
+  const long long* kern64 = nullptr;
   void* dense = nullptr;          // blocks of the dense operators (float16 pairs), both orders; null: not used
   void* dense64 = nullptr;        // the same for float64 (digit fragments)
   // staging of fc_deriv_z_host: three rotating slots of (input, d1, d2) slab

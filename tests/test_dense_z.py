@@ -447,8 +447,8 @@ def test_given_up_waits_are_reported(api):
 
 @pytest.mark.gpu
 def test_a_plans_first_call_prepares_all_others(api):
-    """After one small call on a plan, large ones, of the other precision too, can be captured (nothing is allocated or
-    copied), and fc_deriv_z_noalloc, whose tables are one precision's, only launches after a small call of the same."""
+    """After one small call on a plan, large ones, of the other precision too, can be captured (what they add to the plan
+    is no part of the graph), and fc_deriv_z_noalloc, whose tables are one precision's, only launches after a small call of the same."""
     import torch
     Nz, Ny, Nx = 513, 8, 2560
     plan = api.Plan(5, 25, Nz)
